@@ -65,7 +65,8 @@ typedef struct {
     int32_t samples_per_thread; /* samples each thread of the batched launch keeps in flight
                                    per step of its loop: 1 (default) or 2; the other
                                    samplers take one at a time                             */
-    int32_t adjacency;          /* adjacency test: 1 = hash set of the edges (default),
+    int32_t adjacency;          /* adjacency test: 1 = hub bitmap rows and an edge filter
+                                   whose hits are confirmed in the sorted rows (default),
                                    2 = search of the sorted smaller list + hub bitmaps,
                                    3 = a hash table per adjacency list                      */
     int32_t draw_order;         /* the *_ordered samplers: 0 (default) sort each chunk of
@@ -100,10 +101,7 @@ typedef struct ps_graph ps_graph; /* opaque; host metadata + pointers into the w
 
 /* Bytes of device workspace a graph with n vertices and nnz stored arcs
  * (nnz = 2m) needs under tuning t (NULL = defaults).  0 if the sizes are
- * outside the supported range (n < 2^31, nnz < 2^31).  Test hook: a
- * positive PS_TEST_ESET_LIST_CAP in the environment caps the hash set's
- * per-region key lists (forcing its overflow and slow paths; results are
- * unchanged); it must not change between this call and ps_load_csr. */
+ * outside the supported range (n < 2^31, nnz < 2^31). */
 size_t ps_graph_workspace_bytes(int64_t n, int64_t nnz, const ps_tuning *t);
 
 /* Section 2 input and Section 4 order.  Reads the CSR graph (d_off: int64
@@ -114,16 +112,12 @@ size_t ps_graph_workspace_bytes(int64_t n, int64_t nnz, const ps_tuning *t);
  * ascending, and builds the edge table (u < v, u ascending then v ascending)
  * with the positions of each edge in both endpoint lists, the inclusive
  * uint64 prefix sums of the weights tau_e and lambda_e (in the same pass as
- * the table), and (default adjacency) the hash set of the edges.
+ * the table), and (default adjacency) the edge filter.
  *
  * d_off / d_col belong to the caller and are only read during the call.
  * d_workspace (ws_bytes >= ps_graph_workspace_bytes(n, nnz, t), 256-byte
  * aligned) must stay allocated and untouched until ps_graph_free(*out).
- * Synchronises `stream` (to read the validation flags).  The hash set build
- * (default adjacency), which only sampling reads, runs on a library-owned
- * stream and may still be running when the call returns: ps_tau_prefix
- * orders it before everything it queues on its own stream, and
- * ps_graph_free waits for it.  On error *out is NULL and the status is
+ * Synchronises `stream` (to read the validation flags).  On error *out is NULL and the status is
  * PS_ERR_TIMEOUT (a bounded device wait of one of the scans expired, which
  * makes every other finding of the call unreliable, so it comes first) /
  * PS_ERR_ARG / PS_ERR_NOT_SIMPLE / PS_ERR_ASYMMETRIC (highest-priority
@@ -231,10 +225,8 @@ int ps_count_adaptive(const ps_graph *g, uint64_t seed, double target, double de
                       uint64_t *d_hist4, ps_stream_t stream, uint64_t *k_used, uint64_t hist6[6],
                       uint64_t hist4[4], double est[6], double lo[6], double hi[6]);
 
-/* Releases the host metadata of g (not the workspace, which the caller owns),
- * first waiting for library work that may still write into the workspace
- * (the hash set build of ps_load_csr); work the caller queued on its own
- * streams is the caller's to wait for. */
+/* Releases the host metadata of g (not the workspace, which the caller owns);
+ * work the caller queued on its own streams is the caller's to wait for. */
 void ps_graph_free(ps_graph *g);
 
 /* Short description of a status code (static string). */
@@ -357,7 +349,7 @@ int ps_csr_from_edges(int64_t n, int64_t n_edges, const int32_t *d_src, const in
  *   (d_a + d_b + d_c - 6), N_4 = 4-cycles, N_5 = sum over edges of
  *   C(t_e, 2) (t_e = triangles through e), N_6 = 4-cliques.
  * g must have been through ps_tau_prefix (it uses the canonical graph, W,
- * N_1 and g's adjacency test).  Work: one hash-set test per upper-part entry
+ * N_1 and g's adjacency test).  Work: one adjacency test per upper-part entry
  * of the lower endpoint of every edge, plus one per pair of common upper
  * neighbours (4-cliques), plus the wedges below each vertex (4-cycles).
  *

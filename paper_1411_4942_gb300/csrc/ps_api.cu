@@ -4,7 +4,6 @@
 #include <atomic>
 #include <climits>
 #include <cmath>
-#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -91,9 +90,9 @@ Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz) {
     r.adj_mode = kAdjHash;
     r.draw_order = 0;
     if (t && (t->adjacency == kAdjSearch || t->adjacency == kAdjVtab)) r.adj_mode = t->adjacency;
-    // hub rows beside the hash set cover the top 2^19 labels only: a lookup
+    // hub rows beside the edge filter cover the top 2^19 labels only: a lookup
     // whose larger label is a hub and whose smaller is among them reads one
-    // bit, the rest probe the set.  Narrower rows let more hubs share the
+    // bit, the rest ask the filter.  Narrower rows let more hubs share the
     // same bytes.  The search variant needs the rows for every hub pair and
     // keeps them full width.
     r.hub_span_log2 = r.adj_mode == kAdjHash ? kHubSpanLog2 : 0;
@@ -102,7 +101,7 @@ Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz) {
         else if (t->hub_span_log2 > 0) r.hub_span_log2 = t->hub_span_log2 < 5 ? 5 : (t->hub_span_log2 > 30 ? 30 : t->hub_span_log2);
     }
     // hub bitmap rows: up to 1024 full-width rows within 256 MB for the search
-    // variant; up to kHubRowsMax within 512 MB beside the hash set, and within
+    // variant; up to kHubRowsMax within 512 MB beside the filter, and within
     // 48 bytes per edge there (under a third of the graph's workspace)
     const int64_t span = (r.hub_span_log2 > 0 && n > (int64_t{1} << r.hub_span_log2)) ? (int64_t{1} << r.hub_span_log2) : n;
     const int64_t row_bytes = ((span + 31) / 32) * 4;
@@ -128,6 +127,20 @@ Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz) {
     return r;
 }
 
+// Words of the edge filter for m edges: 16 bits per edge up to 16 MB, then
+// 8 bits per edge, at most 64 MB as long as that leaves 4 bits per edge.
+// The filter should stay in L2 beside the rows and records the sampling
+// reads: the 3-path kernel took 942 us on R-MAT 20 (15.7M edges) with the
+// hash set before it, 787 / 748 / 721 us with 64 / 32 / 16 MB; on the
+// 3M-vertex graph (115M edges) 32 / 64 / 128 MB took 11.5 / 10.9 / 11.9 ms.
+// On graphs of up to 10M edges 8, 16 and 32 bits per edge are within 2%.
+static int64_t filter_words(int64_t m) {
+    int64_t w = m / 2;
+    if (w > (int64_t{1} << 22)) w = m / 4 > (int64_t{1} << 22) ? m / 4 : (int64_t{1} << 22);
+    if (w > (int64_t{1} << 24)) w = m / 8 > (int64_t{1} << 24) ? m / 8 : (int64_t{1} << 24);
+    return w < 32 ? 32 : w;
+}
+
 bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     if (n < 0 || nnz < 0 || n >= INT32_MAX || nnz >= INT32_MAX) return false;
     Layout l{};
@@ -150,26 +163,7 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
         l.hub_bit_base = base > 0 ? (base / 32) * 32 : 0;
     }
     l.hub_words = (n - l.hub_bit_base + 31) / 32;
-    // edge hash set: a power-of-two number of buckets, load <= 1/2
-    l.eset_buckets = 0;
-    if (t.adj_mode == kAdjHash) {
-        int64_t slots = 64;
-        while (slots < 2 * l.m_cap) slots <<= 1;
-        l.eset_buckets = slots / kBucketSlots;
-    }
-    l.eset_regions = l.eset_buckets >= kRegionBuckets ? l.eset_buckets / kRegionBuckets : 0;
-    // a region's keys are Poisson around m / regions (the hash is uniform), so
-    // lists of 9/8 of that plus 64 overflow with negligible probability; the
-    // overflow list catches the rest
-    l.eset_cap = l.eset_regions ? (l.m_cap + l.eset_regions - 1) / l.eset_regions : 0;
-    l.eset_cap += l.eset_cap / 8 + 64;
-    l.eset_ov_cap = l.eset_regions ? 65536 + l.m_cap / 256 : 0;
-    // test hook: PS_TEST_ESET_LIST_CAP=c caps every region list at c keys, so
-    // the overflow list and, past it, the slow path take the other keys
-    if (const char *cap_env = std::getenv("PS_TEST_ESET_LIST_CAP")) {
-        const long long c = std::atoll(cap_env);
-        if (l.eset_regions && c > 0 && c < l.eset_cap) l.eset_cap = c;
-    }
+    l.filt_words = t.adj_mode == kAdjHash ? filter_words(l.m_cap) : 0;
     l.vtab_slots = t.adj_mode == kAdjVtab ? 2 * nnz : 0;
     l.radix_tiles = (n + kRadixTile - 1) / kRadixTile;
     if (l.radix_tiles < 1) l.radix_tiles = 1;
@@ -202,7 +196,7 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.gtau = take(static_cast<size_t>(gtau_words) * sizeof(int32_t));
     l.glam = take(static_cast<size_t>(l.gcap + 2) * sizeof(int32_t));
     l.hub = take(static_cast<size_t>(l.hub_cap) * l.hub_words * sizeof(uint32_t));
-    l.eset = take(static_cast<size_t>(l.eset_buckets) * kBucketSlots * sizeof(uint64_t));
+    l.filt = take(static_cast<size_t>(l.filt_words) * sizeof(uint32_t));
     l.vtab = take(static_cast<size_t>(l.vtab_slots) * sizeof(int32_t));
     l.keys0 = take(n1 * sizeof(uint32_t));
     l.keys1 = take(n1 * sizeof(uint32_t));
@@ -210,11 +204,6 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.vals1 = take(n1 * sizeof(uint32_t));
     l.rcounts = take(static_cast<size_t>(256) * l.radix_tiles * sizeof(uint32_t));
     l.ecounts = take(static_cast<size_t>(256) * edge_sort_tiles(l.m_cap) * sizeof(uint32_t));
-    // the region build's key lists (one per region, then the overflow list)
-    // and their lengths
-    l.ekeys = take(l.eset_regions ? static_cast<size_t>(l.eset_regions * l.eset_cap + l.eset_ov_cap) * sizeof(uint64_t)
-                                  : 0);
-    l.eregion = take(l.eset_regions ? static_cast<size_t>(l.eset_regions + 2) * sizeof(uint32_t) : 0);
     l.scan_flag = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(uint32_t));
     l.scan_agg = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(U64x2));
     l.scan_inc = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(U64x2));
@@ -340,7 +329,7 @@ int ps_load_csr(int64_t n, int64_t nnz, const int64_t *d_off, const int32_t *d_c
     g->gtau = reinterpret_cast<int32_t *>(ws + L.gtau);
     g->glam = reinterpret_cast<int32_t *>(ws + L.glam);
     g->hub = reinterpret_cast<uint32_t *>(ws + L.hub);
-    g->eset = L.eset_buckets ? reinterpret_cast<uint64_t *>(ws + L.eset) : nullptr;
+    g->filt = L.filt_words ? reinterpret_cast<uint32_t *>(ws + L.filt) : nullptr;
     g->vtab = L.vtab_slots ? reinterpret_cast<int32_t *>(ws + L.vtab) : nullptr;
     const int rc = load_graph(g, d_off, d_col, reinterpret_cast<cudaStream_t>(stream));
     if (rc != PS_OK) {

@@ -33,10 +33,10 @@ static int table_adjacency(const void *d_table) {
 
 template <int ADJ>
 __device__ __forceinline__ int batch_sample(const GraphDev &g, int sampler, uint64_t seed, uint64_t id) {
-    return sampler == 0 ? sample_3path<ADJ, false>(g, seed, id) : sample_centred<ADJ, false>(g, seed, id);
+    return sampler == 0 ? sample_3path<ADJ>(g, seed, id) : sample_centred<ADJ>(g, seed, id);
 }
 
-// Two samples of one thread with the hash-set adjacency, their steps
+// Two samples of one thread with the filter adjacency, their steps
 // interleaved: both draws (edge, record, neighbours) as straight-line code,
 // then both samples' tests, so the two dependent chains overlap.  The same
 // counts as two calls of batch_sample.
@@ -47,24 +47,30 @@ __device__ __forceinline__ void batch_sample2_hash(const GraphDev &g, int sample
     if (sampler == 0) {
         path3_draw(g, seed, id0, e0, a0, b0);
         path3_draw(g, seed, id1, e1, a1, b1);
-        bool x0, y0, z0, x1, y1, z1;
-        pair_test3<false>(g, a0, e0.v, e0.u, b0, a0, b0, x0, y0, z0);
-        pair_test3<false>(g, a1, e1.v, e1.u, b1, a1, b1, x1, y1, z1);
-        c0 = a0 == b0 ? 0 : class3(x0, y0, z0);
-        c1 = a1 == b1 ? 0 : class3(x1, y1, z1);
+        const int32_t x[6] = {a0, e0.u, a0, a1, e1.u, a1}, y[6] = {e0.v, b0, b0, e1.v, b1, b1};
+        bool r[6];
+        pair_tests<6>(g, x, y, r);
+        c0 = a0 == b0 ? 0 : class3(r[0], r[1], r[2]);
+        c1 = a1 == b1 ? 0 : class3(r[3], r[4], r[5]);
     } else {
         centred_draw(g, seed, id0, e0, a0, b0);
         centred_draw(g, seed, id1, e1, a1, b1);
-        bool k0, k1;
-        eset_contains2(g.eset, g.eset_mask, a0, b0, a1, b1, k0, k1);
-        // the chords only for centred paths (the pair test also answers u' == v')
-        k0 = k0 && a0 != b0;
-        k1 = k1 && a1 != b1;
-        bool p0 = false, q0 = false, p1 = false, q1 = false;
-        if (k0) pair_test2<false>(g, e0.v, a0, e0.u, b0, p0, q0);
-        if (k1) pair_test2<false>(g, e1.v, a1, e1.u, b1, p1, q1);
-        c0 = k0 ? 1 + (int)p0 + (int)q0 : 0;
-        c1 = k1 ? 1 + (int)p1 + (int)q1 : 0;
+        // the chords only for centred paths (u' == v' is not one)
+        const int32_t x[2] = {a0, a1}, y[2] = {b0, b1};
+        bool k[2];
+        pair_tests<2>(g, x, y, k);
+        c0 = c1 = 0;
+        bool r[2];
+        if (k[0] && a0 != b0) {
+            const int32_t p[2] = {a0, e0.u}, q[2] = {e0.v, b0};
+            pair_tests<2>(g, p, q, r);
+            c0 = 1 + (int)r[0] + (int)r[1];
+        }
+        if (k[1] && a1 != b1) {
+            const int32_t p[2] = {a1, e1.u}, q[2] = {e1.v, b1};
+            pair_tests<2>(g, p, q, r);
+            c1 = 1 + (int)r[0] + (int)r[1];
+        }
     }
 }
 
@@ -72,7 +78,7 @@ __device__ __forceinline__ void batch_sample2_hash(const GraphDev &g, int sample
 // counter[0] hands out items; counter[1] counts items skipped because their
 // graph does not use the variant this kernel was compiled for.  Registers
 // are capped for 1024 resident threads per SM with one sample per thread in
-// flight (SPT = 1), 512 with two (SPT = 2, hash-set graphs; other variants
+// flight (SPT = 1), 512 with two (SPT = 2, graphs with an edge filter; other variants
 // take their two samples one after the other).
 template <int BLOCK, int ADJ, int SPT>
 __global__ void __launch_bounds__(BLOCK, (SPT == 1 ? 1024 : 512) / BLOCK)

@@ -15,7 +15,7 @@ typedef unsigned long long u64;
 // One edge (u < v) of the relabelled graph, 32 bytes = one DRAM sector:
 // everything a sample needs after choosing the edge.  iu / jv are the
 // positions of v in N(u) and of u in N(v); ou / ov the row offsets.
-struct __align__(16) EdgeRec {
+struct __align__(32) EdgeRec {
     int32_t u, v, du, dv, iu, jv, ou, ov;
 };
 
@@ -30,15 +30,15 @@ struct GraphDev {
     const int32_t *gtau;     // [Bt + 1] guide: first edge of each r >> tau_shift bucket
     const int32_t *glam;     // [Bl + 1]
     const uint32_t *hub;     // [hubs][hub_words] adjacency bitmaps of the top labels
-    const uint64_t *eset;    // hash set of the edges (4-slot buckets), or null
-    uint64_t eset_mask;      // buckets - 1
+    uint64_t filt_off;       // the edge filter starts this many words after `hub`
+    uint32_t filt_words;     // words of the edge filter
     const int32_t *vtab;     // per-vertex hash tables: slots [2 off(x), 2 off(x+1)), or null
     uint64_t W, Lambda;
     int64_t n, m;
     int32_t hub_start;       // labels >= hub_start have a bitmap row
     int32_t hub_words;
     int32_t tau_shift, lam_shift;
-    int32_t adj_mode;        // kAdjHash or kAdjSearch
+    int32_t adj_mode;        // kAdjHash, kAdjSearch or kAdjVtab
     int32_t hub_bit_base;    // hub rows hold the bits of labels >= hub_bit_base (a multiple of 32)
 };
 
@@ -57,7 +57,6 @@ enum {
     ST_TIER = 10,      // 5 words: row boundaries of the sort tiers
     ST_LONG = 15,      // first row longer than kLongRow (its arcs are walked by a block)
     ST_COUNTER = 16,   // 16 words: tile counters of scans (as uint32 pairs)
-    ST_ESET_SPILL = 32, // non-zero: the hash set's key lists overflowed (slow path taken)
     ST_WORDS = 64
 };
 
@@ -94,12 +93,13 @@ __device__ __forceinline__ uint32_t wait_flag(const uint32_t *flag, uint32_t lim
 
 // Read-only gathers of data written by earlier kernels.  PS_LOAD_MODE picks
 // the cache path: 0 = the non-coherent path through L1 (__ldg); 1 = L2 only
-// (ld.global.cg); 2 = non-coherent without L1 allocation.  In modes 1 and 2
-// a 32-byte edge record is one 256-bit load.
+// (ld.global.cg); 2 = non-coherent without L1 allocation.
 #ifndef PS_LOAD_MODE
 #define PS_LOAD_MODE 0
 #endif
-#if PS_LOAD_MODE == 1
+#if PS_LOAD_MODE == 0
+#define PS_LD "ld.global.nc"
+#elif PS_LOAD_MODE == 1
 #define PS_LD "ld.global.cg"
 #elif PS_LOAD_MODE == 2
 #define PS_LD "ld.global.nc.L1::no_allocate"
@@ -132,24 +132,29 @@ __device__ __forceinline__ uint64_t ldg_u64(const uint64_t *p) {
     return v;
 #endif
 }
+// A gather that nothing nearby reads again: it takes no line of L1.
+__device__ __forceinline__ int32_t ldg_i32_once(const int32_t *p) {
+#if PS_LOAD_MODE == 1
+    return ldg_i32(p);
+#else
+    int32_t v;
+    asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+#endif
+}
 // Gathers of the skewed "hot" structures (guide entries, prefix probes).
-// (Evict-last L2 hints on these, on the hub rows' adjacency lists, and
-// evict-first on the hash buckets were measured: no gain.)
+// (Evict-last L2 hints on these and on the hub rows' adjacency lists were
+// measured: no gain.)
 __device__ __forceinline__ int32_t ldg_i32_hot(const int32_t *p) { return ldg_i32(p); }
 __device__ __forceinline__ uint64_t ldg_u64_hot(const uint64_t *p) { return ldg_u64(p); }
 
 __device__ __forceinline__ EdgeRec ldg_rec(const EdgeRec *p) {
     EdgeRec e;
-#if PS_LOAD_MODE == 0
-    const int4 *q = reinterpret_cast<const int4 *>(p);
-    int4 a = __ldg(q), b = __ldg(q + 1);
-    e.u = a.x; e.v = a.y; e.du = a.z; e.dv = a.w;
-    e.iu = b.x; e.jv = b.y; e.ou = b.z; e.ov = b.w;
-#else
+    // one 256-bit load (records are 32-byte aligned): two 128-bit loads cost a
+    // second pass through L1's tags
     asm(PS_LD ".v8.s32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
         : "=r"(e.u), "=r"(e.v), "=r"(e.du), "=r"(e.dv), "=r"(e.iu), "=r"(e.jv), "=r"(e.ou), "=r"(e.ov)
         : "l"(p));
-#endif
     return e;
 }
 
@@ -297,210 +302,100 @@ __device__ __forceinline__ bool adjacent_known(const GraphDev &g, int32_t a, int
     return in_sorted(g.col, oa, da, b);
 }
 
-// ----------------------------------------------------------- edge hash set
+// ------------------------------------------------------------- edge filter
 
-// The hash-table adjacency that the O(1) test of Theorem 3.5 assumes: the
-// edges {a, b}, a < b, keyed (a << 32) | b, in buckets of four 8-byte slots
-// (32 bytes, one DRAM sector) with linear probing from bucket to bucket.
-// (8-slot, 64-byte buckets overflow less -- 1.04 instead of 1.18 buckets per
-// absent-key lookup at load 1/2 -- but measured slower: 3-path sampling
-// 1.75 -> 1.88 ms on R-MAT 20 and 20 -> 29 ms on the 3M-vertex graph.)
-// Slots only ever go from empty (all ones) to full, so a lookup that meets a
-// bucket with an empty slot before finding its key can stop: had the key
-// been inserted, it would sit in that bucket or an earlier one.
-constexpr uint64_t kEmptySlot = ~0ull;
-constexpr int kBucketSlots = 4;
-constexpr int kBucketShift = 2;  // log2(kBucketSlots)
+// The O(1) adjacency test of Theorem 3.5, in one 4-byte read for nearly every
+// pair.  Hub rows (bitmaps of the top-degree labels) answer a pair whose
+// larger label is a hub and whose smaller label lies in the rows' span: the
+// edges are drawn in proportion to tau, so most pairs name a hub.  The other
+// pairs are almost never edges (99.8% of those asked on R-MAT 20 and on the
+// 3M-vertex graph are not), so they go to a filter: every edge that no hub
+// row holds sets kFilterBits bits of one 32-bit word, and a pair with one of its bits unset
+// is not an edge.  A pair with all bits set (an edge, or a false positive)
+// is looked up in the sorted row of its smaller label, so every answer is
+// exact.  The filter replaces a hash set of the edges (8-byte keys in
+// 32-byte buckets, 18 bytes written per edge at load, a 32-byte sector and
+// eight registers per test, a second probe in about every tenth test).
+constexpr int kFilterBits = 3;
 
-__device__ __forceinline__ uint64_t edge_key(int32_t a, int32_t b) {
-    return (static_cast<uint64_t>(static_cast<uint32_t>(a)) << 32) | static_cast<uint32_t>(b);
+__device__ __forceinline__ uint64_t edge_hash(int32_t a, int32_t c) {
+    uint64_t h = (static_cast<uint64_t>(static_cast<uint32_t>(a)) << 32) | static_cast<uint32_t>(c);
+    h *= 0x9E3779B97F4A7C15ull;
+    h ^= h >> 32;
+    return h * 0xD6E8FEB86659FD93ull;
 }
 
-// Mixes the key; its low bits pick the home bucket and its top kBucketShift
-// bits the slot an insertion tries first (any slot order is valid for the
-// lookups, which read the whole bucket).
-__device__ __forceinline__ uint64_t key_hash(uint64_t key) {
-    uint64_t h = key * 0x9E3779B97F4A7C15ull;
-    h ^= h >> 31;
-    h *= 0xD6E8FEB86659FD93ull;
-    h ^= h >> 29;
-    return h;
+// Word and bits of the pair a < c: the word from the hash's high half, the
+// bit numbers from the upper bits of its low half.
+__device__ __forceinline__ uint32_t filter_word(uint64_t h, uint32_t words) {
+    return __umulhi(static_cast<uint32_t>(h >> 32), words);
 }
-
-__device__ __forceinline__ uint64_t key_bucket(uint64_t key, uint64_t mask) { return key_hash(key) & mask; }
-
-struct Bucket {
-    ulonglong2 q[kBucketSlots / 2];
-};
-
-__device__ __forceinline__ Bucket load_bucket(const uint64_t *set, uint64_t b) {
-    const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(set + (b << kBucketShift));
-    Bucket k;
+__device__ __forceinline__ uint32_t filter_mask(uint64_t h) {
+    const uint32_t s = static_cast<uint32_t>(h) >> (32 - 5 * kFilterBits);
+    uint32_t m = 0;
 #pragma unroll
-    for (int i = 0; i < kBucketSlots / 2; i++) k.q[i] = __ldg(p + i);
-    return k;
+    for (int i = 0; i < kFilterBits; i++) m |= 1u << ((s >> (5 * i)) & 31);
+    return m;
 }
 
-// 1: key present, 0: absent, -1: bucket full without the key (probe on)
-__device__ __forceinline__ int bucket_verdict(const Bucket &k, uint64_t key) {
-    bool hit = false, empty = false;
-#pragma unroll
-    for (int i = 0; i < kBucketSlots / 2; i++) {
-        hit |= (k.q[i].x == key) | (k.q[i].y == key);
-        empty |= (k.q[i].x == kEmptySlot) | (k.q[i].y == kEmptySlot);
-    }
-    return hit ? 1 : (empty ? 0 : -1);
-}
-
-static __device__ __noinline__ bool probe_on(const uint64_t *set, uint64_t mask, uint64_t key,
-                                             uint64_t b) {
-    for (uint64_t i = 0; i < mask; i++) {
-        b = (b + 1) & mask;
-        const int v = bucket_verdict(load_bucket(set, b), key);
-        if (v >= 0) return v == 1;
-    }
-    return false;
-}
-
-__device__ __forceinline__ bool eset_contains(const uint64_t *set, uint64_t mask, int32_t x, int32_t y) {
-    if (x == y) return false;
-    const uint64_t key = edge_key(min(x, y), max(x, y));
-    const uint64_t b = key_bucket(key, mask);
-    const int v = bucket_verdict(load_bucket(set, b), key);
-    return v >= 0 ? v == 1 : probe_on(set, mask, key, b);
-}
-
-// Two independent lookups (x != y for both) with their first buckets loaded together.
-__device__ __forceinline__ void eset_contains2(const uint64_t *set, uint64_t mask, int32_t x0,
-                                               int32_t y0, int32_t x1, int32_t y1, bool &r0, bool &r1) {
-    const uint64_t k0 = edge_key(min(x0, y0), max(x0, y0));
-    const uint64_t k1 = edge_key(min(x1, y1), max(x1, y1));
-    const uint64_t b0 = key_bucket(k0, mask), b1 = key_bucket(k1, mask);
-    const Bucket q0 = load_bucket(set, b0), q1 = load_bucket(set, b1);
-    const int v0 = bucket_verdict(q0, k0), v1 = bucket_verdict(q1, k1);
-    r0 = v0 >= 0 ? v0 == 1 : probe_on(set, mask, k0, b0);
-    r1 = v1 >= 0 ? v1 == 1 : probe_on(set, mask, k1, b1);
-}
-
-// Three independent lookups with their first buckets loaded together.
-__device__ __forceinline__ void eset_contains3(const uint64_t *set, uint64_t mask, int32_t x0,
-                                               int32_t y0, int32_t x1, int32_t y1, int32_t x2,
-                                               int32_t y2, bool &r0, bool &r1, bool &r2) {
-    const uint64_t k0 = edge_key(min(x0, y0), max(x0, y0));
-    const uint64_t k1 = edge_key(min(x1, y1), max(x1, y1));
-    const uint64_t k2 = edge_key(min(x2, y2), max(x2, y2));
-    const uint64_t b0 = key_bucket(k0, mask), b1 = key_bucket(k1, mask), b2 = key_bucket(k2, mask);
-    const Bucket q0 = load_bucket(set, b0), q1 = load_bucket(set, b1), q2 = load_bucket(set, b2);
-    const int v0 = bucket_verdict(q0, k0), v1 = bucket_verdict(q1, k1), v2 = bucket_verdict(q2, k2);
-    r0 = (x0 != y0) && (v0 >= 0 ? v0 == 1 : probe_on(set, mask, k0, b0));
-    r1 = (x1 != y1) && (v1 >= 0 ? v1 == 1 : probe_on(set, mask, k1, b1));
-    r2 = (x2 != y2) && (v2 >= 0 ? v2 == 1 : probe_on(set, mask, k2, b2));
-}
-
-// Hash set plus hub rows: a pair whose larger label is one of the top-degree
-// labels (>= hub_start, rows of the hub bitmap) is answered from that
-// hub's bitmap row, the rest from the hash set.  The sampled edges are
-// drawn in proportion to tau, so a lookup (u', v) mostly names a hub v, and
-// the hub rows' much-read parts stay in L2.  (The rows' loads once asked L2
-// to keep them -- evict-last; with 1024 rows of 375 KB on the 3M-vertex
-// graph that hint made 3-path sampling 2-5% slower on both benchmark graphs,
-// and it was dropped.)  With no hub rows (hub_start == n) this is the plain
-// hash-set test.
-__device__ __forceinline__ uint32_t ld_hub_word(const uint32_t *p) { return __ldg(p); }
-
-// Address of the hub-row word holding bit a of hub c's row (a >= hub_bit_base).
-__device__ __forceinline__ const uint32_t *hub_word_of(const GraphDev &g, int32_t a, int32_t c) {
-    return g.hub + static_cast<int64_t>(c - g.hub_start) * g.hub_words + ((a - g.hub_bit_base) >> 5);
-}
-
-// Does the pair a < c have a hub-row bit?  (The rows hold the labels from
-// hub_bit_base up: the tests naming a hub mostly name it with another
-// high-degree, high-label vertex, and the rest go to the hash set, which
-// holds every edge.)
+// Does the pair a < c have a hub-row bit?
 __device__ __forceinline__ bool in_hub_rows(const GraphDev &g, int32_t a, int32_t c) {
     return c >= g.hub_start && a >= g.hub_bit_base;
 }
 
-// One pair's first load: its hub-row word (in the first slot of the
-// returned bucket) when it has a hub-row bit, else its home bucket.
-__device__ __forceinline__ Bucket load_pair(const GraphDev &g, int32_t a, int32_t c, uint64_t b) {
-    Bucket q;
-    if (in_hub_rows(g, a, c)) {
-        q.q[0].x = ld_hub_word(hub_word_of(g, a, c));
-    } else {
-        q = load_bucket(g.eset, b);
+// Is c in the sorted row of a?
+static __device__ __noinline__ bool row_contains(const int64_t *off, const int32_t *col, int32_t a, int32_t c) {
+    const int64_t o = ldg_i64(off + a);
+    return in_sorted(col, o, ldg_i64(off + a + 1) - o, c);
+}
+
+// N independent tests (x != y for each), every pair's word -- of its hub row
+// or of the filter, chosen without a branch -- in flight together; the few
+// filter hits are then confirmed one by one at a single call site (three
+// separate second probes made nearly every warp take all three).
+template <int N>
+__device__ __forceinline__ void pair_tests(const GraphDev &g, const int32_t (&x)[N], const int32_t (&y)[N],
+                                           bool (&r)[N]) {
+    uint32_t word[N], mask[N];
+    uint32_t pend = 0;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        const int32_t a = min(x[i], y[i]), c = max(x[i], y[i]);
+        const bool hub = in_hub_rows(g, a, c);
+        const uint64_t h = edge_hash(a, c);
+        const uint64_t hw = static_cast<uint64_t>(static_cast<uint32_t>(c - g.hub_start)) * static_cast<uint32_t>(g.hub_words) +
+                            static_cast<uint32_t>((a - g.hub_bit_base) >> 5);
+        const uint64_t fw = g.filt_off + filter_word(h, g.filt_words);
+        mask[i] = hub ? 1u << (a & 31) : filter_mask(h);
+        word[i] = __ldg(g.hub + (hub ? hw : fw));
+        pend |= hub ? 0u : 1u << i;
     }
-    return q;
-}
-
-__device__ __forceinline__ bool resolve_pair(const GraphDev &g, int32_t a, int32_t c, uint64_t key,
-                                             uint64_t b, const Bucket &q) {
-    if (in_hub_rows(g, a, c)) return ((q.q[0].x >> (a & 31)) & 1u) != 0u;
-    const int v = bucket_verdict(q, key);
-    return v >= 0 ? v == 1 : probe_on(g.eset, g.eset_mask, key, b);
-}
-
-// Three independent tests (x != y for each pair) with all first loads in
-// flight together; a pair whose larger label is a hub reads the hub's row.
-// ALL = false sends only the first pair to a hub row (it names an endpoint
-// of the drawn edge, most often a hub) and keeps the other two on the hash
-// set: fewer registers, for kernels that cannot spare them (the batched
-// kernel runs at 64).
-template <bool ALL>
-__device__ __forceinline__ void pair_test3(const GraphDev &g, int32_t x0, int32_t y0, int32_t x1,
-                                           int32_t y1, int32_t x2, int32_t y2, bool &r0, bool &r1,
-                                           bool &r2) {
-    const int32_t a0 = min(x0, y0), c0 = max(x0, y0);
-    if (!ALL) {
-        if (!in_hub_rows(g, a0, c0)) {
-            eset_contains3(g.eset, g.eset_mask, x0, y0, x1, y1, x2, y2, r0, r1, r2);
-            return;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        r[i] = (word[i] & mask[i]) == mask[i];
+        pend &= r[i] ? ~0u : ~(1u << i);
+    }
+    while (pend) {
+        const int k = __ffs(pend) - 1;
+        pend &= pend - 1;
+        int32_t p = x[0], q = y[0];
+#pragma unroll
+        for (int i = 1; i < N; i++) {
+            p = k == i ? x[i] : p;
+            q = k == i ? y[i] : q;
         }
-        const uint32_t w = ld_hub_word(hub_word_of(g, a0, c0));
-        eset_contains2(g.eset, g.eset_mask, x1, y1, x2, y2, r1, r2);
-        r0 = ((w >> (a0 & 31)) & 1u) != 0u;
-        return;
+        const bool in = row_contains(g.off, g.col, min(p, q), max(p, q));
+#pragma unroll
+        for (int i = 0; i < N; i++) r[i] = r[i] && (k != i || in);
     }
-    const int32_t a1 = min(x1, y1), c1 = max(x1, y1);
-    const int32_t a2 = min(x2, y2), c2 = max(x2, y2);
-    const uint64_t k0 = edge_key(a0, c0), k1 = edge_key(a1, c1), k2 = edge_key(a2, c2);
-    const uint64_t b0 = key_bucket(k0, g.eset_mask), b1 = key_bucket(k1, g.eset_mask),
-                   b2 = key_bucket(k2, g.eset_mask);
-    const Bucket q0 = load_pair(g, a0, c0, b0), q1 = load_pair(g, a1, c1, b1), q2 = load_pair(g, a2, c2, b2);
-    r0 = resolve_pair(g, a0, c0, k0, b0, q0);
-    r1 = resolve_pair(g, a1, c1, k1, b1, q1);
-    r2 = resolve_pair(g, a2, c2, k2, b2, q2);
 }
 
 __device__ __forceinline__ bool pair_test(const GraphDev &g, int32_t x, int32_t y) {
-    const int32_t a = min(x, y), c = max(x, y);
-    if (in_hub_rows(g, a, c))
-        return x != y && ((ld_hub_word(hub_word_of(g, a, c)) >> (a & 31)) & 1u);
-    return eset_contains(g.eset, g.eset_mask, x, y);
-}
-
-// Two independent tests (x != y for each pair), both loads in flight; ALL as
-// for pair_test3.
-template <bool ALL>
-__device__ __forceinline__ void pair_test2(const GraphDev &g, int32_t x0, int32_t y0, int32_t x1,
-                                           int32_t y1, bool &r0, bool &r1) {
-    const int32_t a0 = min(x0, y0), c0 = max(x0, y0);
-    if (!ALL) {
-        if (!in_hub_rows(g, a0, c0)) {
-            eset_contains2(g.eset, g.eset_mask, x0, y0, x1, y1, r0, r1);
-            return;
-        }
-        const uint32_t w = ld_hub_word(hub_word_of(g, a0, c0));
-        r1 = eset_contains(g.eset, g.eset_mask, x1, y1);
-        r0 = ((w >> (a0 & 31)) & 1u) != 0u;
-        return;
-    }
-    const int32_t a1 = min(x1, y1), c1 = max(x1, y1);
-    const uint64_t k0 = edge_key(a0, c0), k1 = edge_key(a1, c1);
-    const uint64_t b0 = key_bucket(k0, g.eset_mask), b1 = key_bucket(k1, g.eset_mask);
-    const Bucket q0 = load_pair(g, a0, c0, b0), q1 = load_pair(g, a1, c1, b1);
-    r0 = resolve_pair(g, a0, c0, k0, b0, q0);
-    r1 = resolve_pair(g, a1, c1, k1, b1, q1);
+    if (x == y) return false;
+    const int32_t xs[1] = {x}, ys[1] = {y};
+    bool r[1];
+    pair_tests<1>(g, xs, ys, r);
+    return r[0];
 }
 
 // ------------------------------------------------ per-vertex hash tables

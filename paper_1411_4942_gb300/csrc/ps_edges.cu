@@ -303,15 +303,21 @@ k_esort_scatter(int64_t count, const uint32_t *__restrict__ kin, const uint32_t 
 // thread builds Q edges at j0, j0 + step, ..., their loads issued together
 // stage by stage (the chain sorted entry -> row of u -> v -> row of v is
 // otherwise a string of dependent round trips per edge), and returns their
-// weights (zero past m or for a bad edge).  With the region build of the
-// hash set (lists.keys set), every edge's key also goes to the end of its
-// home region's list (one atomic per edge).
+// weights (zero past m or for a bad edge).  With an edge filter, every edge
+// that no hub row holds also sets its bits there (one atomic without a
+// result per edge).
+struct EdgeFilter {
+    uint32_t *words;  // null: no filter
+    uint32_t count;
+    int32_t hub_bit_base;
+};
+
 template <int Q>
 __device__ __forceinline__ void edge_group(int64_t j0, int step, int64_t m, int64_t n,
                                            const uint32_t *__restrict__ skey, const uint32_t *__restrict__ sval,
                                            const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                                            const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase,
-                                           EdgeRec *rec, u64 *status, const EsetLists &lists, U64x2 (&w)[Q],
+                                           EdgeRec *rec, const EdgeFilter &F, int32_t hub_start, U64x2 (&w)[Q],
                                            bool &asym) {
     // every offset, label and degree is below 2^31 (nnz < 2^31), so the
     // stages work in 32 bits
@@ -357,17 +363,9 @@ __device__ __forceinline__ void edge_group(int64_t j0, int step, int64_t m, int6
         e[0] = make_int4(u[q], v[q], du[q], dv[q]);
         e[1] = make_int4(iu[q], jv, ou[q], ov[q]);
         w[q] = edge_weights(du[q], dv[q], iu[q], jv);
-        if (lists.keys) {
-            const uint64_t key = edge_key(u[q], v[q]);
-            const uint64_t reg = (key_hash(key) & lists.mask) >> lists.shift;
-            const uint32_t pos = atomicAdd(lists.cur + reg, 1u);
-            if (pos < lists.cap) {
-                lists.keys[reg * lists.cap + pos] = key;
-            } else {
-                const uint32_t o = atomicAdd(lists.ov_count, 1u);
-                if (o < lists.ov_cap) lists.ov_keys[o] = key;
-                else status[ST_ESET_SPILL] = 1;
-            }
+        if (F.words && !(v[q] >= hub_start && u[q] >= F.hub_bit_base)) {
+            const uint64_t h = edge_hash(u[q], v[q]);
+            atomicOr(F.words + filter_word(h, F.count), filter_mask(h));
         }
     }
 }
@@ -390,16 +388,16 @@ __global__ void __launch_bounds__(kScanBlock, 4)
 k_edge_records_scan(int64_t m, int64_t n, const uint32_t *__restrict__ skey, const uint32_t *__restrict__ sval,
                     const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                     const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase, EdgeRec *rec,
-                    u64 *status, EsetLists lists, ScanState<U64x2> st, uint64_t *ptau, uint64_t *plam) {
+                    u64 *status, EdgeFilter F, ScanState<U64x2> st, uint64_t *ptau, uint64_t *plam) {
     __shared__ U64x2 s_w[kRecScanItems * kScanBlock];
     const int64_t tile = scan_ticket(st);
     const int64_t wbase = scan_wbase<kScanBlock, kRecScanItems>(tile);
     bool asym = false;
+    const int32_t hub_start = static_cast<int32_t>(n - static_cast<int64_t>(status[ST_HUBS]));
 #pragma unroll
     for (int g0 = 0; g0 < kRecScanItems; g0 += kRecItems) {
         U64x2 w[kRecItems];
-        edge_group<kRecItems>(wbase + 32 * g0, 32, m, n, skey, sval, coff, ccol, lowcnt, ubase, rec, status, lists,
-                              w, asym);
+        edge_group<kRecItems>(wbase + 32 * g0, 32, m, n, skey, sval, coff, ccol, lowcnt, ubase, rec, F, hub_start, w, asym);
 #pragma unroll
         for (int q = 0; q < kRecItems; q++) s_w[(g0 + q) * kScanBlock + threadIdx.x] = w[q];
     }
@@ -411,7 +409,7 @@ k_edge_records_scan(int64_t m, int64_t n, const uint32_t *__restrict__ skey, con
                                                 StorePrefix{ptau, plam, status, m});
 }
 
-int build_edge_table(ps_graph *g, cudaStream_t s, const EsetLists *lists) {
+int build_edge_table(ps_graph *g, cudaStream_t s) {
     const Layout &L = g->L;
     const int64_t n = L.n, nnz = L.nnz, m = L.m_cap;
     if (nnz <= 0 || m <= 0) return PS_OK;
@@ -466,10 +464,10 @@ int build_edge_table(ps_graph *g, cudaStream_t s, const EsetLists *lists) {
     // ka/va: the sorted list, in the G_tau region
     int rc = reset_scan(g, 3, m, s);
     if (rc) return rc;
+    const EdgeFilter F{g->filt, static_cast<uint32_t>(L.filt_words), static_cast<int32_t>(L.hub_bit_base)};
     const int64_t stiles = (m + kScanBlock * kRecScanItems - 1) / (kScanBlock * kRecScanItems);
-    EsetLists none{};
     k_edge_records_scan<<<(unsigned)stiles, kScanBlock, 0, s>>>(
-        m, n, ka, va, g->off, g->col, g->lowcnt, g->ubase, g->rec, g->status, lists ? *lists : none,
+        m, n, ka, va, g->off, g->col, g->lowcnt, g->ubase, g->rec, g->status, F,
         scan_state<U64x2>(g, 3), g->ptau, g->plam);
     PS_LAUNCH_CHECK();
     return PS_OK;

@@ -38,7 +38,7 @@ constexpr int kCliqueCap = 1024;  // common upper neighbours kept per warp in sh
 
 template <int ADJ>
 __device__ __forceinline__ bool has_edge(const GraphDev &g, int32_t x, int32_t y) {
-    if (ADJ == kAdjHash) return eset_contains(g.eset, g.eset_mask, x, y);
+    if (ADJ == kAdjHash) return pair_test(g, x, y);
     if (ADJ == kAdjVtab) {
         if (x == y) return false;
         const int32_t h = max(x, y);

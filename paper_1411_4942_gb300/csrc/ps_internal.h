@@ -16,17 +16,14 @@ namespace ps {
 constexpr int kTierA = 32;      // one warp, one key per lane
 constexpr int kTierB = 1024;    // one warp, up to 32 keys per lane in registers
 constexpr int kTierC = 4096;    // one block, registers + 16 KB shared; above: block radix sort
-// The edge hash set is built region by region in shared memory (64 KB of
-// buckets each) once the table holds at least one whole region.
-constexpr int64_t kRegionBuckets = 2048;
-// Rows longer than this have their arcs walked by a whole block (lower-arc
-// listing, hash set build); shorter rows by a warp per 32 rows.
+// Rows longer than this have their lower arcs listed a warp or a block per
+// row; shorter rows by a warp per 32 rows.
 constexpr int kLongRow = 128;
 // Hub rows are only worth a bitmap above this degree (default of the tuning
 // field hub_min_degree).
 constexpr int kHubMinDegree = 64;
-constexpr int kHubSpanLog2 = 19;   // default hub-row span beside the hash set
-constexpr int kHubRowsMax = 8192;  // default hub-row cap beside the hash set
+constexpr int kHubSpanLog2 = 19;   // default hub-row span beside the edge filter
+constexpr int kHubRowsMax = 8192;  // default hub-row cap beside the edge filter
 constexpr int64_t kCoarseGuideEdges = int64_t{1} << 25;  // default guide of m/4 buckets from here
 // Items per tile of every scan.
 constexpr int kScanBlock = 256;
@@ -55,12 +52,10 @@ int launch_vertex_totals(ps_graph *g, cudaStream_t s);
 
 struct Layout {
     int64_t n, nnz, m_cap, gcap, hub_cap, hub_words, hub_bit_base, radix_tiles, scan_tiles;
-    int64_t eset_buckets;  // 0 without the edge hash set
-    int64_t eset_regions;  // regions of the region build (0: the direct build)
-    int64_t eset_cap, eset_ov_cap;  // region build: keys per region list, overflow list
+    int64_t filt_words;    // 32-bit words of the edge filter; 0 without it
     int64_t vtab_slots;    // 0 without the per-vertex tables
-    size_t status, off, col, rank, lowcnt, ubase, dnew, rec, ptau, plam, gtau, glam, hub, eset, vtab;
-    size_t keys0, keys1, vals0, vals1, rcounts, ecounts, ekeys, eregion, scan_flag, scan_agg, scan_inc;
+    size_t status, off, col, rank, lowcnt, ubase, dnew, rec, ptau, plam, gtau, glam, hub, filt, vtab;
+    size_t keys0, keys1, vals0, vals1, rcounts, ecounts, scan_flag, scan_agg, scan_inc;
     size_t total;
 };
 bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L);
@@ -86,7 +81,7 @@ struct ps_graph {
     uint64_t *ptau, *plam;
     int32_t *gtau, *glam;
     uint32_t *hub;
-    uint64_t *eset;
+    uint32_t *filt;
     int32_t *vtab;
     bool prefixed;
     // read back at the end of ps_load_csr: W, Lambda, N_1 (lo, hi), the hub
@@ -95,14 +90,9 @@ struct ps_graph {
     uint64_t load_flags = 0;
     ps_stats stats;
     ps::GraphDev dev;
-    // ev[0..2]: fork / join events of this graph's calls; ev[3]: end of the
-    // edge hash set build, which runs on past ps_load_csr (eset_pending)
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    mutable bool eset_pending = false;
+    // fork / join events of this graph's calls
+    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     ~ps_graph() {
-        // the hash set build writes into the caller's workspace: let it end
-        // (returns at once when it has, or was never started)
-        if (ev[3]) cudaEventSynchronize(ev[3]);
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
     }
@@ -122,15 +112,6 @@ int flags_to_status(uint64_t flags);
 // call (created on first use, kept for the process; calls join them with
 // their own events, so concurrent calls stay ordered correctly).
 int get_side_streams(int device, cudaStream_t out[2]);
-
-// Makes `s` wait for a hash set build still running from ps_load_csr; every
-// call that reads the set (or the status words it writes) comes after this.
-inline int wait_eset(const ps_graph *g, cudaStream_t s) {
-    if (!g->eset_pending) return PS_OK;
-    if (cudaStreamWaitEvent(s, g->ev[3], 0) != cudaSuccess) return PS_ERR_CUDA;
-    g->eset_pending = false;
-    return PS_OK;
-}
 
 // Every kernel launch is followed by this: counts the launch (reported by
 // ps_kernel_launches) and checks the launch error.
@@ -171,25 +152,11 @@ inline int run_scan(ps_graph *g, int slot, int64_t count, T identity, Op op, Loa
     return PS_OK;
 }
 
-// The hash set's per-region key lists (region build): the edge-table
-// kernel appends every edge's key to the list of its home bucket's region
-// (cursors zeroed before); keys beyond a list's capacity go to an overflow
-// list, and past that the slow path is flagged in status[ST_ESET_SPILL].
-struct EsetLists {
-    uint32_t *cur;       // [regions] list lengths
-    uint32_t *ov_count;  // overflow list length
-    uint64_t *keys;      // [regions][cap]
-    uint64_t *ov_keys;   // [ov_cap]
-    int64_t cap, ov_cap;
-    uint64_t mask;       // buckets - 1
-    int shift;           // region of bucket b = b >> shift
-};
-
 // The edge table (ps_edges.cu): after the rows are relabelled and sorted and
-// ubase is known, writes every edge record (and, given `lists`, every edge's
-// hash-set key into its region's list), and raises F_ASYM for an asymmetric
+// ubase is known, writes every edge record and prefix, sets every edge's bits
+// in the edge filter (cleared before), and raises F_ASYM for an asymmetric
 // input.
-int build_edge_table(ps_graph *g, cudaStream_t s, const EsetLists *lists);
+int build_edge_table(ps_graph *g, cudaStream_t s);
 // Tiles of the edge table's radix sort for m edges (its digit counts take
 // 256 words per tile).
 int64_t edge_sort_tiles(int64_t m);

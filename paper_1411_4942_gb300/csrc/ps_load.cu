@@ -769,216 +769,6 @@ struct StoreUbase {
     }
 };
 
-// Slots of a bucket are tried from the key's own first slot on, which spreads
-// the first attempts over the four slots (fewer failed compare-and-swaps than
-// always starting at slot 0).
-__device__ __forceinline__ bool eset_insert(uint64_t *set, uint64_t mask, uint64_t key) {
-    const uint64_t h = key_hash(key);
-    const int first = static_cast<int>(h >> (64 - kBucketShift));
-    uint64_t b = h & mask;
-    for (uint64_t probe = 0; probe <= mask; probe++) {
-        unsigned long long *slot = reinterpret_cast<unsigned long long *>(set + (b << kBucketShift));
-        for (int q = 0; q < kBucketSlots; q++) {
-            const unsigned long long old =
-                atomicCAS(slot + ((first + q) & (kBucketSlots - 1)), kEmptySlot, key);
-            if (old == kEmptySlot || old == key) return true;
-        }
-        b = (b + 1) & mask;
-    }
-    return false;
-}
-
-// Inserts every edge {r, x}, r < x, into the hash set with compare-and-swap:
-// the upper arcs of the sorted rows (row r's entries after its lowcnt[r]
-// lower ones) are exactly the edges, so the set needs neither the edge table
-// nor its order and is built as soon as the rows are sorted, on a side
-// stream beside the edge table.  The set's contents are deterministic, its
-// slot layout is not.  kInsertBatch keys per lane: their first
-// compare-and-swaps are issued together (most succeed at once), and only
-// the keys whose first slot was taken go on to the full insertion.
-constexpr int kInsertBatch = 4;
-// resident blocks per SM of the direct hash set build (4, 8 and 16 measured
-// the same)
-constexpr int kEsetBlocksPerSm = 8;
-
-__device__ __forceinline__ bool eset_insert_batch(uint64_t *set, uint64_t mask, const uint64_t (&key)[kInsertBatch],
-                                                  const bool (&ok)[kInsertBatch]) {
-    unsigned long long old[kInsertBatch];
-#pragma unroll
-    for (int u = 0; u < kInsertBatch; u++) {
-        old[u] = kEmptySlot;
-        if (ok[u]) {
-            const uint64_t h = key_hash(key[u]);
-            const int first = static_cast<int>(h >> (64 - kBucketShift));
-            unsigned long long *slot = reinterpret_cast<unsigned long long *>(set + ((h & mask) << kBucketShift));
-            old[u] = atomicCAS(slot + first, kEmptySlot, key[u]);
-        }
-    }
-    bool good = true;
-#pragma unroll
-    for (int u = 0; u < kInsertBatch; u++)
-        if (ok[u] && old[u] != kEmptySlot && old[u] != key[u]) good &= eset_insert(set, mask, key[u]);
-    return good;
-}
-
-// The upper arcs in row-major order are the edges in edge order: edge
-// t = ubase[r] + q is the q-th upper arc of row r, at position
-// lowcnt[r] + q of N(r).  Each warp takes kEsetChunk consecutive edges (rows
-// are in degree order, so 32 consecutive rows can hold 32 sqrt(2m) edges:
-// the work is split by edges, not rows): it finds the row of its first edge
-// by a binary search of ubase, then walks windows of 32 rows, each lane
-// finding its edges' rows within the window by a shuffle search of their
-// ubase values, and hands kInsertBatch keys per lane at a time to `f`.
-constexpr int64_t kEsetChunk = 1024;
-
-template <typename F>
-__device__ __forceinline__ void for_each_edge_key(int64_t n, int64_t m, const int64_t *__restrict__ coff,
-                                                  const int32_t *__restrict__ ccol, const int32_t *__restrict__ lowcnt,
-                                                  const int64_t *__restrict__ ubase, F &f) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
-    for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; c * kEsetChunk < m; c += nwarps) {
-        const int64_t t_lo = c * kEsetChunk, t_hi = (t_lo + kEsetChunk < m) ? t_lo + kEsetChunk : m;
-        // the row holding edge t_lo: the last r with ubase[r] <= t_lo
-        int64_t lo = 0, hi = n - 1;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) >> 1;
-            if (ldg_i64(ubase + mid) <= t_lo) lo = mid;
-            else hi = mid - 1;
-        }
-        // every window advances r0, so the walk ends by the last row even when
-        // an asymmetric input has fewer edges than the chunks cover
-        for (int64_t r0 = lo, t = t_lo; t < t_hi && r0 < n; r0 += 32) {
-            const int64_t r = r0 + lane;
-            int64_t ub = m, first = 0;  // lanes past the last row never match
-            if (r < n) {
-                ub = ldg_i64(ubase + r);
-                first = ldg_i64(coff + r) + ldg_i32(lowcnt + r);  // the row's first upper arc
-            }
-            const int64_t w_end = ldg_i64(ubase + (r0 + 32 < n ? r0 + 32 : n));
-            const int64_t seg_end = w_end < t_hi ? w_end : t_hi;
-            for (int64_t t0 = t; t0 < seg_end; t0 += 32 * kInsertBatch) {
-                uint64_t key[kInsertBatch];
-                bool ok[kInsertBatch];
-#pragma unroll
-                for (int u = 0; u < kInsertBatch; u++) {
-                    const int64_t tt = t0 + 32 * u + lane;
-                    int at = 0;
-#pragma unroll
-                    for (int step = 16; step > 0; step >>= 1) {
-                        const int64_t x = __shfl_sync(0xffffffffu, ub, at + step);
-                        if (x <= tt) at += step;
-                    }
-                    const int64_t i = __shfl_sync(0xffffffffu, first, at) + (tt - __shfl_sync(0xffffffffu, ub, at));
-                    ok[u] = tt < seg_end;
-                    key[u] = ok[u] ? edge_key(static_cast<int32_t>(r0 + at), ldg_i32(ccol + i)) : 0ull;
-                }
-                f(key, ok);
-            }
-            t = seg_end;
-        }
-    }
-}
-
-// Direct build (tables smaller than one region, or no scratch): every key
-// inserted with compare-and-swap into the table in global memory.
-struct InsertDirect {
-    uint64_t *set;
-    uint64_t mask;
-    bool failed;
-    __device__ void operator()(const uint64_t (&key)[kInsertBatch], const bool (&ok)[kInsertBatch]) {
-        failed |= !eset_insert_batch(set, mask, key, ok);
-    }
-};
-
-__global__ void __launch_bounds__(256)
-k_eset_upper(int64_t n, int64_t m, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
-             const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase, uint64_t *set, uint64_t mask,
-             u64 *status) {
-    InsertDirect f{set, mask, false};
-    for_each_edge_key(n, m, coff, ccol, lowcnt, ubase, f);
-    if (f.failed) raise_flag(status, F_OVERFLOW);
-}
-
-// Region build.  The table is cut into regions of kRegionBuckets buckets
-// (64 KB), each small enough for one block's shared memory.  The edge-table
-// kernel appends every key to the list of its home bucket's region
-// (EsetLists); then one block per region inserts that region's keys with
-// shared-memory compare-and-swap, probing linearly within the region, and
-// writes the whole region out (empty slots included, so the table needs no
-// clearing).  A key whose probe runs past its region's end goes to the
-// overflow list, and that list is inserted at the end by ordinary global
-// compare-and-swap, probing on into the following regions -- already
-// written, so every bucket between a key's home and its place is full, as a
-// lookup assumes.  The random read-modify-writes of the direct build become
-// sequential writes of the table plus the key lists' traffic.
-constexpr int kRegionThreads = 512;
-
-// One block per region (grid-stride): the region's keys into shared memory,
-// then the region written out.
-__global__ void __launch_bounds__(kRegionThreads)
-k_eset_regions(int64_t regions, int64_t region_buckets, EsetLists lists, uint64_t *set, u64 *status) {
-    extern __shared__ unsigned long long s_tab[];
-    const int64_t slots = region_buckets << kBucketShift;
-    for (int64_t reg = blockIdx.x; reg < regions; reg += gridDim.x) {
-        for (int64_t q = threadIdx.x; q < slots; q += kRegionThreads) s_tab[q] = kEmptySlot;
-        __syncthreads();
-        const int64_t b0 = reg * region_buckets;
-        const int64_t len = lists.cur[reg] < lists.cap ? lists.cur[reg] : lists.cap;
-        uint64_t *list = lists.keys + reg * lists.cap;
-        for (int64_t e = threadIdx.x; e < len; e += kRegionThreads) {
-            const unsigned long long key = list[e];
-            const uint64_t h = key_hash(key);
-            const int first = static_cast<int>(h >> (64 - kBucketShift));
-            bool placed = false;
-            for (int64_t b = static_cast<int64_t>(h & lists.mask) - b0; b < region_buckets && !placed; b++) {
-                for (int q = 0; q < kBucketSlots; q++) {
-                    const unsigned long long old =
-                        atomicCAS(s_tab + (b << kBucketShift) + ((first + q) & (kBucketSlots - 1)), kEmptySlot, key);
-                    if (old == kEmptySlot || old == key) {
-                        placed = true;
-                        break;
-                    }
-                }
-            }
-            if (!placed) {  // rare: every bucket from its home to the region's end is full
-                const uint32_t o = atomicAdd(lists.ov_count, 1u);
-                if (o < lists.ov_cap) lists.ov_keys[o] = key;
-                else status[ST_ESET_SPILL] = 1;
-            }
-        }
-        __syncthreads();
-        unsigned long long *dst = reinterpret_cast<unsigned long long *>(set) + (b0 << kBucketShift);
-        for (int64_t q = threadIdx.x; q < slots; q += kRegionThreads) dst[q] = s_tab[q];
-        __syncthreads();
-    }
-}
-
-// The overflow list (keys beyond their region list's capacity, and keys
-// whose probe ran past their region): global compare-and-swap.
-__global__ void __launch_bounds__(256)
-k_eset_leftovers(EsetLists lists, uint64_t *set, u64 *status) {
-    const int64_t ov = *lists.ov_count < lists.ov_cap ? *lists.ov_count : lists.ov_cap;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    bool failed = false;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ov; e += stride)
-        failed |= !eset_insert(set, lists.mask, lists.ov_keys[e]);
-    if (failed) raise_flag(status, F_OVERFLOW);
-}
-
-// The slow path, only when the overflow list itself overflowed (the keys it
-// could not hold are in no list): every edge inserted again by direct
-// compare-and-swap (a key already present stops at once).
-__global__ void __launch_bounds__(256)
-k_eset_spill_fallback(int64_t n, int64_t m, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
-                      const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase, uint64_t *set,
-                      uint64_t mask, u64 *status) {
-    if (ld_acquire(reinterpret_cast<const uint32_t *>(status + ST_ESET_SPILL)) == 0u) return;
-    InsertDirect f{set, mask, false};
-    for_each_edge_key(n, m, coff, ccol, lowcnt, ubase, f);
-    if (f.failed) raise_flag(status, F_OVERFLOW);
-}
-
 // ------------------------------------------------------------------- driver
 
 // Runs independent kernels of one call on the device's side streams: fork()
@@ -1075,6 +865,10 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     if (rc) return rc;
     k_tiers<<<1, 32, 0, s>>>(n, g->dnew, g->status);
     PS_LAUNCH_CHECK();
+    // N_1 and the hub count: the edge filter leaves out the pairs that hub
+    // rows hold; both are read back with the flags for ps_tau_prefix
+    rc = launch_vertex_totals(g, s);
+    if (rc) return rc;
 
     // (3) relabel + sort every row, by tier; the tiers touch disjoint rows, so
     // the long-row tiers run on side streams next to the short-row ones
@@ -1123,70 +917,11 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
                            StoreUbase{g->ubase, n, g->status}, s);
     if (rc) return rc;
 
-    // (5) the edge table; with the region build of the hash set (tables of
-    // at least one region), its kernel also lists every edge's key by region
-    const bool region_build = nnz > 0 && g->eset && L.eset_regions > 0;
-    EsetLists lists{};
-    if (region_build) {
-        int shift = 0;
-        while ((int64_t{1} << shift) < kRegionBuckets) shift++;
-        lists.cur = reinterpret_cast<uint32_t *>(ws + L.eregion);
-        lists.ov_count = lists.cur + L.eset_regions;
-        lists.keys = reinterpret_cast<uint64_t *>(ws + L.ekeys);
-        lists.ov_keys = lists.keys + L.eset_regions * L.eset_cap;
-        lists.cap = L.eset_cap;
-        lists.ov_cap = L.eset_ov_cap;
-        lists.mask = static_cast<uint64_t>(L.eset_buckets - 1);
-        lists.shift = shift;
-        PS_CUDA_TRY(cudaMemsetAsync(lists.cur, 0, sizeof(uint32_t) * (L.eset_regions + 1), s));
-    }
-    rc = build_edge_table(g, s, region_build ? &lists : nullptr);
+    // (5) the edge table, the prefixes and the edge filter
+    if (g->filt) PS_CUDA_TRY(cudaMemsetAsync(g->filt, 0, sizeof(uint32_t) * L.filt_words, s));
+    rc = build_edge_table(g, s);
     if (rc) return rc;
 
-    // (6) the edge hash set.  Only sampling reads it, so it is built on a side
-    // stream beside the prefix step; ps_tau_prefix waits for it before its end
-    // (wait_eset).
-    if (nnz > 0 && g->eset) {
-        cudaStream_t es = s;
-        cudaStream_t side[2];
-        if (get_side_streams(g->device, side) == PS_OK) {
-            PS_CUDA_TRY(cudaEventRecord(g->ev[0], s));
-            PS_CUDA_TRY(cudaStreamWaitEvent(side[0], g->ev[0], 0));
-            es = side[0];
-        }
-        g->eset_pending = true;
-        const uint64_t eset_mask = static_cast<uint64_t>(L.eset_buckets - 1);
-        const int64_t m_cap = L.m_cap;
-        int64_t eb = ((m_cap + kEsetChunk - 1) / kEsetChunk + 7) / 8;  // a warp per chunk of edges
-        if (eb > (int64_t)sms * kEsetBlocksPerSm) eb = (int64_t)sms * kEsetBlocksPerSm;
-        if (eb < 1) eb = 1;
-        if (region_build) {
-            const int64_t regions = L.eset_regions;
-            const int smem = static_cast<int>(kRegionBuckets * kBucketSlots * sizeof(uint64_t));
-            PS_CUDA_TRY(cudaFuncSetAttribute(k_eset_regions, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            const int64_t rb = regions < (int64_t)sms * 3 ? regions : (int64_t)sms * 3;
-            k_eset_regions<<<(unsigned)rb, kRegionThreads, smem, es>>>(regions, kRegionBuckets, lists, g->eset,
-                                                                       g->status);
-            PS_LAUNCH_CHECK();
-            int64_t lb = (L.eset_ov_cap + 255) / 256;
-            if (lb > (int64_t)sms * 4) lb = (int64_t)sms * 4;
-            k_eset_leftovers<<<(unsigned)lb, 256, 0, es>>>(lists, g->eset, g->status);
-            PS_LAUNCH_CHECK();
-            k_eset_spill_fallback<<<(unsigned)eb, 256, 0, es>>>(n, m_cap, g->off, g->col, g->lowcnt, g->ubase,
-                                                               g->eset, eset_mask, g->status);
-            PS_LAUNCH_CHECK();
-        } else {
-            PS_CUDA_TRY(cudaMemsetAsync(g->eset, 0xFF, sizeof(uint64_t) * kBucketSlots * L.eset_buckets, es));
-            k_eset_upper<<<(unsigned)eb, 256, 0, es>>>(n, m_cap, g->off, g->col, g->lowcnt, g->ubase, g->eset,
-                                                      eset_mask, g->status);
-            PS_LAUNCH_CHECK();
-        }
-        PS_CUDA_TRY(cudaEventRecord(g->ev[3], es));
-    }
-
-    // N_1 and the hub count (for ps_tau_prefix), read back with the flags
-    rc = launch_vertex_totals(g, s);
-    if (rc) return rc;
     PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));
     PS_CUDA_TRY(cudaStreamSynchronize(s));
     g->load_totals[0] = st[ST_W_LO];

@@ -225,9 +225,6 @@ int prefix_graph(ps_graph *g, cudaStream_t s) {
     S.tau_shift = tshift;
     S.lambda_shift = lshift;
 
-    // the edge hash set is filled by the load step (on a side stream)
-    const uint64_t eset_mask = g->L.eset_buckets > 0 ? static_cast<uint64_t>(g->L.eset_buckets - 1) : 0;
-
     // per-vertex hash tables
     if (g->vtab) {
         PS_CUDA_TRY(cudaMemsetAsync(g->vtab, 0xFF, sizeof(int32_t) * g->L.vtab_slots, s));
@@ -252,16 +249,14 @@ int prefix_graph(ps_graph *g, cudaStream_t s) {
                                                                         g->hub, words, chunks);
         PS_LAUNCH_CHECK();
     }
-    // The kernels queued after the synchronisation, and the hash set build,
-    // cannot fail on valid state (the hash set's load is at most 1/2, so
-    // every insertion finds a slot); later calls on `stream` are ordered
-    // after them.
+    // The kernels queued after the load's synchronisation cannot fail on
+    // valid state; later calls on `stream` are ordered after them.
 
     GraphDev &D = g->dev;
-    D.eset = g->eset;
-    D.eset_mask = eset_mask;
+    D.filt_off = g->filt ? static_cast<uint64_t>(g->filt - g->hub) : 0;
+    D.filt_words = static_cast<uint32_t>(g->L.filt_words);
     D.vtab = g->vtab;
-    D.adj_mode = g->vtab ? kAdjVtab : (g->eset ? kAdjHash : kAdjSearch);
+    D.adj_mode = g->vtab ? kAdjVtab : (g->filt ? kAdjHash : kAdjSearch);
     D.hub_bit_base = static_cast<int32_t>(g->L.hub_bit_base);
     D.off = g->off;
     D.col = g->col;
@@ -279,10 +274,6 @@ int prefix_graph(ps_graph *g, cudaStream_t s) {
     D.hub_words = static_cast<int32_t>(g->L.hub_words);
     D.tau_shift = tshift;
     D.lam_shift = lshift;
-    // the hash set build of the load step ran beside everything above; later
-    // calls on `s` come after it too
-    const int rc = wait_eset(g, s);
-    if (rc) return rc;
     g->prefixed = true;
     return (S.W == 0 || S.Lambda == 0) ? PS_NO_PATHS : PS_OK;
 }

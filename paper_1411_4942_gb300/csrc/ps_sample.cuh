@@ -11,6 +11,13 @@
 
 namespace ps {
 
+// From this many edges the draw of v' from N(v) takes no line of L1: the rows
+// of the heavy endpoints no longer stay near, and their lines push out the
+// records and rows of the samples beside this one (3-path sampling kernel on
+// the 3M-vertex graph, 115M edges: 10.97 -> 10.44 ms; on R-MAT 20, 15.7M
+// edges, the same load made it slower, 725 -> 762 us).
+constexpr int64_t kFarRowsEdges = int64_t{1} << 25;
+
 // Alg. 1 up to the induced subgraph: the edge e drawn with probability
 // tau_e / W and the two neighbours u' (of u, not v) and v' (of v, not u).
 __device__ __forceinline__ void path3_draw(const GraphDev &g, uint64_t seed, uint64_t id, EdgeRec &e, int32_t &up,
@@ -28,7 +35,7 @@ __device__ __forceinline__ void path3_draw(const GraphDev &g, uint64_t seed, uin
     const int32_t pa = (a == static_cast<uint32_t>(e.iu)) ? e.du - 1 : static_cast<int32_t>(a);
     const int32_t pb = (b == static_cast<uint32_t>(e.jv)) ? e.dv - 1 : static_cast<int32_t>(b);
     up = ldg_i32(g.col + e.ou + pa);
-    vp = ldg_i32(g.col + e.ov + pb);
+    vp = g.m >= kFarRowsEdges ? ldg_i32_once(g.col + e.ov + pb) : ldg_i32(g.col + e.ov + pb);
 }
 
 // Class of a 3-path u'-u-v-v' (u' != v') from its three other pairs
@@ -41,9 +48,7 @@ __device__ __forceinline__ int class3(bool e1, bool e2, bool e3) {
 
 // Class of one Alg. 1 output: 0 = triangle (u' == v'), 1 = 3-path,
 // 2 = tailed triangle, 3 = 4-cycle, 4 = chordal 4-cycle, 5 = 4-clique.
-// HUB_ALL: every adjacency test of a sample may read a hub row (see
-// pair_test3); false for kernels short of registers.
-template <int ADJ, bool HUB_ALL = true>
+template <int ADJ>
 __device__ __forceinline__ int sample_3path(const GraphDev &g, uint64_t seed, uint64_t id) {
     EdgeRec e;
     int32_t up, vp;
@@ -52,7 +57,12 @@ __device__ __forceinline__ int sample_3path(const GraphDev &g, uint64_t seed, ui
     // the path u'-u-v-v' is present; the pairs (u',v), (u,v'), (u',v') decide
     bool e1, e2, e3;
     if (ADJ == kAdjHash) {
-        pair_test3<HUB_ALL>(g, up, e.v, e.u, vp, up, vp, e1, e2, e3);
+        const int32_t x[3] = {up, e.u, up}, y[3] = {e.v, vp, vp};
+        bool r[3];
+        pair_tests<3>(g, x, y, r);
+        e1 = r[0];
+        e2 = r[1];
+        e3 = r[2];
     } else if (ADJ == kAdjVtab) {
         // (u', v) in the table of v, (u, v') in the table of u -- both rows
         // are in the edge record -- and (u', v') in the larger label's table
@@ -99,7 +109,7 @@ __device__ __forceinline__ void centred_draw(const GraphDev &g, uint64_t seed, u
 // 4-cycle, 3 = 4-clique.  u' is drawn among the L_{u,v} entries of N(u)
 // after v, v' among the L_{v,u} entries of N(v) after u; the path is centred
 // (Definition 4.1) iff (u', v') is an edge.
-template <int ADJ, bool HUB_ALL = true>
+template <int ADJ>
 __device__ __forceinline__ int sample_centred(const GraphDev &g, uint64_t seed, uint64_t id) {
     EdgeRec e;
     int32_t up, vp;
@@ -123,9 +133,10 @@ __device__ __forceinline__ int sample_centred(const GraphDev &g, uint64_t seed, 
     if (ADJ == kAdjHash) {
         // the closing edge first; the two chords only for centred paths
         if (!pair_test(g, up, vp)) return 0;  // also u' == v'
-        bool c1, c2;
-        pair_test2<HUB_ALL>(g, e.v, up, e.u, vp, c1, c2);
-        return 1 + (int)c1 + (int)c2;
+        const int32_t x[2] = {up, e.u}, y[2] = {e.v, vp};
+        bool c[2];
+        pair_tests<2>(g, x, y, c);
+        return 1 + (int)c[0] + (int)c[1];
     }
     if (!adjacent(g, up, vp)) return 0;  // also covers u' == v'
     // u' > v and v' > u in label order, so the chord tests search N(v) and N(u)
@@ -134,12 +145,14 @@ __device__ __forceinline__ int sample_centred(const GraphDev &g, uint64_t seed, 
     return 1 + (int)c1 + (int)c2;
 }
 
-// Registers for 768 resident threads per SM (three blocks of 256, 85
-// registers): the hub-row tests otherwise take 98 and drop to two blocks
-// (3-path sampling on R-MAT 20: 1.61 ms capped, 1.74 ms not).  Blocks of 512
-// and 1024 keep the compiler's choice.
+// Registers for 1024 resident threads per SM (64 a thread, no spills): the
+// samplers wait on their dependent loads, so more samples in flight are worth
+// more than registers.  With the hash set's 32-byte buckets the tests needed
+// 80 registers (768 threads); against that, 1024 threads took the adaptive
+// run on a 1M-edge graph from 1.57 to 1.46 ms and 3M + 3M samples on a
+// 10M-edge graph from 394 to 367 us.
 template <int BLOCK>
-constexpr int sample_min_blocks() { return BLOCK <= 256 ? 768 / BLOCK : 1; }
+constexpr int sample_min_blocks() { return BLOCK <= 256 ? 1024 / BLOCK : 1; }
 
 // Per-thread class counters kept in registers.
 struct Counts6 {
