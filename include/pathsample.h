@@ -349,16 +349,18 @@ int ps_csr_from_edges(int64_t n, int64_t n_edges, const int32_t *d_src, const in
  *   (d_a + d_b + d_c - 6), N_4 = 4-cycles, N_5 = sum over edges of
  *   C(t_e, 2) (t_e = triangles through e), N_6 = 4-cliques.
  * g must have been through ps_tau_prefix (it uses the canonical graph, W,
- * N_1 and g's adjacency test).  Work: one adjacency test per upper-part entry
- * of the lower endpoint of every edge, plus one per pair of common upper
- * neighbours (4-cliques), plus the wedges below each vertex (4-cycles).
+ * N_1 and, for vertices with more than 1024 neighbours above them, g's
+ * adjacency test).  Work: one lookup per entry of the upper part of N(b) for
+ * every edge (a, b), |U(a)| / 32 words per triangle at its lowest vertex a
+ * (4-cliques), and the wedges below each vertex (4-cycles).
  *
  * d_scratch: device, 256-byte aligned, at least
  * ps_exact_scratch_bytes(g, 1) bytes; ps_exact_scratch_bytes(g, 0) is the
- * size that lets the 4-cycle pass run on two blocks per SM (each block needs
- * 4 n bytes of counters).  On return its first 4 m bytes hold t_e (uint32,
- * edge order of PS_ARRAY_EDGES).  N (uint64 [6]) and C (int64 [6]) are host
- * arrays.  Synchronises `stream`.  Returns PS_ERR_STATE before
+ * size that lets the part of the 4-cycle pass that counts in global memory
+ * (cycles without one of the top labels) run on two blocks per SM (each
+ * needs 4 n bytes of counters).  On return its first 4 m bytes hold t_e
+ * (uint32, edge order of PS_ARRAY_EDGES).  N (uint64 [6]) and C (int64 [6])
+ * are host arrays.  Synchronises `stream`.  Returns PS_ERR_STATE before
  * ps_tau_prefix, PS_ERR_WORKSPACE for a missing, misaligned or too small
  * scratch, PS_ERR_OVERFLOW when a count does not fit its type. */
 size_t ps_exact_scratch_bytes(const ps_graph *g, int max_blocks);
