@@ -1,6 +1,7 @@
 // ps_api.cu -- the C entry points declared in include/pathsample.h: argument
 // checks, workspace layout, the FP64 estimates and error bars, the
 // end-to-end call and the batched-launch wrappers.
+#include <algorithm>
 #include <atomic>
 #include <climits>
 #include <cmath>
@@ -165,14 +166,12 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.hub_words = (n - l.hub_bit_base + 31) / 32;
     l.filt_words = t.adj_mode == kAdjHash ? filter_words(l.m_cap) : 0;
     l.vtab_slots = t.adj_mode == kAdjVtab ? 2 * nnz : 0;
-    l.radix_tiles = (n + kRadixTile - 1) / kRadixTile;
-    if (l.radix_tiles < 1) l.radix_tiles = 1;
-    int64_t scan_max = 256 * l.radix_tiles;
-    if (n > scan_max) scan_max = n;
-    if (l.m_cap > scan_max) scan_max = l.m_cap;
-    if (l.gcap + 1 > scan_max) scan_max = l.gcap + 1;
-    if (256 * edge_sort_tiles(l.m_cap) > scan_max) scan_max = 256 * edge_sort_tiles(l.m_cap);
-    l.scan_tiles = (scan_max + kScanTile - 1) / kScanTile + 1;
+    // scans of a load: up to 4 passes of the rank sort and of the edge sort,
+    // the row offsets, the edge numbering and the edge table's prefixes
+    const int64_t n_tiles = (n + kScanTile - 1) / kScanTile, m_tiles = (l.m_cap + kScanTile - 1) / kScanTile;
+    const int64_t ns = sort_scan_tiles(n), es = sort_scan_tiles(l.m_cap);
+    l.scan_tiles = std::max(std::max(n_tiles, m_tiles), std::max(ns, es)) + 1;
+    l.scan_words = 4 * (scan_words(ns) + scan_words(es)) + 2 * scan_words(n_tiles) + scan_words(m_tiles);
 
     const size_t n1 = static_cast<size_t>(n > 0 ? n : 1);
     size_t p = 0;
@@ -182,6 +181,7 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
         return at;
     };
     l.status = take(ST_WORDS * sizeof(uint64_t));
+    l.scan_flag = take(static_cast<size_t>(l.scan_words) * sizeof(uint32_t));  // cleared together with the status
     l.off = take((n1 + 1) * sizeof(int64_t));
     l.col = take(static_cast<size_t>(nnz) * sizeof(int32_t));
     l.rank = take(n1 * sizeof(int32_t));
@@ -202,9 +202,7 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.keys1 = take(n1 * sizeof(uint32_t));
     l.vals0 = take(n1 * sizeof(uint32_t));
     l.vals1 = take(n1 * sizeof(uint32_t));
-    l.rcounts = take(static_cast<size_t>(256) * l.radix_tiles * sizeof(uint32_t));
-    l.ecounts = take(static_cast<size_t>(256) * edge_sort_tiles(l.m_cap) * sizeof(uint32_t));
-    l.scan_flag = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(uint32_t));
+    l.counts = take(static_cast<size_t>(256) * std::max(sort_tiles(n), sort_tiles(l.m_cap)) * sizeof(uint32_t));
     l.scan_agg = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(U64x2));
     l.scan_inc = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(U64x2));
     l.total = p;

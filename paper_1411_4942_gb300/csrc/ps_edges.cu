@@ -13,28 +13,18 @@
 // edge order), so the prefix step never reads the records back.
 //
 // The sort is an LSD radix sort with 8-bit digits over the bits of n - 1 (3
-// passes for up to 2^24 vertices).  Each pass: per-tile digit counts, one
-// scan of the counts (digit-major, so it yields every (digit, tile) run's
-// global offset), then a scatter in which every tile ranks its items stably
-// in shared memory -- each warp ranks its own contiguous slice with
-// __match_any_sync, warps in order -- and writes each digit's run
-// contiguously.
+// passes for up to 2^24 vertices; ps_sort.cu).
 //
 // Scratch (the load step's own; nothing here is live afterwards): the
 // ping-pong (key, value) buffers use the prefix regions of the workspace
 // (P_tau and P_lambda, 8 bytes per edge each) and, for the sorted list, the
 // G_tau region (written only later, by the guide-table build); the digit
 // counts have their own region.
+#include <algorithm>
+
 #include "ps_internal.h"
 
 namespace ps {
-
-constexpr int kSortBlock = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortWarps = kSortBlock / 32;
-constexpr int64_t kSortTile = static_cast<int64_t>(kSortBlock) * kSortItems;
-
-int64_t edge_sort_tiles(int64_t m) { return m > 0 ? (m + kSortTile - 1) / kSortTile : 1; }
 
 // (1) The lower arcs of every row, compacted in row-major order: entry
 // t = lbase(r) + p for the p-th entry of row r (p < lowcnt[r]), where
@@ -169,133 +159,7 @@ k_lower_arcs_long(int64_t n, const int64_t *__restrict__ coff, const int32_t *__
     }
 }
 
-// (2a) Digit counts of every tile: counts[digit * tiles + tile].
-__global__ void __launch_bounds__(kSortBlock)
-k_esort_hist(int64_t count, const uint32_t *__restrict__ key, int shift, uint32_t *counts, int64_t tiles) {
-    __shared__ uint32_t s_h[kSortWarps][256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortBlock) (&s_h[0][0])[d] = 0u;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)warp * (32 * kSortItems) + lane;
-    // all of a thread's keys in flight at once, then the counts
-    uint32_t k[kSortItems];
-#pragma unroll
-    for (int q = 0; q < kSortItems; q++) {
-        const int64_t idx = base + 32 * q;
-        k[q] = idx < count ? __ldg(key + idx) : 0u;
-    }
-#pragma unroll
-    for (int q = 0; q < kSortItems; q++)
-        if (base + 32 * q < count) atomicAdd(&s_h[warp][(k[q] >> shift) & 255u], 1u);
-    __syncthreads();
-    uint32_t c = 0;
-#pragma unroll
-    for (int w = 0; w < kSortWarps; w++) c += s_h[w][threadIdx.x];
-    counts[(int64_t)threadIdx.x * tiles + blockIdx.x] = c;
-}
-
-struct LoadCounts {
-    const uint32_t *p;
-    __device__ uint32_t operator()(int64_t i) const { return p[i]; }
-};
-struct StoreCountsExcl {
-    uint32_t *p;
-    __device__ void operator()(int64_t i, uint32_t exc, uint32_t) const { p[i] = exc; }
-};
-
-// (2b) Stable scatter of one tile by the digit at `shift`; offsets[digit *
-// tiles + tile] is where the tile's run of that digit starts.  Item order
-// within a tile: warp w owns the w-th slice of 32 * kSortItems items and
-// walks it in rows of 32 lanes, so (warp, row, lane) is index order.  Only
-// the keys and their ranks stay in registers (values are read when placed),
-// which keeps four blocks resident per SM.
-__global__ void __launch_bounds__(kSortBlock, 4)
-k_esort_scatter(int64_t count, const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-                uint32_t *__restrict__ kout, uint32_t *__restrict__ vout, int shift,
-                const uint32_t *__restrict__ offsets, int64_t tiles) {
-    __shared__ uint32_t s_key[kSortTile];
-    __shared__ uint32_t s_val[kSortTile];
-    __shared__ uint32_t s_cnt[kSortWarps][256];  // per-warp counts, then per-warp bases
-    __shared__ uint32_t s_start[256];            // first tile-local slot of each digit
-    __shared__ uint32_t s_glob[256];             // global start of the tile's run of each digit
-    __shared__ uint32_t s_wsum[kSortWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
-    const int64_t base = tile0 + (int64_t)warp * (32 * kSortItems) + lane;
-    for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortBlock) (&s_cnt[0][0])[d] = 0u;
-    s_glob[threadIdx.x] = offsets[(int64_t)threadIdx.x * tiles + blockIdx.x];
-    uint32_t k[kSortItems];
-#pragma unroll
-    for (int q = 0; q < kSortItems; q++) {
-        const int64_t idx = base + 32 * q;
-        k[q] = idx < count ? kin[idx] : 0u;
-    }
-    __syncthreads();
-    // stable rank of every item among its warp's items of the same digit
-    // (below 32 * kSortItems, two to a register)
-    static_assert(32 * kSortItems <= 65536 && kSortItems % 2 == 0, "ranks packed in 16 bits");
-    uint32_t rank2[kSortItems / 2];
-#pragma unroll
-    for (int q = 0; q < kSortItems; q++) {
-        const bool ok = base + 32 * q < count;
-        const uint32_t d = ok ? ((k[q] >> shift) & 255u) : 256u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t before = ok ? s_cnt[warp][d] : 0u;
-        const uint32_t r = before + __popc(peers & lanemask_lt());
-        if (q & 1) rank2[q / 2] |= r << 16;
-        else rank2[q / 2] = r;
-        __syncwarp();
-        if (ok && lane == __ffs(peers) - 1) s_cnt[warp][d] = before + __popc(peers);
-        __syncwarp();
-    }
-    __syncthreads();
-    // thread t = digit t: per-warp bases within the digit, then the digits'
-    // tile-local starts (a block scan of the digit totals)
-    {
-        const int d = threadIdx.x;
-        uint32_t run = 0;
-#pragma unroll
-        for (int w = 0; w < kSortWarps; w++) {
-            const uint32_t c = s_cnt[w][d];
-            s_cnt[w][d] = run;
-            run += c;
-        }
-        uint32_t x = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_wsum[warp] = x;
-        __syncthreads();
-        uint32_t before = 0;
-#pragma unroll
-        for (int w = 0; w < kSortWarps; w++) before += (w < warp) ? s_wsum[w] : 0u;
-        s_start[d] = before + x - run;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kSortItems; q++) {
-        const int64_t idx = base + 32 * q;
-        if (idx < count) {
-            const uint32_t d = (k[q] >> shift) & 255u;
-            const uint32_t p = s_start[d] + s_cnt[warp][d] + ((rank2[q / 2] >> (16 * (q & 1))) & 0xFFFFu);
-            s_key[p] = k[q];
-            s_val[p] = vin[idx];
-        }
-    }
-    __syncthreads();
-    const int64_t n_tile = count - tile0 < kSortTile ? count - tile0 : kSortTile;
-    for (int p = threadIdx.x; p < n_tile; p += kSortBlock) {
-        const uint32_t kk = s_key[p];
-        const uint32_t d = (kk >> shift) & 255u;
-        const int64_t g = static_cast<int64_t>(s_glob[d]) + (p - static_cast<int64_t>(s_start[d]));
-        kout[g] = kk;
-        vout[g] = s_val[p];
-    }
-}
-
-// (3) Edge j from the sorted entry j: u its key, i its arc (in row v, at
+// (2) Edge j from the sorted entry j: u its key, i its arc (in row v, at
 // position jv), v the (j - ubase[u])-th upper neighbour of u.  The checks
 // that u's upper range holds j and that arc i lies in v's row (where, holding
 // u < v, it is a lower arc) hold exactly when the input is symmetric (every
@@ -378,7 +242,7 @@ __device__ __forceinline__ void edge_group(int64_t j0, int step, int64_t m, int6
 constexpr int kRecItems = 4;
 constexpr int kRecScanItems = 8;
 static_assert(kRecScanItems % kRecItems == 0, "whole groups per tile");
-static_assert(kScanBlock * kRecScanItems >= kScanTile, "scan flags are reset per kScanTile items");
+static_assert(kScanBlock * kRecScanItems >= kScanTile, "the workspace holds scan flags per kScanTile items");
 
 // (Capped at 64 registers, four blocks per SM: while one block waits at the
 // tile's barriers or on its look-back, the others build records; the
@@ -442,33 +306,30 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
             PS_LAUNCH_CHECK();
         }
     }
-    const int64_t tiles = edge_sort_tiles(m);
-    uint32_t *counts = reinterpret_cast<uint32_t *>(ws + L.ecounts);
     for (int pass = 0; pass < passes; pass++) {
         const int shift = 8 * pass;
         const bool last = pass == passes - 1;
         uint32_t *ko = last ? kg : kb, *vo = last ? vg : vb;
-        k_esort_hist<<<(unsigned)tiles, kSortBlock, 0, s>>>(m, ka, shift, counts, tiles);
-        PS_LAUNCH_CHECK();
-        int rc = run_scan<uint32_t>(g, 0, 256 * tiles, 0u, OpSum(), LoadCounts{counts}, StoreCountsExcl{counts}, s);
+        ScanState<uint32_t> scan{};
+        int rc = sort_scan_tiles(m) ? take_scan(g, sort_scan_tiles(m), &scan) : PS_OK;
         if (rc) return rc;
-        k_esort_scatter<<<(unsigned)tiles, kSortBlock, 0, s>>>(m, ka, va, ko, vo, shift, counts, tiles);
-        PS_LAUNCH_CHECK();
-        uint32_t *t = ka;
+        rc = sort_pass({m, nullptr, ka, va, ko, vo, shift, std::max(1, std::min(8, bits - shift)), 0,
+                        reinterpret_cast<uint32_t *>(ws + L.counts)}, scan, s);
+        if (rc) return rc;
+        kb = ka;
+        vb = va;
         ka = ko;
-        kb = t;
-        t = va;
         va = vo;
-        vb = t;
     }
     // ka/va: the sorted list, in the G_tau region
-    int rc = reset_scan(g, 3, m, s);
-    if (rc) return rc;
     const EdgeFilter F{g->filt, static_cast<uint32_t>(L.filt_words), static_cast<int32_t>(L.hub_bit_base)};
     const int64_t stiles = (m + kScanBlock * kRecScanItems - 1) / (kScanBlock * kRecScanItems);
+    ScanState<U64x2> scan;
+    const int rc = take_scan(g, stiles, &scan);
+    if (rc) return rc;
     k_edge_records_scan<<<(unsigned)stiles, kScanBlock, 0, s>>>(
         m, n, ka, va, g->off, g->col, g->lowcnt, g->ubase, g->rec, g->status, F,
-        scan_state<U64x2>(g, 3), g->ptau, g->plam);
+        scan, g->ptau, g->plam);
     PS_LAUNCH_CHECK();
     return PS_OK;
 }

@@ -29,10 +29,6 @@ constexpr int64_t kCoarseGuideEdges = int64_t{1} << 25;  // default guide of m/4
 constexpr int kScanBlock = 256;
 constexpr int kScanItems = 8;
 constexpr int64_t kScanTile = kScanBlock * kScanItems;
-// Rank sort (LSD radix, 8-bit digits).
-constexpr int kRadixBlock = 256;
-constexpr int kRadixItems = 16;
-constexpr int64_t kRadixTile = kRadixBlock * kRadixItems;
 
 struct Tuning {
     int block_size;
@@ -46,16 +42,13 @@ struct Tuning {
     int draw_order;        // ordered samplers: 0 by size, 1 always, -1 never
 };
 Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz);
-// N_1 and the hub count into the status words (ps_prefix.cu); queued by the
-// load step once the degrees are known
-int launch_vertex_totals(ps_graph *g, cudaStream_t s);
-
 struct Layout {
-    int64_t n, nnz, m_cap, gcap, hub_cap, hub_words, hub_bit_base, radix_tiles, scan_tiles;
+    int64_t n, nnz, m_cap, gcap, hub_cap, hub_words, hub_bit_base, scan_tiles;
+    int64_t scan_words;    // zeroed words of one load's scans (tile counters and flags)
     int64_t filt_words;    // 32-bit words of the edge filter; 0 without it
     int64_t vtab_slots;    // 0 without the per-vertex tables
     size_t status, off, col, rank, lowcnt, ubase, dnew, rec, ptau, plam, gtau, glam, hub, filt, vtab;
-    size_t keys0, keys1, vals0, vals1, rcounts, ecounts, scan_flag, scan_agg, scan_inc;
+    size_t keys0, keys1, vals0, vals1, counts, scan_flag, scan_agg, scan_inc;
     size_t total;
 };
 bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L);
@@ -69,6 +62,7 @@ struct ps_graph {
     int device;
     int sm_count;
     int64_t n, nnz, m, d_max;
+    int64_t scan_used;  // words of the scan region taken by this load's scans
     // device arrays (inside ws)
     ps::u64 *status;
     int64_t *off;
@@ -122,32 +116,49 @@ void count_launch();
         PS_CUDA_TRY(cudaGetLastError());        \
     } while (0)
 
-// Stable LSD radix-sort passes of ps_load.cu (8-bit digit at `shift`,
-// uint32 keys with uint32 values, tiles of kRadixTile items): per-tile digit
-// counts stored digit-major, then the scatter after their exclusive scan.
-__global__ void __launch_bounds__(kRadixBlock)
-k_radix_hist(int64_t n, const uint32_t *__restrict__ keys, int shift, uint32_t *counts, int64_t tiles);
-__global__ void __launch_bounds__(kRadixBlock)
-k_radix_scatter(int64_t n, const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-                uint32_t *__restrict__ kout, uint32_t *__restrict__ vout, int shift,
-                const uint32_t *__restrict__ offsets, int64_t tiles);
+// One stable pass of a radix sort (ps_sort.cu) by `bits` (at most 8) bits of
+// the key from `shift` on; keys have no bits above those of the sort's last
+// pass.  vin null: the values are the items' indices.  vshift > 0: the digit
+// goes on with the value's lowest bits, vshift of its bits being the key's.
+// dcount (device, may be null) bounds the items at run time.  counts: 256
+// words per tile.
+struct SortPass {
+    int64_t count;
+    const u64 *dcount;
+    const uint32_t *kin, *vin;
+    uint32_t *kout, *vout;
+    int shift, bits, vshift;
+    uint32_t *counts;
+};
+int64_t sort_tiles(int64_t count);
+// tiles of the pass's scan (0: it needs none and `scan` is not touched)
+int64_t sort_scan_tiles(int64_t count);
+int sort_pass(const SortPass &p, const ScanState<uint32_t> &scan, cudaStream_t s);
 
-// scan helpers (ps_load.cu)
+// The scans of a load share the workspace's value arrays (one scan at a time
+// per graph, in stream order) and take their tile counter and flags from a
+// region that the load clears once.
+inline int64_t scan_words(int64_t tiles) { return (tiles + 2 + 3) & ~int64_t{3}; }
 template <typename T>
-ScanState<T> scan_state(ps_graph *g, int counter_slot);
-int reset_scan(ps_graph *g, int counter_slot, int64_t count, cudaStream_t s);
-
-// Scans `count` items of the graph's workspace through the shared scan
-// state (one scan at a time per graph, in stream order).
+inline int take_scan(ps_graph *g, int64_t tiles, ScanState<T> *st) {
+    const int64_t words = scan_words(tiles);
+    if (tiles > g->L.scan_tiles || g->scan_used + words > g->L.scan_words) return PS_ERR_WORKSPACE;
+    st->counter = reinterpret_cast<uint32_t *>(g->ws + g->L.scan_flag) + g->scan_used;
+    st->flag = st->counter + 1;
+    st->agg = reinterpret_cast<T *>(g->ws + g->L.scan_agg);
+    st->inc = reinterpret_cast<T *>(g->ws + g->L.scan_inc);
+    st->status = g->status;
+    g->scan_used += words;
+    return PS_OK;
+}
 template <typename T, typename Op, typename Load, typename Store>
-inline int run_scan(ps_graph *g, int slot, int64_t count, T identity, Op op, Load load, Store store,
-                    cudaStream_t s) {
+inline int run_scan(ps_graph *g, int64_t count, T identity, Op op, Load load, Store store, cudaStream_t s) {
     if (count <= 0) return PS_OK;
-    int rc = reset_scan(g, slot, count, s);
-    if (rc) return rc;
     const int64_t tiles = (count + kScanTile - 1) / kScanTile;
-    k_scan<T, kScanBlock, kScanItems><<<(unsigned)tiles, kScanBlock, 0, s>>>(
-        count, scan_state<T>(g, slot), identity, op, load, store);
+    ScanState<T> st;
+    const int rc = take_scan(g, tiles, &st);
+    if (rc) return rc;
+    k_scan<T, kScanBlock, kScanItems><<<(unsigned)tiles, kScanBlock, 0, s>>>(count, st, identity, op, load, store);
     PS_LAUNCH_CHECK();
     return PS_OK;
 }
@@ -157,10 +168,6 @@ inline int run_scan(ps_graph *g, int slot, int64_t count, T identity, Op op, Loa
 // in the edge filter (cleared before), and raises F_ASYM for an asymmetric
 // input.
 int build_edge_table(ps_graph *g, cudaStream_t s);
-// Tiles of the edge table's radix sort for m edges (its digit counts take
-// 256 words per tile).
-int64_t edge_sort_tiles(int64_t m);
-
 // steps (one translation unit each)
 int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStream_t s);
 int prefix_graph(ps_graph *g, cudaStream_t s);

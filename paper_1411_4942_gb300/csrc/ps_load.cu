@@ -2,41 +2,18 @@
 // degree order of Section 4 made the integer order by relabelling, sorted
 // adjacency lists, and the edge table (u < v, row-major) with the position of
 // each edge in both endpoint lists.
+#include <algorithm>
 #include <climits>
+#include <utility>
 
 #include "ps_internal.h"
 
 namespace ps {
 
-// ------------------------------------------------------------ scan plumbing
-
-template <typename T>
-ScanState<T> scan_state(ps_graph *g, int counter_slot) {
-    ScanState<T> s;
-    s.flag = reinterpret_cast<uint32_t *>(g->ws + g->L.scan_flag);
-    s.agg = reinterpret_cast<T *>(g->ws + g->L.scan_agg);
-    s.inc = reinterpret_cast<T *>(g->ws + g->L.scan_inc);
-    s.counter = reinterpret_cast<uint32_t *>(g->status + ST_COUNTER + counter_slot);
-    s.status = g->status;
-    return s;
-}
-template ScanState<uint32_t> scan_state<uint32_t>(ps_graph *, int);
-template ScanState<int64_t> scan_state<int64_t>(ps_graph *, int);
-template ScanState<int32_t> scan_state<int32_t>(ps_graph *, int);
-template ScanState<U64x2> scan_state<U64x2>(ps_graph *, int);
-
-int reset_scan(ps_graph *g, int counter_slot, int64_t count, cudaStream_t s) {
-    const int64_t tiles = (count + kScanTile - 1) / kScanTile;
-    if (tiles > g->L.scan_tiles) return PS_ERR_WORKSPACE;
-    PS_CUDA_TRY(cudaMemsetAsync(g->ws + g->L.scan_flag, 0, sizeof(uint32_t) * (tiles + 1), s));
-    PS_CUDA_TRY(cudaMemsetAsync(g->status + ST_COUNTER + counter_slot, 0, sizeof(uint64_t), s));
-    return PS_OK;
-}
-
 // ------------------------------------------------------------------ degrees
 
 __global__ void k_degrees(int64_t n, int64_t nnz, const int64_t *__restrict__ off,
-                          uint32_t *__restrict__ keys, uint32_t *__restrict__ vals, u64 *status) {
+                          uint32_t *__restrict__ keys, u64 *status) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t0 == 0) {
@@ -53,7 +30,6 @@ __global__ void k_degrees(int64_t n, int64_t nnz, const int64_t *__restrict__ of
         }
         if (d > n - 1) longrow = true;  // cannot be a simple row
         keys[v] = static_cast<uint32_t>(d);
-        vals[v] = static_cast<uint32_t>(v);
         dmax = max(dmax, static_cast<uint32_t>(d));
     }
     if (bad) raise_flag(status, F_ARG);
@@ -64,82 +40,40 @@ __global__ void k_degrees(int64_t n, int64_t nnz, const int64_t *__restrict__ of
         atomicMax(reinterpret_cast<unsigned long long *>(status + ST_DMAX), (unsigned long long)dmax);
 }
 
-// ------------------------------------------------ rank: stable LSD radix sort
-
-// Per-tile digit histogram, stored digit-major: counts[digit * tiles + tile].
-__global__ void __launch_bounds__(kRadixBlock)
-k_radix_hist(int64_t n, const uint32_t *__restrict__ keys, int shift, uint32_t *counts, int64_t tiles) {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    for (int i = threadIdx.x; i < kRadixTile; i += kRadixBlock) {
-        const int64_t idx = base + i;
-        if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    counts[(int64_t)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
-}
-
-// Stable scatter: items are ranked round by round in input order; within a
-// round, lanes with equal digits are ranked by __match_any_sync and warps by
-// their per-digit counts.
-__global__ void __launch_bounds__(kRadixBlock)
-k_radix_scatter(int64_t n, const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-                uint32_t *__restrict__ kout, uint32_t *__restrict__ vout, int shift,
-                const uint32_t *__restrict__ offsets, int64_t tiles) {
-    constexpr int NW = kRadixBlock / 32;
-    __shared__ uint32_t s_base[256];
-    __shared__ uint32_t s_wcnt[NW][256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    s_base[threadIdx.x] = offsets[(int64_t)threadIdx.x * tiles + blockIdx.x];
-    for (int w = 0; w < NW; w++) s_wcnt[w][threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    for (int round = 0; round < kRadixItems; round++) {
-        const int64_t idx = base + (int64_t)round * kRadixBlock + threadIdx.x;
-        const bool valid = idx < n;
-        const uint32_t key = valid ? kin[idx] : 0u;
-        const uint32_t digit = valid ? ((key >> shift) & 255u) : 256u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-        const uint32_t wrank = __popc(peers & lanemask_lt());
-        if (valid && lane == __ffs(peers) - 1) s_wcnt[warp][digit] = __popc(peers);
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = s_base[digit] + wrank;
-            for (int w = 0; w < warp; w++) pos += s_wcnt[w][digit];
-            kout[pos] = key;
-            vout[pos] = vin[idx];
-        }
-        __syncthreads();
-        uint32_t tot = 0;
-        for (int w = 0; w < NW; w++) {
-            tot += s_wcnt[w][threadIdx.x];
-            s_wcnt[w][threadIdx.x] = 0;
-        }
-        s_base[threadIdx.x] += tot;
-        __syncthreads();
-    }
-}
-
-struct LoadU32 {
-    const uint32_t *p;
-    __device__ uint32_t operator()(int64_t i) const { return p[i]; }
-};
-struct StoreExclU32 {
-    uint32_t *p;
-    __device__ void operator()(int64_t i, uint32_t exc, uint32_t) const { p[i] = exc; }
-};
-
-// rank[v] = position of v in (degree, id) order; dnew[r] = degree of row r
-__global__ void k_rank(int64_t n, const uint32_t *__restrict__ skeys, const uint32_t *__restrict__ svals,
-                       int32_t *rank, int32_t *dnew, uint32_t *inv) {
+// The sorted (degree, vertex) pairs, position r = label r: rank[v] = the label
+// of v, dnew[r] = its degree, lowcnt[r] = 0; the first label whose degree
+// exceeds each row-length limit; N_1 = sum_v C(d_v, 3) (128-bit); and the
+// number of hub rows: the top `hub_cap` labels whose degree is at least
+// `hub_min`.
+__global__ void __launch_bounds__(256)
+k_rank(int64_t n, const uint32_t *__restrict__ skeys, const uint32_t *__restrict__ svals, int32_t *rank,
+       int32_t *dnew, int32_t *lowcnt, int64_t hub_cap, int64_t hub_min, u64 *status) {
+    const uint32_t lim[5] = {0, kTierA, kTierB, kTierC, kLongRow};
+    const int slot[5] = {ST_TIER, ST_TIER + 1, ST_TIER + 2, ST_TIER + 3, ST_LONG};
+    uint64_t lo = 0, hi = 0;
+    unsigned long long hubs = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
-        const uint32_t v = svals[r];
-        rank[v] = static_cast<int32_t>(r);
-        dnew[r] = static_cast<int32_t>(skeys[r]);
-        if (inv) inv[r] = v;
+        const uint32_t d = __ldg(skeys + r);
+        rank[__ldg(svals + r)] = static_cast<int32_t>(r);
+        dnew[r] = static_cast<int32_t>(d);
+        lowcnt[r] = 0;
+        const uint32_t before = r ? __ldg(skeys + r - 1) : 0u;
+#pragma unroll
+        for (int t = 0; t < 5; t++) {
+            if (d > lim[t] && (r == 0 || before <= lim[t])) status[slot[t]] = static_cast<u64>(r);
+            if (r == n - 1 && d <= lim[t]) status[slot[t]] = static_cast<u64>(n);
+        }
+        if (r == n - 1) status[ST_TIER + 4] = static_cast<u64>(n);
+        add_stars(lo, hi, d);
+        hubs += r >= n - hub_cap && d >= static_cast<uint64_t>(hub_min);
+    }
+    warp_add128(lo, hi);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) hubs += __shfl_down_sync(0xffffffffu, hubs, o);
+    if ((threadIdx.x & 31) == 0) {
+        if (lo | hi) atomic_add128(status + ST_N1_LO, lo, hi);
+        if (hubs) atomicAdd(reinterpret_cast<unsigned long long *>(status + ST_HUBS), hubs);
     }
 }
 
@@ -155,23 +89,6 @@ struct StoreOffsets {
         if (i == n - 1) off[n] = inc;
     }
 };
-
-// first row whose degree exceeds each tier limit (rows are degree-sorted)
-__global__ void k_tiers(int64_t n, const int32_t *__restrict__ dnew, u64 *status) {
-    const int lim[5] = {0, kTierA, kTierB, kTierC, kLongRow};
-    const int slot[5] = {ST_TIER, ST_TIER + 1, ST_TIER + 2, ST_TIER + 3, ST_LONG};
-    const int t = threadIdx.x;
-    if (t < 5) {
-        int64_t lo = 0, hi = n;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (dnew[mid] > lim[t]) hi = mid;
-            else lo = mid + 1;
-        }
-        status[slot[t]] = static_cast<u64>(lo);
-    }
-    if (t == 5) status[ST_TIER + 4] = static_cast<u64>(n);
-}
 
 // ------------------------------------------------------- row relabel + sort
 
@@ -817,15 +734,17 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     const int64_t n = L.n, nnz = L.nnz;
     char *ws = g->ws;
     const int sms = g->sm_count;
-    PS_CUDA_TRY(cudaMemsetAsync(g->status, 0, ST_WORDS * sizeof(uint64_t), s));
-    PS_CUDA_TRY(cudaMemsetAsync(g->lowcnt, 0, sizeof(int32_t) * (n > 0 ? n : 1), s));
+    // the status words and, right behind them, the counters and flags of every
+    // scan of this load
+    g->scan_used = 0;
+    PS_CUDA_TRY(cudaMemsetAsync(g->status, 0, L.scan_flag - L.status + sizeof(uint32_t) * L.scan_words, s));
     uint32_t *k0 = reinterpret_cast<uint32_t *>(ws + L.keys0);
     uint32_t *k1 = reinterpret_cast<uint32_t *>(ws + L.keys1);
     uint32_t *v0 = reinterpret_cast<uint32_t *>(ws + L.vals0);
     uint32_t *v1 = reinterpret_cast<uint32_t *>(ws + L.vals1);
 
     // (1) degrees and offset validation; nothing else may index with bad offsets
-    k_degrees<<<sms * 8, 256, 0, s>>>(n, nnz, d_off, k0, v0, g->status);
+    k_degrees<<<sms * 8, 256, 0, s>>>(n, nnz, d_off, k0, g->status);
     PS_LAUNCH_CHECK();
     uint64_t st[ST_WORDS];
     PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));
@@ -833,41 +752,30 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     if (st[ST_FLAGS] & F_ARG) return PS_ERR_ARG;
     g->d_max = static_cast<int64_t>(st[ST_DMAX]);
 
-    // (2) stable LSD radix sort of (degree, id): ties keep increasing id
-    int bits = 0;
+    // (2) stable radix sort of (degree, id): ties keep increasing id
+    int bits = 1;
     while (bits < 32 && (static_cast<uint64_t>(g->d_max) >> bits) != 0) bits++;
-    uint32_t *counts = reinterpret_cast<uint32_t *>(ws + L.rcounts);
-    const int64_t tiles = L.radix_tiles;
+    int rc = PS_OK;
     for (int shift = 0; shift < bits && n > 0; shift += 8) {
-        k_radix_hist<<<(unsigned)tiles, kRadixBlock, 0, s>>>(n, k0, shift, counts, tiles);
-        PS_LAUNCH_CHECK();
-        int rc = run_scan<uint32_t>(g, 0, 256 * tiles, 0u, OpSum(), LoadU32{counts},
-                                    StoreExclU32{counts}, s);
+        ScanState<uint32_t> scan{};
+        if (sort_scan_tiles(n)) rc = take_scan(g, sort_scan_tiles(n), &scan);
         if (rc) return rc;
-        k_radix_scatter<<<(unsigned)tiles, kRadixBlock, 0, s>>>(n, k0, v0, k1, v1, shift, counts,
-                                                                tiles);
-        PS_LAUNCH_CHECK();
-        uint32_t *t = k0;
-        k0 = k1;
-        k1 = t;
-        t = v0;
-        v0 = v1;
-        v1 = t;
+        rc = sort_pass({n, nullptr, k0, shift ? v0 : nullptr, k1, v1, shift, std::min(8, bits - shift), 0,
+                        reinterpret_cast<uint32_t *>(ws + L.counts)}, scan, s);
+        if (rc) return rc;
+        std::swap(k0, k1);
+        std::swap(v0, v1);
     }
-    // k0/v0 hold the sorted (degree, vertex) pairs; v1 receives inv[r]
+    // k0 / v0 hold the sorted (degree, vertex) pairs: v0[r] is the vertex with label r
     if (n > 0) {
-        k_rank<<<sms * 8, 256, 0, s>>>(n, k0, v0, g->rank, g->dnew, v1);
+        k_rank<<<sms * 8, 256, 0, s>>>(n, k0, v0, g->rank, g->dnew, g->lowcnt, L.hub_cap, g->tune.hub_min_degree, g->status);
         PS_LAUNCH_CHECK();
+    } else {
+        PS_CUDA_TRY(cudaMemsetAsync(g->off, 0, sizeof(int64_t), s));
+        PS_CUDA_TRY(cudaMemsetAsync(g->ubase, 0, sizeof(int64_t), s));
     }
-    const uint32_t *inv = v1;
-    PS_CUDA_TRY(cudaMemsetAsync(g->off, 0, sizeof(int64_t), s));
-    int rc = run_scan<int64_t>(g, 1, n, (int64_t)0, OpSum(), LoadDeg{g->dnew}, StoreOffsets{g->off, n}, s);
-    if (rc) return rc;
-    k_tiers<<<1, 32, 0, s>>>(n, g->dnew, g->status);
-    PS_LAUNCH_CHECK();
-    // N_1 and the hub count: the edge filter leaves out the pairs that hub
-    // rows hold; both are read back with the flags for ps_tau_prefix
-    rc = launch_vertex_totals(g, s);
+    const uint32_t *inv = v0;
+    rc = run_scan<int64_t>(g, n, (int64_t)0, OpSum(), LoadDeg{g->dnew}, StoreOffsets{g->off, n}, s);
     if (rc) return rc;
 
     // (3) relabel + sort every row, by tier; the tiers touch disjoint rows, so
@@ -912,8 +820,7 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     }
 
     // (4) the edge numbering: ubase[r] = the edges (upper arcs) of the rows before r
-    PS_CUDA_TRY(cudaMemsetAsync(g->ubase, 0, sizeof(int64_t), s));
-    rc = run_scan<int64_t>(g, 2, n, (int64_t)0, OpSum(), LoadUp{g->dnew, g->lowcnt},
+    rc = run_scan<int64_t>(g, n, (int64_t)0, OpSum(), LoadUp{g->dnew, g->lowcnt},
                            StoreUbase{g->ubase, n, g->status}, s);
     if (rc) return rc;
 

@@ -7,40 +7,6 @@
 
 namespace ps {
 
-// N_1 = sum_v C(d_v, 3) (128-bit) and the number of hub rows: the top
-// `hub_cap` labels whose degree is at least `hub_min` (labels are in degree
-// order, so these are the last rows).
-__global__ void __launch_bounds__(256)
-k_vertex_totals(int64_t n, const int32_t *__restrict__ dnew, int64_t hub_cap, int64_t hub_min, u64 *status) {
-    uint64_t lo = 0, hi = 0;
-    unsigned long long hubs = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
-        const uint64_t d = static_cast<uint64_t>(dnew[r]);
-        if (d >= 3) {
-            // d (d - 1) (d - 2) / 6 with d < 2^31: the product fits in 128 bits
-            const uint64_t a = d * (d - 1);  // < 2^62
-            const uint64_t b = d - 2;
-            uint64_t plo = a * b, phi = __umul64hi(a, b);
-            // divide the 128-bit product by 6 (exact)
-            const uint64_t qhi = phi / 6, rhi = phi % 6;
-            // (rhi * 2^64 + plo) / 6 with rhi < 6
-            const unsigned __int128 rest = (static_cast<unsigned __int128>(rhi) << 64) | plo;
-            const uint64_t qlo = static_cast<uint64_t>(rest / 6);
-            add128(lo, hi, qlo);
-            hi += qhi;
-        }
-        if (r >= n - hub_cap && d >= static_cast<uint64_t>(hub_min)) hubs++;
-    }
-    warp_add128(lo, hi);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) hubs += __shfl_down_sync(0xffffffffu, hubs, o);
-    if ((threadIdx.x & 31) == 0) {
-        if (lo | hi) atomic_add128(status + ST_N1_LO, lo, hi);
-        if (hubs) atomicAdd(reinterpret_cast<unsigned long long *>(status + ST_HUBS), hubs);
-    }
-}
-
 // Guide table: bucket b holds r in [b << shift, (b + 1) << shift), and G[b]
 // is the edge that the first r of bucket b selects.  Edge j covers r in
 // [P[j-1], P[j] - 1], so it owns the buckets whose first r falls in that
@@ -182,13 +148,6 @@ static int build_guide(ps_graph *g, const uint64_t *P, uint64_t total, int32_t *
     int64_t blocks = (m + 256 * kGuideGroups - 1) / (256 * kGuideGroups);
     if (blocks > (int64_t)g->sm_count * (occ > 0 ? occ : 1)) blocks = (int64_t)g->sm_count * (occ > 0 ? occ : 1);
     k_guide_fill<<<(unsigned)blocks, 256, 0, s>>>(m, P, shift, G, B);
-    PS_LAUNCH_CHECK();
-    return PS_OK;
-}
-
-int launch_vertex_totals(ps_graph *g, cudaStream_t s) {
-    if (g->n <= 0) return PS_OK;
-    k_vertex_totals<<<g->sm_count * 8, 256, 0, s>>>(g->n, g->dnew, g->L.hub_cap, g->tune.hub_min_degree, g->status);
     PS_LAUNCH_CHECK();
     return PS_OK;
 }

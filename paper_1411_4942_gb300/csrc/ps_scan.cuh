@@ -80,6 +80,20 @@ __device__ __forceinline__ void warp_add128(uint64_t &lo, uint64_t &hi) {
     }
 }
 
+// C(d, 3) added to a 128-bit sum, d < 2^31 (the product fits in 128 bits).
+__device__ __forceinline__ void add_stars(uint64_t &lo, uint64_t &hi, uint64_t d) {
+    if (d < 3) return;
+    const uint64_t a = d * (d - 1);  // < 2^62
+    const uint64_t b = d - 2;
+    const uint64_t plo = a * b, phi = __umul64hi(a, b);
+    // divide the 128-bit product by 6 (exact)
+    const uint64_t qhi = phi / 6, rhi = phi % 6;
+    // (rhi * 2^64 + plo) / 6 with rhi < 6
+    const unsigned __int128 rest = (static_cast<unsigned __int128>(rhi) << 64) | plo;
+    add128(lo, hi, static_cast<uint64_t>(rest / 6));
+    hi += qhi;
+}
+
 // ------------------------------------------------ decoupled look-back scan
 
 // Tile status for the single-pass scan of Merrill & Garland (2016): a flag

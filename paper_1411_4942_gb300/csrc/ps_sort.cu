@@ -1,0 +1,257 @@
+// ps_sort.cu -- one pass of a stable LSD radix sort of (uint32 key, uint32
+// value) pairs by a digit of up to 8 bits: used by the degree order (Section
+// 4), the transposition that builds the edge table, and edge-list ingest.
+//
+// A pass counts the digits of every tile (digit-major), turns the counts into
+// run offsets, and scatters: every tile ranks its items stably in shared
+// memory -- each warp its own contiguous slice, warps in order -- and writes
+// each digit's run contiguously.
+//
+// The lanes of a row that share a digit are found by one ballot per digit
+// bit.  __match_any_sync takes longer the more different values a warp holds
+// (with random 8-bit digits the scatter waited on it most of the time): 115M
+// pairs took 0.79 ms per scatter with it.
+//
+// A sort by (value, key) -- the value as the more significant half -- can take
+// its digits over the boundary of the two (`vshift`): 40 bits of an R-MAT 20
+// edge in 5 passes instead of 6.
+//
+// Up to kDirectTiles tiles every scatter block adds up the raw counts it needs
+// itself, which saves the scan's launch (small graphs are bound by the number
+// of launches); above that one look-back scan makes the offsets.
+#include "ps_internal.h"
+
+namespace ps {
+
+constexpr int kSortBlock = 256;
+constexpr int kSortItems = 16;
+constexpr int kSortWarps = kSortBlock / 32;
+constexpr int64_t kSortTile = static_cast<int64_t>(kSortBlock) * kSortItems;
+constexpr int64_t kDirectTiles = 32;
+
+int64_t sort_tiles(int64_t count) { return count > 0 ? (count + kSortTile - 1) / kSortTile : 1; }
+
+int64_t sort_scan_tiles(int64_t count) {
+    const int64_t tiles = sort_tiles(count);
+    return tiles <= kDirectTiles ? 0 : (256 * tiles + kScanTile - 1) / kScanTile;
+}
+
+__device__ __forceinline__ int64_t live_count(int64_t count, const u64 *dcount) {
+    return dcount && static_cast<int64_t>(*dcount) < count ? static_cast<int64_t>(*dcount) : count;
+}
+
+// Digit of (key, value): the key's bits from `shift` on and, with CROSS, the
+// value's lowest bits above them (vshift = the key's bits left of shift).
+template <bool CROSS>
+__device__ __forceinline__ uint32_t digit_of(uint32_t k, uint32_t v, int shift, int vshift, uint32_t mask) {
+    return (CROSS ? (k >> shift) | (v << vshift) : k >> shift) & mask;
+}
+
+// Digit counts of every tile: counts[digit * tiles + tile].
+template <bool CROSS>
+__global__ void __launch_bounds__(kSortBlock)
+k_sort_hist(int64_t count, const u64 *dcount, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
+            int shift, int vshift, uint32_t mask, uint32_t *counts, int64_t tiles) {
+    count = live_count(count, dcount);
+    __shared__ uint32_t s_h[kSortWarps][256];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortBlock) (&s_h[0][0])[d] = 0u;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)warp * (32 * kSortItems) + lane;
+    // all of a thread's keys in flight at once, then the counts
+    uint32_t k[kSortItems];
+#pragma unroll
+    for (int q = 0; q < kSortItems; q++) {
+        const int64_t idx = base + 32 * q;
+        k[q] = idx < count ? digit_of<CROSS>(__ldg(key + idx), CROSS ? __ldg(val + idx) : 0u, shift, vshift, mask) : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < kSortItems; q++)
+        if (base + 32 * q < count) atomicAdd(&s_h[warp][k[q]], 1u);
+    __syncthreads();
+    uint32_t c = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; w++) c += s_h[w][threadIdx.x];
+    counts[(int64_t)threadIdx.x * tiles + blockIdx.x] = c;
+}
+
+struct LoadCounts {
+    const uint32_t *p;
+    __device__ uint32_t operator()(int64_t i) const { return p[i]; }
+};
+struct StoreCountsExcl {
+    uint32_t *p;
+    __device__ void operator()(int64_t i, uint32_t exc, uint32_t) const { p[i] = exc; }
+};
+
+// Exclusive prefix of v over the block's 256 threads (s_wsum: scratch).
+__device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t *s_wsum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_wsum[warp] = x;
+    __syncthreads();
+    uint32_t before = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; w++) before += (w < warp) ? s_wsum[w] : 0u;
+    return before + x - v;
+}
+
+// Stable scatter of one tile.  Item order within a tile: warp w owns the w-th
+// slice of 32 * kSortItems items and walks it in rows of 32 lanes, so (warp,
+// row, lane) is index order.  Only the keys and their ranks stay in registers
+// (values are read when placed), which keeps four blocks resident per SM.
+// DIRECT: `offsets` holds the raw counts; otherwise offsets[digit * tiles +
+// tile] is where the tile's run of that digit starts.  VAL: values read from
+// vin, or the items' indices, or read and part of the digit.
+enum { kValRead = 0, kValIota = 1, kValCross = 2 };
+
+template <int BITS, bool DIRECT, int VAL>
+__global__ void __launch_bounds__(kSortBlock, 4)
+k_sort_scatter(int64_t count, const u64 *dcount, const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
+               uint32_t *__restrict__ kout, uint32_t *__restrict__ vout, int shift, int vshift,
+               const uint32_t *__restrict__ offsets, int64_t tiles) {
+    constexpr uint32_t kMask = (1u << BITS) - 1;
+    constexpr bool CROSS = VAL == kValCross;
+    count = live_count(count, dcount);
+    __shared__ uint32_t s_key[kSortTile];
+    __shared__ uint32_t s_val[kSortTile];
+    __shared__ uint32_t s_cnt[kSortWarps][256];  // per-warp counts, then per-warp bases
+    __shared__ uint32_t s_start[256];            // first tile-local slot of each digit
+    __shared__ uint32_t s_glob[256];             // global start of the tile's run of each digit
+    __shared__ uint32_t s_wsum[2 * kSortWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // positions within the tile are 32-bit; a tile past a run-time count is empty
+    const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
+    const int n_tile = static_cast<int>(count - tile0 < kSortTile ? count - tile0 : kSortTile);
+    if (n_tile <= 0) return;
+    kin += tile0;
+    if (VAL != kValIota) vin += tile0;
+    const int base = warp * (32 * kSortItems) + lane;
+    for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortBlock) (&s_cnt[0][0])[d] = 0u;
+    uint32_t k[kSortItems];
+#pragma unroll
+    for (int q = 0; q < kSortItems; q++) k[q] = base + 32 * q < n_tile ? __ldg(kin + base + 32 * q) : 0u;
+    if (DIRECT) {
+        const uint32_t *mine = offsets + (int64_t)threadIdx.x * tiles;
+        uint32_t before = 0, all = 0;
+        for (int i = 0; i < static_cast<int>(tiles); i++) {
+            const uint32_t c = __ldg(mine + i);
+            before += i < static_cast<int>(blockIdx.x) ? c : 0u;
+            all += c;
+        }
+        s_glob[threadIdx.x] = block_excl(all, s_wsum + kSortWarps) + before;
+    } else {
+        s_glob[threadIdx.x] = offsets[(int64_t)threadIdx.x * tiles + blockIdx.x];
+    }
+    __syncthreads();
+    // stable rank of every item among its warp's items of the same digit
+    // (below 32 * kSortItems, two to a register)
+    static_assert(32 * kSortItems <= 65536 && kSortItems % 2 == 0, "ranks packed in 16 bits");
+    uint32_t rank2[kSortItems / 2];
+#pragma unroll
+    for (int q = 0; q < kSortItems; q++) {
+        const bool ok = base + 32 * q < n_tile;
+        // (a crossing digit reads the value here and again when placing it)
+        const uint32_t d = digit_of<CROSS>(k[q], CROSS && ok ? __ldg(vin + base + 32 * q) : 0u, shift, vshift, kMask);
+        uint32_t peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+        for (int b = 0; b < BITS; b++) {
+            const bool bit = (d >> b) & 1u;
+            const uint32_t v = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? v : ~v;
+        }
+        const uint32_t before = s_cnt[warp][d];
+        const uint32_t r = before + __popc(peers & lanemask_lt());
+        if (q & 1) rank2[q / 2] |= r << 16;
+        else rank2[q / 2] = r;
+        __syncwarp();
+        if (ok && lane == __ffs(peers) - 1) s_cnt[warp][d] = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    // thread t = digit t: per-warp bases within the digit, then the digits'
+    // tile-local starts (a block scan of the digit totals)
+    {
+        const int d = threadIdx.x;
+        uint32_t run = 0;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; w++) {
+            const uint32_t c = s_cnt[w][d];
+            s_cnt[w][d] = run;
+            run += c;
+        }
+        s_start[d] = block_excl(run, s_wsum);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kSortItems; q++) {
+        if (base + 32 * q < n_tile) {
+            const uint32_t v = VAL == kValIota ? static_cast<uint32_t>(tile0) + base + 32 * q : __ldg(vin + base + 32 * q);
+            const uint32_t d = digit_of<CROSS>(k[q], v, shift, vshift, kMask);
+            const uint32_t p = s_start[d] + s_cnt[warp][d] + ((rank2[q / 2] >> (16 * (q & 1))) & 0xFFFFu);
+            s_key[p] = k[q];
+            s_val[p] = v;
+        }
+    }
+    __syncthreads();
+    for (int p = threadIdx.x; p < n_tile; p += kSortBlock) {
+        const uint32_t kk = s_key[p], vv = s_val[p];
+        const uint32_t d = digit_of<CROSS>(kk, vv, shift, vshift, kMask);
+        const uint32_t g = s_glob[d] + (p - s_start[d]);
+        kout[g] = kk;
+        vout[g] = vv;
+    }
+}
+
+template <int BITS, int VAL>
+static void launch_scatter(const SortPass &p, int64_t tiles, cudaStream_t s) {
+    const unsigned blocks = static_cast<unsigned>(tiles);
+    if (tiles <= kDirectTiles)
+        k_sort_scatter<BITS, true, VAL><<<blocks, kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, p.vin, p.kout, p.vout,
+                                                                      p.shift, p.vshift, p.counts, tiles);
+    else
+        k_sort_scatter<BITS, false, VAL><<<blocks, kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, p.vin, p.kout, p.vout,
+                                                                       p.shift, p.vshift, p.counts, tiles);
+}
+
+template <int BITS>
+static void launch_scatter(const SortPass &p, int64_t tiles, cudaStream_t s) {
+    if (p.vshift) launch_scatter<BITS, kValCross>(p, tiles, s);
+    else if (p.vin) launch_scatter<BITS, kValRead>(p, tiles, s);
+    else launch_scatter<BITS, kValIota>(p, tiles, s);
+}
+
+int sort_pass(const SortPass &p, const ScanState<uint32_t> &scan, cudaStream_t s) {
+    if (p.count <= 0) return PS_OK;
+    if (p.bits < 1 || p.bits > 8 || (p.vshift && !p.vin)) return PS_ERR_ARG;
+    const int64_t tiles = sort_tiles(p.count);
+    const int bits = (p.bits + 1) & ~1;  // the keys have no bits above the sort's last digit
+    const uint32_t mask = (1u << bits) - 1u;
+    if (p.vshift)
+        k_sort_hist<true><<<static_cast<unsigned>(tiles), kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, p.vin, p.shift,
+                                                                              p.vshift, mask, p.counts, tiles);
+    else
+        k_sort_hist<false><<<static_cast<unsigned>(tiles), kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, nullptr,
+                                                                               p.shift, 0, mask, p.counts, tiles);
+    PS_LAUNCH_CHECK();
+    if (tiles > kDirectTiles) {
+        k_scan<uint32_t, kScanBlock, kScanItems><<<static_cast<unsigned>(sort_scan_tiles(p.count)), kScanBlock, 0, s>>>(
+            256 * tiles, scan, 0u, OpSum(), LoadCounts{p.counts}, StoreCountsExcl{p.counts});
+        PS_LAUNCH_CHECK();
+    }
+    switch (bits) {  // ballots for the digit's own bits only
+        case 2: launch_scatter<2>(p, tiles, s); break;
+        case 4: launch_scatter<4>(p, tiles, s); break;
+        case 6: launch_scatter<6>(p, tiles, s); break;
+        default: launch_scatter<8>(p, tiles, s); break;
+    }
+    PS_LAUNCH_CHECK();
+    return PS_OK;
+}
+
+}  // namespace ps
