@@ -380,7 +380,7 @@ int ps_count_exact(const ps_graph *g, void *d_scratch, size_t scratch_bytes, ps_
  *
  * Computes d_pa[i] = d_a[0] + ... + d_a[i] and d_pb[i] = d_b[0] + ... + d_b[i]
  * exactly in uint64 for i < count (device arrays; outputs may not alias the
- * inputs).  The scan's scratch is a fixed array of about 2.3 MB inside the
+ * inputs).  The scan's scratch is a fixed array of about 2.1 MB inside the
  * library that every GPU using the library keeps until the process exits;
  * the call allocates and frees no device memory and calls no allocating
  * library routine.  The first call on each device does the set-up: it looks

@@ -170,8 +170,8 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     // the row offsets, the edge numbering and the edge table's prefixes
     const int64_t n_tiles = (n + kScanTile - 1) / kScanTile, m_tiles = (l.m_cap + kScanTile - 1) / kScanTile;
     const int64_t ns = sort_scan_tiles(n), es = sort_scan_tiles(l.m_cap);
-    l.scan_tiles = std::max(std::max(n_tiles, m_tiles), std::max(ns, es)) + 1;
-    l.scan_words = 4 * (scan_words(ns) + scan_words(es)) + 2 * scan_words(n_tiles) + scan_words(m_tiles);
+    l.scan_words = 4 * (scan_words<uint32_t>(ns) + scan_words<uint32_t>(es)) + 2 * scan_words<int64_t>(n_tiles) +
+                   scan_words<U64x2>(m_tiles);
 
     const size_t n1 = static_cast<size_t>(n > 0 ? n : 1);
     size_t p = 0;
@@ -181,7 +181,7 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
         return at;
     };
     l.status = take(ST_WORDS * sizeof(uint64_t));
-    l.scan_flag = take(static_cast<size_t>(l.scan_words) * sizeof(uint32_t));  // cleared together with the status
+    l.scan = take(static_cast<size_t>(l.scan_words) * sizeof(uint64_t));  // cleared together with the status
     l.off = take((n1 + 1) * sizeof(int64_t));
     l.col = take(static_cast<size_t>(nnz) * sizeof(int32_t));
     l.rank = take(n1 * sizeof(int32_t));
@@ -203,8 +203,6 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.vals0 = take(n1 * sizeof(uint32_t));
     l.vals1 = take(n1 * sizeof(uint32_t));
     l.counts = take(static_cast<size_t>(256) * std::max(sort_tiles(n), sort_tiles(l.m_cap)) * sizeof(uint32_t));
-    l.scan_agg = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(U64x2));
-    l.scan_inc = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(U64x2));
     l.total = p;
     *L = l;
     return true;
@@ -253,9 +251,10 @@ static void binomial_bar(uint64_t count, uint64_t k, double delta, double *pl, d
     *pu = 0.5 * (a + b);
 }
 
-// Runs the bounded wait of the scans on a flag that nothing sets.
-__global__ void k_wait_selftest(const uint32_t *flag, uint32_t limit, u64 *status) {
-    if (threadIdx.x == 0 && blockIdx.x == 0 && wait_flag(flag, limit) == 0u) raise_flag(status, F_TIMEOUT);
+// Runs the bounded wait of the scans on a slot that nothing sets.
+__global__ void k_wait_selftest(const u64 *slot, uint32_t limit, u64 *status) {
+    uint32_t v;
+    if (threadIdx.x == 0 && blockIdx.x == 0 && wait_slot(slot, v, limit) == 0u) raise_flag(status, F_TIMEOUT);
 }
 
 }  // namespace ps
@@ -268,10 +267,10 @@ int ps_selftest_bounded_wait(void *d_scratch, uint32_t spin_limit, ps_stream_t s
     if (!d_scratch || (reinterpret_cast<uintptr_t>(d_scratch) & 15u) != 0) return PS_ERR_ARG;
     if (spin_limit > kSpinLimit) spin_limit = kSpinLimit;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    uint32_t *flag = static_cast<uint32_t *>(d_scratch);
+    const u64 *slot = static_cast<const u64 *>(d_scratch);
     u64 *status = reinterpret_cast<u64 *>(static_cast<char *>(d_scratch) + 8);
     PS_CUDA_TRY(cudaMemsetAsync(d_scratch, 0, 16, s));
-    k_wait_selftest<<<1, 32, 0, s>>>(flag, spin_limit, status - ST_FLAGS);
+    k_wait_selftest<<<1, 32, 0, s>>>(slot, spin_limit, status - ST_FLAGS);
     PS_LAUNCH_CHECK();
     uint64_t flags = 0;
     PS_CUDA_TRY(cudaMemcpyAsync(&flags, status, sizeof(flags), cudaMemcpyDeviceToHost, s));

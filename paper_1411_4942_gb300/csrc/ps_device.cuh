@@ -56,7 +56,7 @@ enum {
     ST_HUBS = 9,
     ST_TIER = 10,      // 5 words: row boundaries of the sort tiers
     ST_LONG = 15,      // first row longer than kLongRow (its arcs are walked by a block)
-    ST_COUNTER = 16,   // 16 words: tile counters of scans (as uint32 pairs)
+    ST_COUNTER = 16,   // tile counter of the allocation-free scan
     ST_WORDS = 64
 };
 
@@ -75,19 +75,6 @@ __device__ __forceinline__ void raise_flag(u64 *status, u64 f) {
 
 // Bound on every device spin-wait (iterations with nanosleep back-off).
 constexpr uint32_t kSpinLimit = 1u << 24;
-
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p);
-
-// Waits until *flag is non-zero and returns it, or returns 0 after `limit`
-// polls (the caller then reports PS_ERR_TIMEOUT instead of hanging).
-__device__ __forceinline__ uint32_t wait_flag(const uint32_t *flag, uint32_t limit) {
-    uint32_t f = ld_acquire(flag);
-    for (uint32_t it = 0; f == 0u && it < limit; it++) {
-        __nanosleep(it < 64 ? 32 : 256);
-        f = ld_acquire(flag);
-    }
-    return f;
-}
 
 // ------------------------------------------------------------------ loads
 
@@ -156,15 +143,6 @@ __device__ __forceinline__ EdgeRec ldg_rec(const EdgeRec *p) {
         : "=r"(e.u), "=r"(e.v), "=r"(e.du), "=r"(e.dv), "=r"(e.iu), "=r"(e.jv), "=r"(e.ou), "=r"(e.ov)
         : "l"(p));
     return e;
-}
-
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release(uint32_t *p, uint32_t v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // ----------------------------------------------------------------- Philox

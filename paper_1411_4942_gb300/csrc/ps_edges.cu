@@ -242,7 +242,7 @@ __device__ __forceinline__ void edge_group(int64_t j0, int step, int64_t m, int6
 constexpr int kRecItems = 4;
 constexpr int kRecScanItems = 8;
 static_assert(kRecScanItems % kRecItems == 0, "whole groups per tile");
-static_assert(kScanBlock * kRecScanItems >= kScanTile, "the workspace holds scan flags per kScanTile items");
+static_assert(kScanBlock * kRecScanItems >= kScanTile, "the workspace holds scan slots per kScanTile items");
 
 // (Capped at 64 registers, four blocks per SM: while one block waits at the
 // tile's barriers or on its look-back, the others build records; the

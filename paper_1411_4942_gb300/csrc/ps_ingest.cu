@@ -38,8 +38,8 @@ int id_bits(int64_t n) {
 constexpr int kPairLists = 3;
 
 struct IngestLayout {
-    int64_t scan_tiles, scan_words;
-    size_t status, scan_flag, spans, clear_end, k[kPairLists], v[kPairLists], counts, scan_agg, scan_inc, total;
+    int64_t scan_words;
+    size_t status, scan, spans, clear_end, k[kPairLists], v[kPairLists], counts, total;
 };
 
 bool ingest_layout(int64_t n, int64_t n_edges, IngestLayout *L) {
@@ -47,9 +47,8 @@ bool ingest_layout(int64_t n, int64_t n_edges, IngestLayout *L) {
     IngestLayout l{};
     const int64_t n_tiles = (n + kScanTile - 1) / kScanTile, e_tiles = (n_edges + kScanTile - 1) / kScanTile;
     const int64_t es = sort_scan_tiles(n_edges);
-    l.scan_tiles = std::max(std::max(n_tiles, e_tiles), es) + 1;
     // up to 8 passes by (lo, hi) and 4 by hi, the compaction and the offsets
-    l.scan_words = 12 * scan_words(es) + scan_words(e_tiles) + scan_words(n_tiles);
+    l.scan_words = 12 * scan_words<uint32_t>(es) + scan_words<uint32_t>(e_tiles) + scan_words<int64_t>(n_tiles);
     const size_t e1 = static_cast<size_t>(n_edges > 0 ? n_edges : 1), n1 = static_cast<size_t>(n > 0 ? n : 1);
     size_t p = 0;
     auto take = [&](size_t bytes) {
@@ -58,7 +57,7 @@ bool ingest_layout(int64_t n, int64_t n_edges, IngestLayout *L) {
         return at;
     };
     l.status = take(IS_WORDS * sizeof(uint64_t));
-    l.scan_flag = take(static_cast<size_t>(l.scan_words) * sizeof(uint32_t));
+    l.scan = take(static_cast<size_t>(l.scan_words) * sizeof(uint64_t));
     l.spans = take(2 * n1 * sizeof(int2));
     l.clear_end = p;
     for (int i = 0; i < kPairLists; i++) {
@@ -66,8 +65,6 @@ bool ingest_layout(int64_t n, int64_t n_edges, IngestLayout *L) {
         l.v[i] = take(e1 * sizeof(uint32_t));
     }
     l.counts = take(static_cast<size_t>(256) * sort_tiles(n_edges) * sizeof(uint32_t));
-    l.scan_agg = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(int64_t));
-    l.scan_inc = take(static_cast<size_t>(l.scan_tiles + 1) * sizeof(int64_t));
     l.total = p;
     *L = l;
     return true;
@@ -171,17 +168,12 @@ k_ingest_columns(const u64 *__restrict__ pairs, const uint32_t *__restrict__ bhi
     }
 }
 
-// Takes a scan's counter and flags from the cleared region.
+// Takes a scan's counter and slots from the cleared region.
 template <typename T>
 ScanState<T> ingest_scan_state(char *ws, const IngestLayout &L, int64_t tiles, int64_t *used) {
-    ScanState<T> s;
-    s.counter = reinterpret_cast<uint32_t *>(ws + L.scan_flag) + *used;
-    s.flag = s.counter + 1;
-    s.agg = reinterpret_cast<T *>(ws + L.scan_agg);
-    s.inc = reinterpret_cast<T *>(ws + L.scan_inc);
-    s.status = reinterpret_cast<u64 *>(ws + L.status) + IS_FLAGS;
-    *used += scan_words(tiles);
-    return s;
+    u64 *at = reinterpret_cast<u64 *>(ws + L.scan) + *used;
+    *used += scan_words<T>(tiles);
+    return ScanState<T>{at + 2, reinterpret_cast<uint32_t *>(at), reinterpret_cast<u64 *>(ws + L.status) + IS_FLAGS};
 }
 
 }  // namespace
@@ -216,7 +208,7 @@ extern "C" int ps_csr_from_edges(int64_t n, int64_t n_edges, const int32_t *d_sr
     uint32_t *counts = reinterpret_cast<uint32_t *>(ws + L.counts);
     const int sms = sm_count_of_current_device();
     int64_t used = 0;
-    // the status words, the scans' counters and flags, and the rows' spans
+    // the status words, the scans' counters and slots, and the rows' spans
     PS_CUDA_TRY(cudaMemsetAsync(ws, 0, L.clear_end, s));
     if (n_edges > 0) {
         auto blocks = [&](int64_t items) { return static_cast<unsigned>(std::min<int64_t>((items + 255) / 256, (int64_t)sms * 16)); };

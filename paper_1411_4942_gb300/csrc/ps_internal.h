@@ -43,12 +43,12 @@ struct Tuning {
 };
 Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz);
 struct Layout {
-    int64_t n, nnz, m_cap, gcap, hub_cap, hub_words, hub_bit_base, scan_tiles;
-    int64_t scan_words;    // zeroed words of one load's scans (tile counters and flags)
+    int64_t n, nnz, m_cap, gcap, hub_cap, hub_words, hub_bit_base;
+    int64_t scan_words;    // 64-bit words of one load's scans (tile counters and slots)
     int64_t filt_words;    // 32-bit words of the edge filter; 0 without it
     int64_t vtab_slots;    // 0 without the per-vertex tables
     size_t status, off, col, rank, lowcnt, ubase, dnew, rec, ptau, plam, gtau, glam, hub, filt, vtab;
-    size_t keys0, keys1, vals0, vals1, counts, scan_flag, scan_agg, scan_inc;
+    size_t keys0, keys1, vals0, vals1, counts, scan;
     size_t total;
 };
 bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L);
@@ -135,18 +135,17 @@ int64_t sort_tiles(int64_t count);
 int64_t sort_scan_tiles(int64_t count);
 int sort_pass(const SortPass &p, const ScanState<uint32_t> &scan, cudaStream_t s);
 
-// The scans of a load share the workspace's value arrays (one scan at a time
-// per graph, in stream order) and take their tile counter and flags from a
-// region that the load clears once.
-inline int64_t scan_words(int64_t tiles) { return (tiles + 2 + 3) & ~int64_t{3}; }
+// The scans of a load take their tile counter and slots from a region of
+// 64-bit words that the load clears once.
+template <typename T>
+inline int64_t scan_words(int64_t tiles) { return 2 + ((SlotOf<T>::kWords * tiles + 1) & ~int64_t{1}); }
 template <typename T>
 inline int take_scan(ps_graph *g, int64_t tiles, ScanState<T> *st) {
-    const int64_t words = scan_words(tiles);
-    if (tiles > g->L.scan_tiles || g->scan_used + words > g->L.scan_words) return PS_ERR_WORKSPACE;
-    st->counter = reinterpret_cast<uint32_t *>(g->ws + g->L.scan_flag) + g->scan_used;
-    st->flag = st->counter + 1;
-    st->agg = reinterpret_cast<T *>(g->ws + g->L.scan_agg);
-    st->inc = reinterpret_cast<T *>(g->ws + g->L.scan_inc);
+    const int64_t words = scan_words<T>(tiles);
+    if (g->scan_used + words > g->L.scan_words) return PS_ERR_WORKSPACE;
+    u64 *at = reinterpret_cast<u64 *>(g->ws + g->L.scan) + g->scan_used;
+    st->counter = reinterpret_cast<uint32_t *>(at);
+    st->slots = at + 2;
     st->status = g->status;
     g->scan_used += words;
     return PS_OK;

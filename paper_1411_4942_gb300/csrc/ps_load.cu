@@ -734,10 +734,10 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     const int64_t n = L.n, nnz = L.nnz;
     char *ws = g->ws;
     const int sms = g->sm_count;
-    // the status words and, right behind them, the counters and flags of every
+    // the status words and, right behind them, the counters and slots of every
     // scan of this load
     g->scan_used = 0;
-    PS_CUDA_TRY(cudaMemsetAsync(g->status, 0, L.scan_flag - L.status + sizeof(uint32_t) * L.scan_words, s));
+    PS_CUDA_TRY(cudaMemsetAsync(g->status, 0, L.scan - L.status + sizeof(uint64_t) * L.scan_words, s));
     uint32_t *k0 = reinterpret_cast<uint32_t *>(ws + L.keys0);
     uint32_t *k1 = reinterpret_cast<uint32_t *>(ws + L.keys1);
     uint32_t *v0 = reinterpret_cast<uint32_t *>(ws + L.vals0);

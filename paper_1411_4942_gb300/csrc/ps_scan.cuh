@@ -96,27 +96,106 @@ __device__ __forceinline__ void add_stars(uint64_t &lo, uint64_t &hi, uint64_t d
 
 // ------------------------------------------------ decoupled look-back scan
 
-// Tile status for the single-pass scan of Merrill & Garland (2016): a flag
-// per tile (0 = empty, 1 = aggregate ready, 2 = inclusive prefix ready) and
-// the two values.  `counter` hands out tile ids in launch order, so a block
-// only ever waits on tiles already owned by running blocks.
+// Tile status for the single-pass scan of Merrill & Garland (2016): one slot
+// per tile with its aggregate (state 1), then its inclusive prefix (state 2).
+// Every 64-bit word of a slot carries the state and 32 bits of the value, so a
+// word is complete by itself and no fence orders a flag against a value: a
+// fence waits for all of the thread's earlier stores, and the edge-table
+// kernel's threads have their records and filter bits in flight.  A reader
+// takes a slot whose words all carry the same state.  `counter` hands out
+// tile ids in launch order, so a block only ever waits on tiles already
+// owned by running blocks.  Slots and counter start at zero.
 template <typename T>
 struct ScanState {
-    uint32_t *flag;
-    T *agg;
-    T *inc;
+    u64 *slots;
     uint32_t *counter;
     u64 *status;
 };
 
 template <typename T>
-__device__ __forceinline__ T ld_cg(const T *p) {
-    return *reinterpret_cast<const volatile T *>(p);
-}
+struct SlotOf;
 template <>
-__device__ __forceinline__ U64x2 ld_cg<U64x2>(const U64x2 *p) {
-    const volatile uint64_t *q = reinterpret_cast<const volatile uint64_t *>(p);
-    return U64x2{q[0], q[1]};
+struct SlotOf<uint32_t> {
+    static constexpr int kWords = 1;
+    static __device__ __forceinline__ void split(uint32_t v, uint32_t (&h)[1]) { h[0] = v; }
+    static __device__ __forceinline__ uint32_t join(const uint32_t (&h)[1]) { return h[0]; }
+};
+template <>
+struct SlotOf<int64_t> {
+    static constexpr int kWords = 2;
+    static __device__ __forceinline__ void split(int64_t v, uint32_t (&h)[2]) {
+        h[0] = static_cast<uint32_t>(v);
+        h[1] = static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32);
+    }
+    static __device__ __forceinline__ int64_t join(const uint32_t (&h)[2]) {
+        return static_cast<int64_t>((static_cast<uint64_t>(h[1]) << 32) | h[0]);
+    }
+};
+template <>
+struct SlotOf<U64x2> {
+    static constexpr int kWords = 4;
+    static __device__ __forceinline__ void split(U64x2 v, uint32_t (&h)[4]) {
+        h[0] = static_cast<uint32_t>(v.a);
+        h[1] = static_cast<uint32_t>(v.a >> 32);
+        h[2] = static_cast<uint32_t>(v.b);
+        h[3] = static_cast<uint32_t>(v.b >> 32);
+    }
+    static __device__ __forceinline__ U64x2 join(const uint32_t (&h)[4]) {
+        return U64x2{(static_cast<uint64_t>(h[1]) << 32) | h[0], (static_cast<uint64_t>(h[3]) << 32) | h[2]};
+    }
+};
+
+template <typename T>
+__device__ __forceinline__ void publish_slot(u64 *slot, T v, uint32_t state) {
+    constexpr int N = SlotOf<T>::kWords;
+    uint32_t h[N];
+    SlotOf<T>::split(v, h);
+    u64 w[N];
+#pragma unroll
+    for (int i = 0; i < N; i++) w[i] = (static_cast<u64>(state) << 32) | h[i];
+    if (N == 1) {
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(slot), "l"(w[0]) : "memory");
+    } else {
+#pragma unroll
+        for (int i = 0; i + 1 < N; i += 2)
+            asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(slot + i), "l"(w[i]), "l"(w[i + 1]) : "memory");
+    }
+}
+
+// The slot's state (0: nothing yet) and, unless 0, its value.
+template <typename T>
+__device__ __forceinline__ uint32_t read_slot(const u64 *slot, T &v) {
+    constexpr int N = SlotOf<T>::kWords;
+    u64 w[N];
+    if (N == 1) {
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w[0]) : "l"(slot) : "memory");
+    } else {
+#pragma unroll
+        for (int i = 0; i + 1 < N; i += 2)
+            asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[i]), "=l"(w[i + 1]) : "l"(slot + i) : "memory");
+    }
+    uint32_t h[N];
+    const uint32_t state = static_cast<uint32_t>(w[0] >> 32);
+    bool same = true;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        h[i] = static_cast<uint32_t>(w[i]);
+        same = same && static_cast<uint32_t>(w[i] >> 32) == state;
+    }
+    v = SlotOf<T>::join(h);
+    return same ? state : 0u;
+}
+
+// Waits until the slot holds something, or returns 0 after `limit` polls (the
+// caller then reports PS_ERR_TIMEOUT instead of hanging).
+template <typename T>
+__device__ __forceinline__ uint32_t wait_slot(const u64 *slot, T &v, uint32_t limit) {
+    uint32_t state = read_slot(slot, v);
+    for (uint32_t it = 0; state == 0u && it < limit; it++) {
+        __nanosleep(it < 64 ? 32 : 256);
+        state = read_slot(slot, v);
+    }
+    return state;
 }
 
 // A tile is BLOCK * ITEMS consecutive items; warp w owns the w-th run of
@@ -177,18 +256,11 @@ __device__ __forceinline__ void scan_tile(int64_t tile, int64_t wbase, T (&v)[IT
 
     if (warp == 0) {
         T excl = identity;
+        constexpr int N = SlotOf<T>::kWords;
         if (tile == 0) {
-            if (lane == 0) {
-                st.inc[0] = tile_agg;
-                __threadfence();
-                st_release(st.flag, 2u);
-            }
+            if (lane == 0) publish_slot(st.slots, tile_agg, 2u);
         } else {
-            if (lane == 0) {
-                st.agg[tile] = tile_agg;
-                __threadfence();
-                st_release(st.flag + tile, 1u);
-            }
+            if (lane == 0) publish_slot(st.slots + N * tile, tile_agg, 1u);
             int64_t pred = tile - 1;
             bool timed_out = false;
             while (true) {
@@ -196,12 +268,11 @@ __device__ __forceinline__ void scan_tile(int64_t tile, int64_t wbase, T (&v)[IT
                 uint32_t f = 2u;
                 T val = identity;
                 if (p >= 0) {
-                    f = wait_flag(st.flag + p, kSpinLimit);
+                    f = wait_slot(st.slots + N * p, val, kSpinLimit);
                     if (f == 0u) {
                         timed_out = true;
                         f = 2u;
-                    } else {
-                        val = (f == 2u) ? ld_cg(st.inc + p) : ld_cg(st.agg + p);
+                        val = identity;
                     }
                 }
                 const uint32_t incmask = __ballot_sync(0xffffffffu, f == 2u);
@@ -215,11 +286,7 @@ __device__ __forceinline__ void scan_tile(int64_t tile, int64_t wbase, T (&v)[IT
                 pred -= 32;
             }
             if (__any_sync(0xffffffffu, timed_out) && lane == 0) raise_flag(st.status, F_TIMEOUT);
-            if (lane == 0) {
-                st.inc[tile] = op(excl, tile_agg);
-                __threadfence();
-                st_release(st.flag + tile, 2u);
-            }
+            if (lane == 0) publish_slot(st.slots + N * tile, op(excl, tile_agg), 2u);
         }
         if (lane == 0) s_excl = excl;
     }

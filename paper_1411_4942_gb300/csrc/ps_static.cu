@@ -1,7 +1,7 @@
 // ps_static.cu -- ps_prefix_pairs_static: the exact uint64 prefix scan of
 // two weight arrays (the same single-pass scan that builds the tau / lambda
 // prefixes) for callers that cannot allocate device memory.  Its scratch --
-// the scan's tile flags, tile sums and tile counter -- lives in one
+// the scan's tile slots and tile counter -- lives in one
 // fixed-size array in this file instead of a caller's workspace.
 #include <cuda.h>
 
@@ -15,12 +15,8 @@ namespace {
 constexpr int64_t kStaticMaxItems = PS_PREFIX_STATIC_MAX_ITEMS;
 constexpr int64_t kStaticTiles = (kStaticMaxItems + kScanTile - 1) / kScanTile;
 constexpr size_t kStatusBytes = ST_WORDS * sizeof(uint64_t);
-constexpr size_t kFlagBytes = ((kStaticTiles + 1) * sizeof(uint32_t) + 255) / 256 * 256;
-constexpr size_t kSumBytes = (kStaticTiles + 1) * sizeof(U64x2);
-constexpr size_t kOffFlags = kStatusBytes;
-constexpr size_t kOffAgg = kOffFlags + kFlagBytes;
-constexpr size_t kOffInc = kOffAgg + kSumBytes;
-constexpr size_t kScratchBytes = kOffInc + kSumBytes;  // about 2.3 MB
+constexpr size_t kOffSlots = kStatusBytes;
+constexpr size_t kScratchBytes = kOffSlots + kStaticTiles * SlotOf<U64x2>::kWords * sizeof(u64);  // about 2.1 MB
 
 // Every GPU that loads the library holds this array until the process exits.
 static __device__ __align__(256) unsigned char g_prefix_scratch[kScratchBytes];
@@ -119,15 +115,12 @@ extern "C" int ps_prefix_pairs_static(const uint64_t *d_a, const uint64_t *d_b, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int64_t tiles = (count + kScanTile - 1) / kScanTile;
     // the array keeps the previous call's contents: clear the status words,
-    // the tile counter and the flags this call will use
-    PS_CUDA_TRY(cudaMemsetAsync(p, 0, kStatusBytes, s));
-    PS_CUDA_TRY(cudaMemsetAsync(p + kOffFlags, 0, sizeof(uint32_t) * (tiles + 1), s));
+    // the tile counter and, right behind them, the slots this call will use
+    PS_CUDA_TRY(cudaMemsetAsync(p, 0, kOffSlots + tiles * SlotOf<U64x2>::kWords * sizeof(u64), s));
     ScanState<U64x2> st;
     st.status = reinterpret_cast<u64 *>(p);
     st.counter = reinterpret_cast<uint32_t *>(st.status + ST_COUNTER);
-    st.flag = reinterpret_cast<uint32_t *>(p + kOffFlags);
-    st.agg = reinterpret_cast<U64x2 *>(p + kOffAgg);
-    st.inc = reinterpret_cast<U64x2 *>(p + kOffInc);
+    st.slots = reinterpret_cast<u64 *>(p + kOffSlots);
     k_scan<U64x2, kScanBlock, kScanItems><<<(unsigned)tiles, kScanBlock, 0, s>>>(
         count, st, U64x2{0, 0}, OpSum(), LoadPairs{d_a, d_b}, StorePairs{d_pa, d_pb, st.status});
     PS_LAUNCH_CHECK();
