@@ -74,6 +74,8 @@ __device__ __forceinline__ void batch_sample2_hash(const GraphDev &g, int sample
     }
 }
 
+constexpr int kAheadItems = 4;
+
 // ADJ = 0: any variant, chosen per item; otherwise the table's only variant.
 // counter[0] hands out items; counter[1] counts items skipped because their
 // graph does not use the variant this kernel was compiled for.  Registers
@@ -84,33 +86,60 @@ template <int BLOCK, int ADJ, int SPT>
 __global__ void __launch_bounds__(BLOCK, (SPT == 1 ? 1024 : 512) / BLOCK)
 k_batch(const GraphDev *__restrict__ table, int32_t n_graphs, const ps_work *__restrict__ items,
         int64_t n_items, uint64_t *hist, uint32_t *counter) {
-    __shared__ int64_t s_item;
+    // The next item is copied, and the one after it claimed, while this one
+    // runs, so a block does not stand still for the queue's three round trips
+    // (claim, item, graph); items come grouped by graph, so the graph is mostly
+    // in place: 96 R-MAT graphs, 4096-sample items, 6.29 -> 5.29 ms.  Only
+    // while kAheadItems items per block are left: near the end of the queue a
+    // claimed item would wait for its block while others idle (200 served
+    // requests in items of 65536 samples took 12.4 ms claiming ahead to the
+    // end, 11.0 ms so).
+    __shared__ ps_work s_w[2];
+    __shared__ uint32_t s_item[2];
     __shared__ GraphDev s_g;
-    __shared__ ps_work s_w;
-    while (true) {
+    static_assert(sizeof(ps_work) == 32 && sizeof(GraphDev) % 4 == 0, "copied by words");
+    constexpr uint32_t kNone = ~0u;
+    const int64_t ahead_end = n_items - static_cast<int64_t>(kAheadItems) * gridDim.x;
+    uint32_t claim = kNone;  // thread 0: the item after the current one
+    if (threadIdx.x == 0) {
+        const uint32_t it = atomicAdd(counter, 1u);
+        if (it < ahead_end) claim = atomicAdd(counter, 1u);
+        s_item[0] = it;
+        if (it < n_items) s_w[0] = items[it];
+    }
+    __syncthreads();
+    uint32_t graph = kNone;  // of s_g
+    for (int at = 0; s_item[at] < n_items; at ^= 1) {
         if (threadIdx.x == 0) {
-            const int64_t it = static_cast<int64_t>(atomicAdd(counter, 1u));
-            s_item = it;
-            if (it < n_items) {
-                s_w = items[it];
-                if (s_w.graph < static_cast<uint32_t>(n_graphs)) {
-                    s_g = table[s_w.graph];
-                    if (ADJ != 0 && s_g.adj_mode != ADJ) {
-                        s_w.count = 0;
-                        atomicAdd(counter + 1, 1u);
-                    }
-                } else {
-                    s_w.count = 0;  // item names no graph: skipped
-                }
+            s_item[at ^ 1] = claim;
+            if (claim < n_items) {
+                const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&s_w[at ^ 1]));
+                const char *src = reinterpret_cast<const char *>(items + claim);  // 8-byte aligned
+#pragma unroll
+                for (int i = 0; i < 32; i += 8)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + i), "l"(src + i) : "memory");
+                claim = claim < ahead_end ? atomicAdd(counter, 1u) : kNone;
             }
         }
-        __syncthreads();
-        if (s_item >= n_items) break;
-        const ps_work w = s_w;
+        const ps_work w = s_w[at];
+        if (w.graph != graph) {
+            // (an item that names no graph leaves an empty one: nothing to sample)
+            graph = w.graph;
+            if (graph < static_cast<uint32_t>(n_graphs)) {
+                for (int i = threadIdx.x; i < static_cast<int>(sizeof(GraphDev) / 4); i += BLOCK)
+                    reinterpret_cast<uint32_t *>(&s_g)[i] = __ldg(reinterpret_cast<const uint32_t *>(table + graph) + i);
+            } else if (threadIdx.x == 0) {
+                s_g.W = s_g.Lambda = 0;
+                s_g.adj_mode = ADJ;
+            }
+            __syncthreads();
+        }
+        const bool skip = ADJ != 0 && s_g.adj_mode != ADJ;
+        if (skip && threadIdx.x == 0) atomicAdd(counter + 1, 1u);
         Counts6 cnt;
         cnt.zero();
         const int sampler = static_cast<int>(w.sampler);
-        const bool any = sampler == 0 ? s_g.W > 0 : s_g.Lambda > 0;
+        const bool any = !skip && (sampler == 0 ? s_g.W > 0 : s_g.Lambda > 0);
         if (any && SPT == 2 && (ADJ == kAdjHash || (ADJ == 0 && s_g.adj_mode == kAdjHash))) {
             for (uint32_t s = threadIdx.x; s < w.count; s += 2 * BLOCK) {
                 // a lone last sample repeats its own id as the second, whose class is dropped
@@ -132,6 +161,16 @@ k_batch(const GraphDev *__restrict__ table, int32_t n_graphs, const ps_work *__r
                 }
             }
         }
+        if (threadIdx.x == 0) {
+            if (s_item[at ^ 1] == kNone) {
+                const uint32_t it = atomicAdd(counter, 1u);
+                s_item[at ^ 1] = it;
+                if (it < n_items) s_w[at ^ 1] = items[it];
+            } else {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+            }
+        }
+        // its barriers also publish the next item and free this one and s_g
         flush_counts<BLOCK>(cnt, sampler == 0 ? 6 : 4, hist + 6ull * w.slot);
     }
 }

@@ -168,7 +168,8 @@ struct Counts6 {
 };
 
 // Block-wide sum of the counters, added to hist[0..nbins) with one atomic per
-// bin per block.
+// bin per block.  The warp sums take two reductions of 16-bit halves each (a
+// counter may hold up to 2^30, a warp's sum more than 32 bits).
 template <int BLOCK>
 __device__ __forceinline__ void flush_counts(Counts6 &cnt, int nbins, uint64_t *hist) {
     __shared__ unsigned long long s_bins[6];
@@ -176,9 +177,9 @@ __device__ __forceinline__ void flush_counts(Counts6 &cnt, int nbins, uint64_t *
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 6; i++) {
-        unsigned long long x = cnt.c[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        const uint32_t lo = __reduce_add_sync(0xffffffffu, cnt.c[i] & 0xffffu);
+        const uint32_t hi = __reduce_add_sync(0xffffffffu, cnt.c[i] >> 16);
+        const unsigned long long x = (static_cast<unsigned long long>(hi) << 16) + lo;
         if ((threadIdx.x & 31) == 0 && x) atomicAdd(&s_bins[i], x);
     }
     __syncthreads();
