@@ -872,13 +872,13 @@ def main():
                     help="samples per chunk of the draw-ordered samplers (0: all of a call's "
                          f"samples, up to {MAX_ORDER_CHUNK})")
     ap.add_argument("--adjacency", type=int, default=0,
-                    help="adjacency test: 0 default (hash set), 1 hash set, 2 search + hub rows, "
+                    help="adjacency test: 0 default (edge filter), 1 edge filter, 2 search + hub rows, "
                          "3 per-vertex tables")
     ap.add_argument("--hub-count", type=int, default=0, help="hub bitmap rows (0 default, -1 none)")
     ap.add_argument("--hub-span", type=int, default=0, help="hub rows cover the top 2^k labels (0 default, -1 all)")
     ap.add_argument("--draw-order", type=int, default=0,
-                    help="draw-ordered samplers: 0 by size (default), 1 one pass (256 ranges of r), "
-                         "2 two passes (65536 ranges), -1 id order")
+                    help="draw-ordered samplers: 0 by size (default), 1 or 2 always sorted, "
+                         "-1 id order")
     ap.add_argument("--oracle-protocol", action="store_true",
                     help="time the oracle alone (prepare and samplers separately, one core and all "
                          "cores) on --workload and print its JSON line")

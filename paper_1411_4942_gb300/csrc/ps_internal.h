@@ -39,7 +39,7 @@ struct Tuning {
     int hub_min_degree;
     int hub_span_log2;     // hub rows cover the top 2^span labels; 0: all labels
     int adj_mode;          // kAdjHash or kAdjSearch
-    int draw_order;        // ordered samplers: 0 by size, 1 always, -1 never
+    int draw_order;        // ordered samplers: 0 by size, > 0 always, -1 never
 };
 Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz);
 struct Layout {

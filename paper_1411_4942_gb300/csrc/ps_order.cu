@@ -6,270 +6,296 @@
 // histograms are sums, so the order in which ids are classified changes no
 // count.  In id order, consecutive samples draw unrelated edges: the guide
 // entry, the prefix probe, the edge record and the row N(u) of every sample
-// are separate random reads of HBM.  Here the ids of a chunk are first
-// counting-sorted by r >> shift into kOrderBuckets equal-width ranges of
-// [0, W) (or [0, Lambda)); the sampling grid then walks the sorted ids, so the
-// samples in flight at any time draw from a narrow band of consecutive edges
-// and those reads mostly hit L1 and L2.  Only the second endpoint's row and
-// the adjacency tests stay random.
+// are separate random reads of HBM.  Here the ids of a chunk are first sorted
+// by the leading bits of the 64-bit word their edge draw is made from (r grows
+// with it); the sampling grid then walks the sorted ids, so the samples in
+// flight at any time draw from a narrow band of consecutive edges, the samples
+// of a warp mostly from a few edges, and those reads hit L1 and L2 or are one
+// read for several lanes.  Only the second endpoint's row and the adjacency
+// tests stay random.
+//
+// The sort is two kernels.  The word is uniform, so equal-width ranges of it
+// hold nearly equal numbers of ids: the first kernel draws each id's word once
+// and puts the ids into up to kOrderBuckets buckets of a fixed capacity (8
+// standard deviations above the mean), reserving room tile by tile, with no
+// counting pass before it.  The second sorts every bucket by the next
+// 11 or 12 bits in one block's shared memory and writes the ids out densely.
+// Should a bucket ever run over, the sampling kernel takes the ids in their
+// own order instead.
+//
+// The finer the order, the more the lanes of a warp share: on the 3M-vertex
+// graph (115M edges, 2^27 ids) the 3-path sampling kernel took 10.6 / 9.4 / 8.5
+// / 7.9 / 7.8 ms with the ids in order of 12 / 16 / 20 / 24 / 32 bits; on R-MAT
+// 20 (2^24 ids) 710 / 568 / 527 / 522 us with 8 / 16 / 20 / 24.  This sort
+// gives 24 and 21 bits; a sort by 16 bits in two passes of counting,
+// offsets and scatter took 1.91 ms on the former, this one 1.70.
 #include "ps_internal.h"
 #include "ps_sample.cuh"
 
 namespace ps {
 
-// kOrderBuckets equal-width ranges of r; a chunk of ids is split into at
-// most kOrderMaxRuns contiguous runs, one per block of the counting sort.
-// On R-MAT 20 with 2^24 samples, finer orders made the 3-path sampling
-// kernel faster (1.08 ms at 256 buckets, 0.96 ms at 65536 through a second
-// pass, 0.94 ms with global atomics) but cost more to sort than they saved.
-constexpr int kOrderBuckets = 256;
-constexpr int kOrderMaxRuns = 1024;
-constexpr int kOrderThreads = 512;
-constexpr int kOrderWarps = kOrderThreads / 32;
-constexpr int kOrderItems = 8;                            // ids per scatter thread and tile
-constexpr int kOrderTile = kOrderItems * kOrderThreads;   // ids a scatter block sorts in shared memory at once
-// hist[b * kOrderMaxRuns + run]: run counts, then offsets; then the bucket totals
-constexpr size_t kOrderHist = static_cast<size_t>(kOrderMaxRuns) * kOrderBuckets * sizeof(uint32_t);
-constexpr size_t kOrderHeader = kOrderHist + kOrderBuckets * sizeof(uint32_t);
-// after the header, per sample of a chunk: the sorted order (uint32 id
-// offsets from the chunk's first id), then each id's bucket (uint8)
-// By default (tuning draw_order 0) chunks below kOrderMinChunk samples, and
-// graphs below kOrderMinEdges edges (whose records and rows mostly stay in
-// L2 anyway), take the plain sampler: there the sort costs more than it
-// saves.  The counts are the same either way.
-constexpr uint64_t kOrderMinChunk = 1ull << 18;
-constexpr int64_t kOrderMinEdges = 1ll << 20;
-// From this many edges the default sorts by 16 bits of r in two passes: a
-// 256th of r then spans too many edges for their records and rows to be
-// read again before L2 drops them.  Measured (one box, both samplers):
-// 3M-vertex graph, 116.6M edges, 14.75 / 5.47 -> 14.22 / 5.16 ms with the
-// sorts; R-MAT 20, 15.7M edges, 1.22 / 0.87 -> 1.23 / 0.96 ms.
-constexpr int64_t kOrderTwoPassEdges = 1ll << 25;
+constexpr int kOrderBuckets = 4096;              // of the first kernel, at most
+// Buckets of the second kernel: a block of 1024 with 34 ids per thread for
+// means of 2^14 to 2^15 ids, or, for chunks that would leave SMs without a
+// bucket, a block of 512 with 18 per thread for means of 2^12 to 2^13.
+constexpr int kLargeThreads = 1024, kLargeItems = 34, kLargeMeanBits = 15;
+constexpr int kSmallThreads = 512, kSmallItems = 18, kSmallMeanBits = 13;
+constexpr uint64_t kLargeFrom = 1u << 22;        // ids per chunk
+constexpr uint64_t kOrderMaxSorted = static_cast<uint64_t>(kOrderBuckets) << kLargeMeanBits;  // ids sorted at once
+constexpr int kOrderItems = 16;                  // ids per thread and tile of the first kernel
+constexpr int kCursorStride = 8;                 // cursors in sectors of their own
+// Scratch: the cursors and the overflow flag in a header, then per sample of a
+// chunk its id (uint32) in the final order, and per place of the buckets an id
+// (uint32) and its key's next bits (uint16): at most 10.9 bytes per sample.
+constexpr size_t kOrderHeader = (1u << 20) + 1024;
+constexpr size_t kOrderPerSample = 11;
+static_assert((kOrderBuckets * kCursorStride + 1) * sizeof(uint32_t) <= kOrderHeader, "cursors and flag");
+// By default (tuning draw_order 0) small graphs, whose records and rows stay
+// in L2 anyway, and short chunks take the plain sampler: there the sort costs
+// more than it saves.  The counts are the same either way.  Measured, ordered
+// against plain, 3-path / centred (Chung-Lu; R-MAT crosses a little earlier):
+//   2.5M edges: 2^23 ids 285 / 272 against 287 / 266 us;
+//   5M edges: 2^21 ids 121 / 115 against 113 / 107, 2^22 184 / 174 against 204 / 192;
+//   10M edges: 2^20 ids 92 / 93 against 80 / 79, 2^21 138 / 138 against 143 / 137;
+//   40M edges: 2^20 ids 120 / 117 against 116 / 113, 2^24 971 / 777 against 1493 / 1506.
+constexpr int64_t kOrderMinEdges = 1ll << 22;
+static uint64_t order_min_chunk(int64_t m) { return m >= (1ll << 23) ? 1ull << 21 : 1ull << 22; }
 
-// The edge draw r of sample id, exactly as the samplers take it.
-template <int SAMPLER>
-__device__ __forceinline__ uint64_t draw_r_of(uint64_t total, uint64_t seed, uint64_t id) {
-    const uint4 w = sample_block(seed, id, 0, SAMPLER);
-    uint64_t r;
-    if (!lemire64((static_cast<uint64_t>(w.y) << 32) | w.x, total, r)) r = draw_r_retry(seed, id, SAMPLER, total);
-    return r;
+// Buckets for kk ids (a power of two) and the room of each: the whole chunk
+// in one bucket, or 8 standard deviations above the mean.
+struct OrderPlan {
+    int bits;          // log2 of the buckets
+    uint32_t room;     // ids per bucket
+    bool large;        // which second kernel
+};
+static OrderPlan order_plan(uint64_t kk) {
+    OrderPlan p{0, static_cast<uint32_t>(kk), kk >= kLargeFrom};
+    const int mean_bits = p.large ? kLargeMeanBits : kSmallMeanBits;
+    while (((kk - 1) >> mean_bits) >> p.bits) p.bits++;
+    if (p.bits) {
+        const uint32_t mean = static_cast<uint32_t>((kk >> p.bits) + 1);
+        uint32_t root = 1;
+        while (root * root < mean) root++;
+        p.room = mean + 8 * root + 64;
+    }
+    return p;
 }
 
-// Bucket of every id of block b's run [b * per, (b + 1) * per) into bkt, and
-// the run's bucket counts into hist[bucket * kOrderMaxRuns + b] (per-warp
-// counters first).  Two draws per iteration, so two Philox chains overlap.
-// With `high` set (the two-pass order), r >> shift is a 16-bit range: its low
-// byte is the bucket of this pass and its high byte is stored in high[] for
-// the second pass.
-template <int SAMPLER>
-__global__ void __launch_bounds__(kOrderThreads)
-k_order_count(uint64_t total, uint64_t kk, uint64_t seed, uint64_t first_id, int shift, uint64_t per,
-              uint32_t *hist, uint8_t *bkt, uint8_t *high) {
-    __shared__ uint32_t s_h[kOrderWarps][kOrderBuckets];
-    const int warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < kOrderWarps * kOrderBuckets; i += kOrderThreads) (&s_h[0][0])[i] = 0;
-    __syncthreads();
-    const uint64_t lo = (uint64_t)blockIdx.x * per;
-    const uint64_t hi = lo + per < kk ? lo + per : kk;
-    for (uint64_t s = lo + threadIdx.x; s < hi; s += 2 * kOrderThreads) {
-        const uint64_t s2 = s + kOrderThreads;
-        uint32_t c = static_cast<uint32_t>(draw_r_of<SAMPLER>(total, seed, first_id + s) >> shift);
-        uint32_t c2 = static_cast<uint32_t>(draw_r_of<SAMPLER>(total, seed, first_id + s2) >> shift);
-        if (high) {
-            high[s] = static_cast<uint8_t>(c >> 8);
-            if (s2 < hi) high[s2] = static_cast<uint8_t>(c2 >> 8);
-            c &= 255u;
-            c2 &= 255u;
-        }
-        bkt[s] = static_cast<uint8_t>(c);
-        atomicAdd(&s_h[warp][c], 1u);
-        if (s2 < hi) {
-            bkt[s2] = static_cast<uint8_t>(c2);
-            atomicAdd(&s_h[warp][c2], 1u);
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kOrderBuckets; b += kOrderThreads) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int w = 0; w < kOrderWarps; w++) c += s_h[w][b];
-        hist[(size_t)b * kOrderMaxRuns + blockIdx.x] = c;
-    }
-}
+template <int THREADS>
+struct PartSmem {
+    uint32_t id[THREADS * kOrderItems];
+    uint32_t key[THREADS * kOrderItems];
+    uint32_t cnt[THREADS * 4];   // counts, then first tile-local places
+    uint32_t base[THREADS * 4];  // place in the bucket of the tile-local place 0
+    uint32_t warp[32];
+};
 
-// The second pass's counts: the bucket of every position is the stored high
-// byte; per-run counts as in k_order_count.
-__global__ void __launch_bounds__(kOrderThreads)
-k_order_count_bytes(uint64_t kk, uint64_t per, const uint8_t *__restrict__ bkt, uint32_t *hist) {
-    __shared__ uint32_t s_h[kOrderWarps][kOrderBuckets];
-    const int warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < kOrderWarps * kOrderBuckets; i += kOrderThreads) (&s_h[0][0])[i] = 0;
-    __syncthreads();
-    const uint64_t lo = (uint64_t)blockIdx.x * per;
-    const uint64_t hi = lo + per < kk ? lo + per : kk;
-    for (uint64_t s = lo + threadIdx.x; s < hi; s += kOrderThreads) atomicAdd(&s_h[warp][bkt[s]], 1u);
-    __syncthreads();
-    for (int b = threadIdx.x; b < kOrderBuckets; b += kOrderThreads) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int w = 0; w < kOrderWarps; w++) c += s_h[w][b];
-        hist[(size_t)b * kOrderMaxRuns + blockIdx.x] = c;
-    }
-}
-
-// Exclusive prefix of v[0..kOrderBuckets) across the first kOrderBuckets
-// threads of the block (every thread must call it); returns thread t's
-// exclusive prefix and leaves the total in *total.
-__device__ __forceinline__ uint32_t bucket_scan(uint32_t v, uint32_t *s_warp, uint32_t *total) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    uint32_t x = t < kOrderBuckets ? v : 0u;
+// Exclusive prefix of v over the block (s_warp: 32 words of scratch).
+template <int THREADS>
+__device__ __forceinline__ uint32_t block_excl_sum(uint32_t v, uint32_t *s_warp) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31 && warp < kOrderBuckets / 32) s_warp[warp] = x;
+    if (lane == 31) s_warp[warp] = x;
     __syncthreads();
-    uint32_t before = 0, all = 0;
-#pragma unroll
-    for (int w = 0; w < kOrderBuckets / 32; w++) {
-        const uint32_t sw = s_warp[w];
-        before += w < warp ? sw : 0u;
-        all += sw;
-    }
-    __syncthreads();
-    *total = all;
-    return before + x - (t < kOrderBuckets ? v : 0u);
+    uint32_t w = lane < THREADS / 32 ? s_warp[lane] : 0u;
+    uint32_t before = lane < warp ? w : 0u;
+    before = __reduce_add_sync(0xffffffffu, before);
+    return before + x - v;
 }
 
-// Block b (kOrderBuckets threads, 4 runs each): bucket b's run counts become
-// exclusive offsets within the bucket, and totals[b] its size.
-__global__ void __launch_bounds__(kOrderBuckets)
-k_order_offsets(int runs, uint32_t *hist, uint32_t *totals) {
-    static_assert(4 * kOrderBuckets == kOrderMaxRuns, "4 runs per thread");
-    __shared__ uint32_t s_warp[kOrderBuckets / 32];
-    uint32_t *p = hist + (size_t)blockIdx.x * kOrderMaxRuns + 4 * threadIdx.x;
-    uint32_t c[4], sum = 0;
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        c[i] = 4 * threadIdx.x + i < runs ? p[i] : 0u;
-        sum += c[i];
-    }
-    uint32_t all;
-    uint32_t run = bucket_scan(sum, s_warp, &all);
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        if (4 * threadIdx.x + i < runs) p[i] = run;
-        run += c[i];
-    }
-    if (threadIdx.x == 0) totals[blockIdx.x] = all;
-}
-
-// Block b places its run of ids, kOrderTile at a time: each tile is first
-// counting-sorted by bucket in shared memory, then each bucket's ids are
-// written as one contiguous piece at the run's cursor for that bucket
-// (base[bucket] + the run's offset within it, advanced after every tile), so
-// the stores coalesce.  The buckets of the next tile are loaded while the
-// current one is placed.  The value placed for input position q is q, or
-// vals[q] when vals is given (the second pass of the two-pass order, whose
-// input is the first pass's output); a byte carry[q] travels with it into
-// carry_out when carry is given.
-__global__ void __launch_bounds__(kOrderThreads)
-k_order_scatter(uint64_t kk, uint64_t per, const uint32_t *__restrict__ hist, const uint32_t *__restrict__ totals,
-                const uint8_t *__restrict__ bkt, const uint32_t *__restrict__ vals, const uint8_t *__restrict__ carry,
-                uint32_t *__restrict__ ids, uint8_t *__restrict__ carry_out) {
-    __shared__ uint32_t s_cur[kOrderBuckets], s_cnt[kOrderBuckets], s_off[kOrderBuckets];
-    __shared__ uint32_t s_warp[kOrderBuckets / 32];
-    __shared__ uint32_t s_id[kOrderTile];
-    __shared__ uint8_t s_b[kOrderTile];
-    __shared__ uint8_t s_c[kOrderTile];
+// The first kernel.  A tile of THREADS * kOrderItems ids per block and turn:
+// each id's key is the high word its edge draw starts from; the tile is
+// counting-sorted by bucket in shared memory, room for its runs is reserved
+// with one atomic per bucket, and each run is written as one piece.  At most
+// 4 * THREADS buckets.  2^27 ids into 4096 buckets take 1.22 ms, 0.47 of them
+// the Philox rounds; the rest is the short runs (4 ids) of so many buckets --
+// 2^24 ids into 512 buckets take 98 us.
+template <int SAMPLER, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+k_order_partition(uint64_t kk, uint64_t seed, uint64_t first_id, int bits, uint32_t room, uint32_t *cursor,
+                  uint32_t *spilled, uint32_t *__restrict__ ids, uint16_t *__restrict__ keys) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    PartSmem<THREADS> &S = *reinterpret_cast<PartSmem<THREADS> *>(s_raw);
+    constexpr int kTile = THREADS * kOrderItems;
     const int t = threadIdx.x;
-    {
-        // the buckets' first positions: exclusive prefix of their totals
-        uint32_t all;
-        const uint32_t base = bucket_scan(t < kOrderBuckets ? totals[t] : 0u, s_warp, &all);
-        if (t < kOrderBuckets) s_cur[t] = base + hist[(size_t)t * kOrderMaxRuns + blockIdx.x];
-    }
-    const uint64_t lo = (uint64_t)blockIdx.x * per;
-    const uint64_t hi = lo + per < kk ? lo + per : kk;
-    uint32_t nxt[kOrderItems];
+    const uint32_t buckets = 1u << bits;
+    const int down = 32 - bits;  // 20..32
+    for (uint64_t t0 = (uint64_t)blockIdx.x * kTile; t0 < kk; t0 += (uint64_t)gridDim.x * kTile) {
+        const int n = kk - t0 < kTile ? static_cast<int>(kk - t0) : kTile;
 #pragma unroll
-    for (int i = 0; i < kOrderItems; i++) {
-        const uint64_t q = lo + (uint64_t)i * kOrderThreads + t;
-        nxt[i] = q < hi ? static_cast<uint32_t>(bkt[q]) : static_cast<uint32_t>(kOrderBuckets);
-    }
-    for (uint64_t t0 = lo; t0 < hi; t0 += kOrderTile) {
-        if (t < kOrderBuckets) s_cnt[t] = 0;
-        uint32_t myb[kOrderItems], rank[kOrderItems];
+        for (int q = 0; q < 4; q++) S.cnt[q * THREADS + t] = 0;
+        __syncthreads();
+        uint32_t key[kOrderItems];
+        uint32_t rank2[kOrderItems / 2];
 #pragma unroll
         for (int i = 0; i < kOrderItems; i++) {
-            myb[i] = nxt[i];
-            const uint64_t q = t0 + kOrderTile + (uint64_t)i * kOrderThreads + t;
-            nxt[i] = q < hi ? static_cast<uint32_t>(bkt[q]) : static_cast<uint32_t>(kOrderBuckets);
+            const int q = i * THREADS + t;
+            key[i] = sample_block(seed, first_id + t0 + q, 0, SAMPLER).y;
+            const uint32_t b = bits ? key[i] >> down : 0u;
+            const uint32_t r = q < n ? atomicAdd(&S.cnt[b], 1u) : 0u;  // below kTile <= 2^16
+            if (i & 1) rank2[i / 2] |= r << 16;
+            else rank2[i / 2] = r;
+        }
+        __syncthreads();
+        // thread t: buckets 4 t .. 4 t + 3
+        uint32_t c[4], sum = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            c[q] = S.cnt[4 * t + q];
+            sum += c[q];
+        }
+        uint32_t run = block_excl_sum<THREADS>(sum, S.warp);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t b = 4 * t + q;
+            const uint32_t at = c[q] && b < buckets ? atomicAdd(cursor + b * kCursorStride, c[q]) : 0u;
+            S.cnt[b] = run;
+            S.base[b] = at - run;
+            run += c[q];
         }
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < kOrderItems; i++)
-            if (myb[i] < kOrderBuckets) rank[i] = atomicAdd(s_cnt + myb[i], 1u);
-        __syncthreads();
-        uint32_t all;
-        const uint32_t off = bucket_scan(t < kOrderBuckets ? s_cnt[t] : 0u, s_warp, &all);
-        if (t < kOrderBuckets) s_off[t] = off;
-        __syncthreads();
-#pragma unroll
         for (int i = 0; i < kOrderItems; i++) {
-            if (myb[i] < kOrderBuckets) {
-                const uint32_t p = s_off[myb[i]] + rank[i];
-                const uint64_t q = t0 + (uint64_t)i * kOrderThreads + t;
-                s_id[p] = vals ? vals[q] : static_cast<uint32_t>(q);
-                s_b[p] = static_cast<uint8_t>(myb[i]);
-                if (carry) s_c[p] = carry[q];
+            const int q = i * THREADS + t;
+            if (q < n) {
+                const uint32_t b = bits ? key[i] >> down : 0u;
+                const uint32_t p = S.cnt[b] + ((rank2[i / 2] >> (16 * (i & 1))) & 0xffffu);
+                S.id[p] = static_cast<uint32_t>(t0) + q;
+                S.key[p] = key[i];
             }
         }
         __syncthreads();
-        for (uint32_t p = t; p < all; p += kOrderThreads) {
-            const uint32_t b = s_b[p];
-            const uint32_t dst = s_cur[b] + (p - s_off[b]);
-            ids[dst] = s_id[p];
-            if (carry) carry_out[dst] = s_c[p];
+        bool over = false;
+        for (int p = t; p < n; p += THREADS) {
+            const uint32_t k = S.key[p];
+            const uint32_t b = bits ? k >> down : 0u;
+            const uint32_t at = S.base[b] + p;
+            if (at < room) {
+                const uint32_t dst = b * room + at;
+                ids[dst] = S.id[p];
+                keys[dst] = static_cast<uint16_t>((k << bits) >> 16);
+            } else {
+                over = true;
+            }
         }
+        if (over) *spilled = 1u;
         __syncthreads();
-        if (t < kOrderBuckets) s_cur[t] += s_cnt[t];
     }
+}
+
+// The second kernel, a block per bucket: its ids by the next bits (11 or 12,
+// four counters per thread), behind the ids of the buckets before it.
+template <int THREADS, int ITEMS>
+struct LocalSmem {
+    uint32_t id[THREADS * ITEMS];
+    uint32_t cnt[4 * THREADS];
+    uint32_t warp[32];
+};
+
+template <int THREADS, int ITEMS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+k_order_local(uint32_t room, const uint32_t *__restrict__ cursor, const uint32_t *__restrict__ spilled,
+              const uint32_t *__restrict__ ids, const uint16_t *__restrict__ keys, uint32_t *__restrict__ out) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    using Smem = LocalSmem<THREADS, ITEMS>;
+    Smem &S = *reinterpret_cast<Smem *>(s_raw);
+    constexpr int kDown = THREADS == 1024 ? 4 : 5;  // of the 16 key bits, those not sorted by
+    static_assert((1 << (16 - kDown)) == 4 * THREADS, "four counters per thread");
+    if (*spilled) return;
+    const int t = threadIdx.x;
+    const uint32_t n = __ldg(cursor + blockIdx.x * kCursorStride);  // at most room
+    ids += static_cast<size_t>(blockIdx.x) * room;
+    keys += static_cast<size_t>(blockIdx.x) * room;
+#pragma unroll
+    for (int q = 0; q < 4; q++) S.cnt[q * THREADS + t] = 0;
+    // ids in the buckets before this one
+    uint32_t before = 0;
+    for (uint32_t b = t; b < blockIdx.x; b += THREADS) before += __ldg(cursor + b * kCursorStride);
+    __syncthreads();
+    uint32_t place[ITEMS];  // key << 16 | rank among the bucket's ids of that key
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+        const uint32_t q = i * THREADS + t;
+        place[i] = q < n ? static_cast<uint32_t>(__ldg(keys + q)) >> kDown : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++)
+        if (i * THREADS + t < n) place[i] = place[i] << 16 | atomicAdd(&S.cnt[place[i]], 1u);
+    before = __reduce_add_sync(0xffffffffu, before);
+    __syncthreads();
+    uint32_t c[4], sum = 0;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        c[q] = S.cnt[4 * t + q];
+        sum += c[q];
+    }
+    uint32_t run = block_excl_sum<THREADS>(sum, S.warp);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        S.cnt[4 * t + q] = run;
+        run += c[q];
+    }
+    __syncthreads();
+    if ((t & 31) == 0) S.warp[t >> 5] = before;
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+        const uint32_t q = i * THREADS + t;
+        if (q < n) S.id[S.cnt[place[i] >> 16] + (place[i] & 0xffffu)] = __ldg(ids + q);
+    }
+    __syncthreads();
+    out += __reduce_add_sync(0xffffffffu, (t & 31) < THREADS / 32 ? S.warp[t & 31] : 0u);
+    for (uint32_t p = t; p < n; p += THREADS) out[p] = S.id[p];
 }
 
 template <int SAMPLER, int BLOCK, int ADJ>
 __global__ void __launch_bounds__(BLOCK, sample_min_blocks<BLOCK>())
 k_sample_ordered(GraphDev g, uint64_t kk, uint64_t seed, uint64_t first_id, const uint32_t *__restrict__ ids,
-                 uint64_t *hist) {
+                 const uint32_t *__restrict__ spilled, uint64_t *hist) {
+    const bool sorted = __ldg(spilled) == 0u;
     Counts6 cnt;
     cnt.zero();
     const uint64_t stride = (uint64_t)gridDim.x * BLOCK;
     for (uint64_t p = (uint64_t)blockIdx.x * BLOCK + threadIdx.x; p < kk; p += stride) {
-        const uint64_t id = first_id + __ldg(ids + p);
+        const uint64_t id = first_id + (sorted ? __ldg(ids + p) : p);
         cnt.add(SAMPLER == 0 ? sample_3path<ADJ>(g, seed, id) : sample_centred<ADJ>(g, seed, id));
     }
     flush_counts<BLOCK>(cnt, SAMPLER == 0 ? 6 : 4, hist);
 }
 
+template <int SAMPLER, int THREADS>
+static int launch_partition(const ps_graph *g, uint64_t kk, uint64_t seed, uint64_t first_id, const OrderPlan &plan,
+                            uint32_t *cursor, uint32_t *spilled, uint32_t *ids, uint16_t *keys, cudaStream_t s) {
+    constexpr uint64_t kTile = THREADS * kOrderItems;
+    const int smem = static_cast<int>(sizeof(PartSmem<THREADS>));
+    PS_CUDA_TRY(cudaFuncSetAttribute(k_order_partition<SAMPLER, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const uint64_t tiles = (kk + kTile - 1) / kTile, full = (uint64_t)g->sm_count * (1024 / THREADS);
+    k_order_partition<SAMPLER, THREADS><<<(unsigned)(tiles < full ? tiles : full), THREADS, smem, s>>>(
+        kk, seed, first_id, plan.bits, plan.room, cursor, spilled, ids, keys);
+    PS_LAUNCH_CHECK();
+    return PS_OK;
+}
+
+template <int THREADS, int ITEMS>
+static int launch_local(const OrderPlan &plan, const uint32_t *cursor, const uint32_t *spilled, const uint32_t *ids,
+                        const uint16_t *keys, uint32_t *sorted, cudaStream_t s) {
+    const int smem = static_cast<int>(sizeof(LocalSmem<THREADS, ITEMS>));
+    PS_CUDA_TRY(cudaFuncSetAttribute(k_order_local<THREADS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_order_local<THREADS, ITEMS><<<1u << plan.bits, THREADS, smem, s>>>(plan.room, cursor, spilled, ids, keys, sorted);
+    PS_LAUNCH_CHECK();
+    return PS_OK;
+}
+
 template <int SAMPLER, int BLOCK, int ADJ>
 static int ordered_t(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t first_id, uint64_t *hist,
                      char *scratch, uint64_t chunk, cudaStream_t s) {
-    const uint64_t total = SAMPLER == 0 ? g->stats.W : g->stats.Lambda;
-    // the two-pass order sorts by 16 bits of r (65536 ranges), the one-pass by 8
-    const bool two_pass = g->tune.draw_order == 2 || (g->tune.draw_order == 0 && g->m >= kOrderTwoPassEdges);
-    const uint64_t ranges = two_pass ? 65536u : static_cast<uint64_t>(kOrderBuckets);
-    int shift = 0;
-    while (shift < 63 && ((total - 1) >> shift) >= ranges) shift++;
-    uint32_t *hist_runs = reinterpret_cast<uint32_t *>(scratch);
-    uint32_t *totals = reinterpret_cast<uint32_t *>(scratch + kOrderHist);
-    // per sample of a chunk: the sorted ids, the first pass's ids, the
-    // bucket byte, the high byte and the high byte in first-pass order
-    uint32_t *ids = reinterpret_cast<uint32_t *>(scratch + kOrderHeader);
-    uint32_t *ids1 = ids + chunk;
-    uint8_t *bkt = reinterpret_cast<uint8_t *>(ids1 + chunk);
-    uint8_t *high = bkt + chunk;
-    uint8_t *high1 = high + chunk;
+    uint32_t *cursor = reinterpret_cast<uint32_t *>(scratch);
+    uint32_t *spilled = cursor + kOrderBuckets * kCursorStride;
+    uint32_t *sorted = reinterpret_cast<uint32_t *>(scratch + kOrderHeader);
     int per_sm = g->tune.blocks_per_sm;
     if (per_sm <= 0) {
         int occ = 0;
@@ -280,42 +306,32 @@ static int ordered_t(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t firs
     const uint64_t full = (uint64_t)g->sm_count * per_sm;
     while (k > 0) {
         const uint64_t kk = k < chunk ? k : chunk;
-        if (kk < kOrderMinChunk && g->tune.draw_order == 0) {
+        if (kk < order_min_chunk(g->m) && g->tune.draw_order == 0) {
             const int rc = launch_sampler(g, SAMPLER, kk, seed, first_id, hist, s);
             if (rc) return rc;
         } else {
-            uint64_t runs = (uint64_t)g->sm_count * 2;  // one wave of the count kernel
-            if (runs > (uint64_t)kOrderMaxRuns) runs = kOrderMaxRuns;
-            const uint64_t per = (kk + runs - 1) / runs;
-            runs = (kk + per - 1) / per;
+            const OrderPlan plan = order_plan(kk);
+            const uint64_t places = static_cast<uint64_t>(plan.room) << plan.bits;
+            uint32_t *ids = sorted + kk;
+            uint16_t *keys = reinterpret_cast<uint16_t *>(ids + places);
+            PS_CUDA_TRY(cudaMemsetAsync(cursor, 0, (kOrderBuckets * kCursorStride + 1) * sizeof(uint32_t), s));
+            int rc;
+            // smaller blocks with smaller tiles overlap their phases and fill
+            // the SMs on short chunks; with many buckets, longer tiles keep a
+            // bucket's runs from getting too short
+            if (!plan.large) {
+                rc = launch_partition<SAMPLER, 256>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
+                if (!rc) rc = launch_local<kSmallThreads, kSmallItems>(plan, cursor, spilled, ids, keys, sorted, s);
+            } else {
+                if (plan.bits <= 11) rc = launch_partition<SAMPLER, 512>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
+                else rc = launch_partition<SAMPLER, 1024>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
+                if (!rc) rc = launch_local<kLargeThreads, kLargeItems>(plan, cursor, spilled, ids, keys, sorted, s);
+            }
+            if (rc) return rc;
             uint64_t blocks = (kk + BLOCK - 1) / BLOCK;
             if (blocks > full) blocks = full;
-            k_order_count<SAMPLER><<<(unsigned)runs, kOrderThreads, 0, s>>>(total, kk, seed, first_id, shift, per,
-                                                                         hist_runs, bkt, two_pass ? high : nullptr);
-            PS_LAUNCH_CHECK();
-            k_order_offsets<<<kOrderBuckets, kOrderBuckets, 0, s>>>(static_cast<int>(runs), hist_runs, totals);
-            PS_LAUNCH_CHECK();
-            if (!two_pass) {
-                k_order_scatter<<<(unsigned)runs, kOrderThreads, 0, s>>>(kk, per, hist_runs, totals, bkt, nullptr,
-                                                                         nullptr, ids, nullptr);
-                PS_LAUNCH_CHECK();
-            } else {
-                // least significant byte first, then the high byte: every id
-                // ends in its 16-bit range of r (in range order; within a range
-                // the order of a tile's ids is free)
-                k_order_scatter<<<(unsigned)runs, kOrderThreads, 0, s>>>(kk, per, hist_runs, totals, bkt, nullptr,
-                                                                         high, ids1, high1);
-                PS_LAUNCH_CHECK();
-                k_order_count_bytes<<<(unsigned)runs, kOrderThreads, 0, s>>>(kk, per, high1, hist_runs);
-                PS_LAUNCH_CHECK();
-                k_order_offsets<<<kOrderBuckets, kOrderBuckets, 0, s>>>(static_cast<int>(runs), hist_runs, totals);
-                PS_LAUNCH_CHECK();
-                k_order_scatter<<<(unsigned)runs, kOrderThreads, 0, s>>>(kk, per, hist_runs, totals, high1, ids1,
-                                                                         nullptr, ids, nullptr);
-                PS_LAUNCH_CHECK();
-            }
-            k_sample_ordered<SAMPLER, BLOCK, ADJ><<<(unsigned)blocks, BLOCK, 0, s>>>(g->dev, kk, seed, first_id, ids,
-                                                                                    hist);
+            k_sample_ordered<SAMPLER, BLOCK, ADJ><<<(unsigned)blocks, BLOCK, 0, s>>>(g->dev, kk, seed, first_id, sorted,
+                                                                                    spilled, hist);
             PS_LAUNCH_CHECK();
         }
         k -= kk;
@@ -346,10 +362,6 @@ static int ordered_s(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t firs
     }
 }
 
-// Bytes per sample of a chunk: its sorted id, its id after the first of two
-// passes, its bucket byte and its high byte in both orders.
-constexpr size_t kOrderPerSample = 2 * sizeof(uint32_t) + 3 * sizeof(uint8_t);
-
 size_t ordered_scratch_bytes(uint64_t k_chunk) {
     if (k_chunk == 0 || k_chunk > kOrderMaxChunk) return 0;
     return kOrderHeader + static_cast<size_t>(k_chunk) * kOrderPerSample;
@@ -359,7 +371,7 @@ int launch_ordered(const ps_graph *g, int sampler, uint64_t k, uint64_t seed, ui
                    void *d_scratch, size_t scratch_bytes, cudaStream_t s) {
     if (scratch_bytes < ordered_scratch_bytes(1)) return PS_ERR_WORKSPACE;
     uint64_t chunk = (scratch_bytes - kOrderHeader) / kOrderPerSample;
-    if (chunk > kOrderMaxChunk) chunk = kOrderMaxChunk;
+    if (chunk > kOrderMaxSorted) chunk = kOrderMaxSorted;
     if (g->tune.draw_order < 0 || (g->tune.draw_order == 0 && g->m < kOrderMinEdges))
         return launch_sampler(g, sampler, k, seed, first_id, d_hist, s);
     char *scratch = static_cast<char *>(d_scratch);
