@@ -110,7 +110,8 @@ size_t ps_graph_workspace_bytes(int64_t n, int64_t nnz, const ps_tuning *t);
  * ascending, and builds the edge table (u < v, u ascending then v ascending)
  * with the positions of each edge in both endpoint lists, the inclusive
  * uint64 prefix sums of the weights tau_e and lambda_e (in the same pass as
- * the table), and (default adjacency) the edge filter.
+ * the table), the guide tables of the edge draw, the hub bitmap rows and
+ * (default adjacency) the edge filter.
  *
  * d_off / d_col belong to the caller and are only read during the call.
  * d_workspace (ws_bytes >= ps_graph_workspace_bytes(n, nnz, t), 256-byte
@@ -127,13 +128,13 @@ int ps_load_csr(int64_t n, int64_t nnz, const int64_t *d_off, const int32_t *d_c
 /* Section 3 (tau_e, W) and Section 4 (lambda_e, Lambda), the edge
  * distributions of Alg. 1 and Alg. 3: publishes the totals W and Lambda of
  * the inclusive uint64 prefix sums that ps_load_csr wrote (exact, so the edge
- * draw is exact), computes N_1 of Alg. 2, the guide tables of the
- * inverse-CDF search and the structures of the chosen adjacency variant; no
- * sampler may run before it.  Does not synchronise: the totals were read
- * back by ps_load_csr, *out is filled at once, and the guide tables and
- * adjacency structures are finished in `stream` order, so sampling on
- * another stream must first wait for `stream`.  A second call returns the same totals without
- * recomputing.  Returns PS_NO_PATHS when W == 0 or Lambda == 0
+ * draw is exact), N_1 of Alg. 2 and the hub count; no sampler may run before
+ * it.  The guide tables of the inverse-CDF search and the hub rows were built
+ * by ps_load_csr too; the per-vertex tables of adjacency 3 are built here.
+ * Does not synchronise: *out is filled at once, and what the call queues is
+ * finished in `stream` order, so sampling on another stream must first wait
+ * for `stream`.  A second call returns the same totals without recomputing.
+ * Returns PS_NO_PATHS when W == 0 or Lambda == 0
  * (sampling then leaves histograms untouched), PS_ERR_OVERFLOW when a sum
  * does not fit in 64 bits, PS_ERR_TIMEOUT when a scan's bounded wait
  * expired. */

@@ -202,6 +202,7 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.keys1 = take(n1 * sizeof(uint32_t));
     l.vals0 = take(n1 * sizeof(uint32_t));
     l.vals1 = take(n1 * sizeof(uint32_t));
+    l.inv = take(n1 * sizeof(uint32_t));
     l.counts = take(static_cast<size_t>(256) * std::max(sort_tiles(n), sort_tiles(l.m_cap)) * sizeof(uint32_t));
     l.total = p;
     *L = l;

@@ -40,6 +40,7 @@ namespace ps {
 // more lower arcs than the buffers hold; those beyond m_cap are dropped (the
 // status check after the load rejects the graph).
 constexpr int kListBatch = 4;
+constexpr int64_t kFewRows = int64_t{1} << 18;
 
 __global__ void __launch_bounds__(256)
 k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
@@ -85,17 +86,17 @@ k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restr
     }
 }
 
-// Rows of kLongRow + 1 .. kTierC entries: a warp per row, the next row's
-// offsets fetched while the current one is copied.
+// Rows of kLongRow + 1 .. kTierC entries (from status[first_slot] on): a warp
+// per row, the next row's offsets fetched while the current one is copied.
 __global__ void __launch_bounds__(256)
 k_lower_arcs_mid(const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                  const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase,
                  uint32_t *__restrict__ key, uint32_t *__restrict__ val, int64_t m_cap,
-                 const u64 *__restrict__ status) {
+                 const u64 *__restrict__ status, int first_slot) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
     const int64_t r_end = static_cast<int64_t>(status[ST_TIER + 3]);
-    int64_t r = static_cast<int64_t>(status[ST_LONG]) + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    int64_t r = static_cast<int64_t>(status[first_slot]) + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     int64_t o_ = 0, ub_ = 0;
     int32_t low_ = 0;
     if (r < r_end) {
@@ -291,13 +292,18 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
     while (bits < 31 && (static_cast<uint64_t>(n > 0 ? n - 1 : 0) >> bits) != 0) bits++;
     const int passes = bits > 0 ? (bits + 7) / 8 : 1;
     if (n > 0) {
-        int64_t blocks = (n + 255) / 256;  // a warp per 32 rows
-        if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-        k_lower_arcs<<<(unsigned)blocks, 256, 0, s>>>(n, g->off, g->col, g->ubase, ka, va, m, g->status);
-        PS_LAUNCH_CHECK();
-        if (g->d_max > kLongRow) {
-            k_lower_arcs_mid<<<(unsigned)(sms * 6), 256, 0, s>>>(g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
-                                                                  g->status);
+        // few rows: a warp each for the short ones too (5,000 rows: 16 -> 4 us;
+        // 32 short rows are up to 32 steps for one warp)
+        const bool few = n < kFewRows;
+        if (!few) {
+            int64_t blocks = (n + 255) / 256;  // a warp per 32 rows
+            if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
+            k_lower_arcs<<<(unsigned)blocks, 256, 0, s>>>(n, g->off, g->col, g->ubase, ka, va, m, g->status);
+            PS_LAUNCH_CHECK();
+        }
+        if (few || g->d_max > kLongRow) {
+            k_lower_arcs_mid<<<(unsigned)(sms * (few ? 8 : 6)), 256, 0, s>>>(g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
+                                                                             g->status, few ? ST_TIER : ST_LONG);
             PS_LAUNCH_CHECK();
         }
         if (g->d_max > kTierC) {

@@ -48,7 +48,7 @@ struct Layout {
     int64_t filt_words;    // 32-bit words of the edge filter; 0 without it
     int64_t vtab_slots;    // 0 without the per-vertex tables
     size_t status, off, col, rank, lowcnt, ubase, dnew, rec, ptau, plam, gtau, glam, hub, filt, vtab;
-    size_t keys0, keys1, vals0, vals1, counts, scan;
+    size_t keys0, keys1, vals0, vals1, inv, counts, scan;
     size_t total;
 };
 bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L);
@@ -121,7 +121,8 @@ void count_launch();
 // pass.  vin null: the values are the items' indices.  vshift > 0: the digit
 // goes on with the value's lowest bits, vshift of its bits being the key's.
 // dcount (device, may be null) bounds the items at run time.  counts: 256
-// words per tile.
+// words per tile.  max_key (device, may be null): the largest key; a pass
+// after the first that sorts by higher bits only does nothing.
 struct SortPass {
     int64_t count;
     const u64 *dcount;
@@ -129,6 +130,7 @@ struct SortPass {
     uint32_t *kout, *vout;
     int shift, bits, vshift;
     uint32_t *counts;
+    const u64 *max_key = nullptr;
 };
 int64_t sort_tiles(int64_t count);
 // tiles of the pass's scan (0: it needs none and `scan` is not touched)
@@ -160,6 +162,19 @@ inline int run_scan(ps_graph *g, int64_t count, T identity, Op op, Load load, St
     k_scan<T, kScanBlock, kScanItems><<<(unsigned)tiles, kScanBlock, 0, s>>>(count, st, identity, op, load, store);
     PS_LAUNCH_CHECK();
     return PS_OK;
+}
+
+// The guide tables and the hub rows (ps_prefix.cu), queued by the load step:
+// both take their sizes (the totals W and Lambda, the hub count) from the
+// status words on the device.  The guide tables are left alone when the input
+// has turned out invalid.
+int launch_guides(ps_graph *g, cudaStream_t s);
+int launch_hub_rows(ps_graph *g, cudaStream_t s);
+// Guide bucket of r is r >> guide_shift(total, buckets).
+__host__ __device__ inline int guide_shift(uint64_t total, int64_t gcap) {
+    int s = 0;
+    while (s < 63 && ((total - 1) >> s) >= static_cast<uint64_t>(gcap)) s++;
+    return s;
 }
 
 // The edge table (ps_edges.cu): after the rows are relabelled and sorted and

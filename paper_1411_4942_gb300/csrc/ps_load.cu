@@ -28,7 +28,7 @@ __global__ void k_degrees(int64_t n, int64_t nnz, const int64_t *__restrict__ of
             bad = true;
             d = 0;
         }
-        if (d > n - 1) longrow = true;  // cannot be a simple row
+        if (d > n - 1) longrow = true;  // cannot be a simple row; the load ends early
         keys[v] = static_cast<uint32_t>(d);
         dmax = max(dmax, static_cast<uint32_t>(d));
     }
@@ -40,22 +40,41 @@ __global__ void k_degrees(int64_t n, int64_t nnz, const int64_t *__restrict__ of
         atomicMax(reinterpret_cast<unsigned long long *>(status + ST_DMAX), (unsigned long long)dmax);
 }
 
+// F_ARG for a column out of range (when the rows themselves are not walked).
+__global__ void __launch_bounds__(256) k_check_columns(int64_t n, int64_t nnz, const int32_t *__restrict__ col, u64 *status) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    bool bad = false;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += stride) {
+        const int32_t c = ldg_i32(col + i);
+        bad |= c < 0 || c >= n;
+    }
+    if (bad) raise_flag(status, F_ARG);
+}
+
 // The sorted (degree, vertex) pairs, position r = label r: rank[v] = the label
-// of v, dnew[r] = its degree, lowcnt[r] = 0; the first label whose degree
+// of v, inv[r] = v, dnew[r] = its degree, lowcnt[r] = 0.  The pairs are in the
+// first or the second buffers, by how many sort passes the largest degree
+// needed.  Also the first label whose degree
 // exceeds each row-length limit; N_1 = sum_v C(d_v, 3) (128-bit); and the
 // number of hub rows: the top `hub_cap` labels whose degree is at least
 // `hub_min`.
 __global__ void __launch_bounds__(256)
-k_rank(int64_t n, const uint32_t *__restrict__ skeys, const uint32_t *__restrict__ svals, int32_t *rank,
-       int32_t *dnew, int32_t *lowcnt, int64_t hub_cap, int64_t hub_min, u64 *status) {
+k_rank(int64_t n, int bits, const uint32_t *__restrict__ k0, const uint32_t *__restrict__ v0,
+       const uint32_t *__restrict__ k1, const uint32_t *__restrict__ v1, int32_t *rank, uint32_t *inv, int32_t *dnew,
+       int32_t *lowcnt, int64_t hub_cap, int64_t hub_min, u64 *status) {
     const uint32_t lim[5] = {0, kTierA, kTierB, kTierC, kLongRow};
     const int slot[5] = {ST_TIER, ST_TIER + 1, ST_TIER + 2, ST_TIER + 3, ST_LONG};
+    bool second = true;  // the first pass moves the pairs to the second buffers, and so on
+    for (int shift = 8; shift < bits && (status[ST_DMAX] >> shift) != 0; shift += 8) second = !second;
+    const uint32_t *skeys = second ? k1 : k0, *svals = second ? v1 : v0;
     uint64_t lo = 0, hi = 0;
     unsigned long long hubs = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
         const uint32_t d = __ldg(skeys + r);
-        rank[__ldg(svals + r)] = static_cast<int32_t>(r);
+        const uint32_t v = __ldg(svals + r);
+        rank[v] = static_cast<int32_t>(r);
+        inv[r] = v;
         dnew[r] = static_cast<int32_t>(d);
         lowcnt[r] = 0;
         const uint32_t before = r ? __ldg(skeys + r - 1) : 0u;
@@ -746,37 +765,56 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     // (1) degrees and offset validation; nothing else may index with bad offsets
     k_degrees<<<sms * 8, 256, 0, s>>>(n, nnz, d_off, k0, g->status);
     PS_LAUNCH_CHECK();
-    uint64_t st[ST_WORDS];
-    PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));
-    PS_CUDA_TRY(cudaStreamSynchronize(s));
-    if (st[ST_FLAGS] & F_ARG) return PS_ERR_ARG;
-    g->d_max = static_cast<int64_t>(st[ST_DMAX]);
+    SideFork read(g, s);
+    int rc = read.fork(1);
+    if (rc) return rc;
 
-    // (2) stable radix sort of (degree, id): ties keep increasing id
+    // (2) stable radix sort of (degree, id): ties keep increasing id.  Queued
+    // before the host has seen the largest degree (below n on valid input):
+    // passes above its bits do nothing.
     int bits = 1;
-    while (bits < 32 && (static_cast<uint64_t>(g->d_max) >> bits) != 0) bits++;
-    int rc = PS_OK;
+    while (bits < 31 && (static_cast<uint64_t>(n > 0 ? n - 1 : 0) >> bits) != 0) bits++;
     for (int shift = 0; shift < bits && n > 0; shift += 8) {
+        const bool even = shift % 16 == 0;
         ScanState<uint32_t> scan{};
         if (sort_scan_tiles(n)) rc = take_scan(g, sort_scan_tiles(n), &scan);
         if (rc) return rc;
-        rc = sort_pass({n, nullptr, k0, shift ? v0 : nullptr, k1, v1, shift, std::min(8, bits - shift), 0,
-                        reinterpret_cast<uint32_t *>(ws + L.counts)}, scan, s);
+        rc = sort_pass({n, nullptr, even ? k0 : k1, shift ? (even ? v0 : v1) : nullptr, even ? k1 : k0, even ? v1 : v0,
+                        shift, std::min(8, bits - shift), 0, reinterpret_cast<uint32_t *>(ws + L.counts),
+                        g->status + ST_DMAX}, scan, s);
         if (rc) return rc;
-        std::swap(k0, k1);
-        std::swap(v0, v1);
     }
-    // k0 / v0 hold the sorted (degree, vertex) pairs: v0[r] is the vertex with label r
+    uint32_t *inv = reinterpret_cast<uint32_t *>(ws + L.inv);
     if (n > 0) {
-        k_rank<<<sms * 8, 256, 0, s>>>(n, k0, v0, g->rank, g->dnew, g->lowcnt, L.hub_cap, g->tune.hub_min_degree, g->status);
+        k_rank<<<sms * 8, 256, 0, s>>>(n, bits, k0, v0, k1, v1, g->rank, inv, g->dnew, g->lowcnt, L.hub_cap,
+                                       g->tune.hub_min_degree, g->status);
         PS_LAUNCH_CHECK();
     } else {
         PS_CUDA_TRY(cudaMemsetAsync(g->off, 0, sizeof(int64_t), s));
         PS_CUDA_TRY(cudaMemsetAsync(g->ubase, 0, sizeof(int64_t), s));
     }
-    const uint32_t *inv = v0;
     rc = run_scan<int64_t>(g, n, (int64_t)0, OpSum(), LoadDeg{g->dnew}, StoreOffsets{g->off, n}, s);
     if (rc) return rc;
+
+    // the offsets' verdict and the largest degree, read on the side while the
+    // sort runs
+    uint64_t st[ST_WORDS];
+    PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, read.side(0)));
+    PS_CUDA_TRY(cudaStreamSynchronize(read.side(0)));
+    rc = read.join();
+    if (rc) return rc;
+    g->d_max = static_cast<int64_t>(st[ST_DMAX]);
+    if ((st[ST_FLAGS] & F_ARG) || g->d_max >= std::max<int64_t>(n, 1)) {
+        // bad offsets, or a row too long to be simple (then only a column out
+        // of range outranks that)
+        if (!(st[ST_FLAGS] & F_ARG)) {
+            k_check_columns<<<sms * 8, 256, 0, s>>>(n, nnz, d_col, g->status);
+            PS_LAUNCH_CHECK();
+        }
+        PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));
+        PS_CUDA_TRY(cudaStreamSynchronize(s));
+        return flags_to_status(st[ST_FLAGS] | F_NOT_SIMPLE);
+    }
 
     // (3) relabel + sort every row, by tier; the tiers touch disjoint rows, so
     // the long-row tiers run on side streams next to the short-row ones
@@ -824,9 +862,19 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
                            StoreUbase{g->ubase, n, g->status}, s);
     if (rc) return rc;
 
-    // (5) the edge table, the prefixes and the edge filter
+    // (5) on a side stream the hub rows, which need only the sorted rows; here
+    // the edge table, the prefixes and the edge filter, then the guide tables
+    SideFork hubs(g, s);
+    rc = hubs.fork(1);
+    if (rc) return rc;
+    rc = launch_hub_rows(g, hubs.side(0));
+    if (rc) return rc;
     if (g->filt) PS_CUDA_TRY(cudaMemsetAsync(g->filt, 0, sizeof(uint32_t) * L.filt_words, s));
     rc = build_edge_table(g, s);
+    if (rc) return rc;
+    rc = launch_guides(g, s);
+    if (rc) return rc;
+    rc = hubs.join();
     if (rc) return rc;
 
     PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));

@@ -1,8 +1,9 @@
-// ps_prefix.cu -- ps_tau_prefix: the edge weights of Section 3 (tau) and
-// Section 4 (lambda), their exact inclusive uint64 prefixes (the
-// distributions p_e of Alg. 1 / Alg. 3), N_1 of Alg. 2, the guide
-// tables that shorten the inverse-CDF search, and the hub bitmaps used by
-// the adjacency test.
+// ps_prefix.cu -- the guide tables that shorten the inverse-CDF search over
+// the prefixes of tau (Section 3) and lambda (Section 4), and the hub bitmaps
+// of the adjacency test, both queued by the load step; ps_tau_prefix, which
+// publishes the totals; and the per-vertex tables of one adjacency variant.
+#include <algorithm>
+
 #include "ps_internal.h"
 
 namespace ps {
@@ -14,18 +15,32 @@ namespace ps {
 // lane writes its own short run; a warp writes long runs together.  A warp
 // takes kGuideGroups groups of 32 edges per step with all their prefix loads
 // issued first.
+// The heavy edges, with the long runs, are the last ones: on small graphs a
+// warp takes one group, so more warps share them (49k edges: 20 -> 6 us for
+// both tables).
 constexpr int kGuideGroups = 4;
 
+// Table blockIdx.y: 0 = tau, 1 = lambda, its total from the status words.
+// Nothing is written when the load has found the input invalid or a sum too
+// large (the prefixes need not ascend then).
+template <int GROUPS>
 __global__ void __launch_bounds__(256)
-k_guide_fill(int64_t m, const uint64_t *__restrict__ P, int shift, int32_t *G, int64_t B) {
+k_guide_fill(int64_t m, const uint64_t *__restrict__ ptau, const uint64_t *__restrict__ plam, int64_t gcap,
+             int32_t *gtau, int32_t *glam, const u64 *__restrict__ status) {
+    const uint64_t *P = blockIdx.y ? plam : ptau;
+    int32_t *G = blockIdx.y ? glam : gtau;
+    const uint64_t total = status[blockIdx.y ? ST_L_LO : ST_W_LO];
+    if (status[ST_FLAGS] != 0 || status[ST_M_UPPER] != static_cast<u64>(m) || total == 0) return;
+    const int shift = guide_shift(total, gcap);
+    const int64_t B = static_cast<int64_t>(((total - 1) >> shift) + 1);
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     if (blockIdx.x == 0 && threadIdx.x == 0) G[B] = static_cast<int32_t>(m - 1);
-    for (int64_t g0 = wid * kGuideGroups; g0 * 32 < m; g0 += nw * kGuideGroups) {
-        uint64_t prev[kGuideGroups], cur[kGuideGroups];
+    for (int64_t g0 = wid * GROUPS; g0 * 32 < m; g0 += nw * GROUPS) {
+        uint64_t prev[GROUPS], cur[GROUPS];
 #pragma unroll
-        for (int u = 0; u < kGuideGroups; u++) {
+        for (int u = 0; u < GROUPS; u++) {
             const int64_t j = (g0 + u) * 32 + lane;
             prev[u] = (j >= 1 && j <= m) ? __ldg(P + j - 1) : 0ull;
             cur[u] = j < m ? __ldg(P + j) : 0ull;
@@ -33,7 +48,7 @@ k_guide_fill(int64_t m, const uint64_t *__restrict__ P, int shift, int32_t *G, i
         // bucket numbers are below B + 1 <= 2^31, so after the shift the runs
         // are handled in 32 bits
 #pragma unroll
-        for (int u = 0; u < kGuideGroups; u++) {
+        for (int u = 0; u < GROUPS; u++) {
             const int64_t j = (g0 + u) * 32 + lane;
             uint32_t bstart = 0, len = 0;
             if (j < m && cur[u] != prev[u]) {
@@ -57,31 +72,39 @@ k_guide_fill(int64_t m, const uint64_t *__restrict__ P, int shift, int32_t *G, i
     }
 }
 
-// Hub bitmap rows, one block per (hub, chunk of 2^20 labels): the block sets
+// Hub bitmap rows, a block per (hub, chunk of labels) at a time: the block sets
 // bit x for every neighbour x inside its chunk in shared memory, then writes
 // the chunk out whole (coalesced), so no clearing pass and no global atomics.
-constexpr int kHubThreads = 1024;
-constexpr int64_t kHubChunkWords = 1 << 15;  // 128 KB of shared memory
+// Bound by the rows' bytes (512 MB on R-MAT 20); blocks of 512 with 32 KB, four
+// per SM, so that one writes while another clears or sets bits.
+constexpr int kHubThreads = 512;
+constexpr int64_t kHubChunkWords = 1 << 13;
 
-__global__ void __launch_bounds__(kHubThreads)
-k_hub_rows(int64_t hub_start, int64_t bit_base, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
-           uint32_t *bits, int64_t words, int64_t chunks) {
-    extern __shared__ uint32_t s_row[];
-    const int64_t h = blockIdx.x / chunks, c = blockIdx.x % chunks;
-    const int64_t w0 = c * kHubChunkWords;
-    const int64_t nw = min(kHubChunkWords, words - w0);
-    for (int64_t w = threadIdx.x; w < nw; w += kHubThreads) s_row[w] = 0u;
-    __syncthreads();
-    const int64_t r = hub_start + h;
-    const int64_t o = coff[r], e = coff[r + 1];
-    const int64_t lo = bit_base + w0 * 32, hi = bit_base + (w0 + nw) * 32;  // bit_base % 32 == 0
-    for (int64_t i = o + threadIdx.x; i < e; i += kHubThreads) {
-        const int64_t x = ccol[i];
-        if (x >= lo && x < hi) atomicOr(s_row + ((x - lo) >> 5), 1u << (x & 31));
+__global__ void __launch_bounds__(kHubThreads, 4)
+k_hub_rows(int64_t n, int64_t bit_base, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
+           uint32_t *bits, int64_t words, const u64 *__restrict__ status) {
+    __shared__ __align__(16) uint32_t s_row[kHubChunkWords];
+    const int64_t hubs = static_cast<int64_t>(status[ST_HUBS]);
+    const int64_t chunks = (words + kHubChunkWords - 1) / kHubChunkWords;
+    for (int64_t b = blockIdx.x; b < hubs * chunks; b += gridDim.x) {
+        const int64_t h = b / chunks, w0 = (b % chunks) * kHubChunkWords;
+        const int nw = static_cast<int>(min(kHubChunkWords, words - w0));
+        for (int w = threadIdx.x; w < (nw + 3) / 4; w += kHubThreads)
+            reinterpret_cast<uint4 *>(s_row)[w] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        const int64_t r = n - hubs + h;
+        const int64_t o = ldg_i64(coff + r), e = ldg_i64(coff + r + 1);
+        const int64_t lo = bit_base + w0 * 32;  // bit_base % 32 == 0
+        const uint32_t span = static_cast<uint32_t>(nw) * 32;
+        for (int64_t i = o + threadIdx.x; i < e; i += kHubThreads) {
+            const uint32_t x = static_cast<uint32_t>(ldg_i32(ccol + i) - lo);  // below lo: wraps past the span
+            if (x < span) atomicOr(s_row + (x >> 5), 1u << (x & 31));
+        }
+        __syncthreads();
+        uint32_t *row = bits + h * words + w0;
+        for (int w = threadIdx.x; w < nw; w += kHubThreads) row[w] = s_row[w];
+        __syncthreads();
     }
-    __syncthreads();
-    uint32_t *row = bits + h * words + w0;
-    for (int64_t w = threadIdx.x; w < nw; w += kHubThreads) row[w] = s_row[w];
 }
 
 // Inserts every arc (x -> y) into the table of x with compare-and-swap; the
@@ -129,25 +152,25 @@ k_vtab_build(int64_t n, int64_t nnz, const int64_t *__restrict__ coff, const int
     if (failed) raise_flag(status, F_OVERFLOW);
 }
 
-static int guide_shift(uint64_t W, int64_t gcap) {
-    int s = 0;
-    while (s < 63 && (((W - 1) >> s) + 1) > static_cast<uint64_t>(gcap)) s++;
-    return s;
+int launch_guides(ps_graph *g, cudaStream_t s) {
+    const int64_t m = g->L.m_cap;
+    if (m <= 0) return PS_OK;
+    // one resident wave (the loop strides over the edges)
+    const bool small = m < (int64_t{1} << 22);
+    auto kernel = small ? k_guide_fill<1> : k_guide_fill<kGuideGroups>;
+    const int64_t per_block = 256 * (small ? 1 : kGuideGroups);
+    const int64_t blocks = std::min<int64_t>((m + per_block - 1) / per_block, (int64_t)g->sm_count * 8);
+    kernel<<<dim3((unsigned)blocks, 2), 256, 0, s>>>(m, g->ptau, g->plam, g->L.gcap, g->gtau, g->glam, g->status);
+    PS_LAUNCH_CHECK();
+    return PS_OK;
 }
 
-static int build_guide(ps_graph *g, const uint64_t *P, uint64_t total, int32_t *G, int slot,
-                       int *shift_out, cudaStream_t s) {
-    const int64_t m = g->m;
-    const int shift = guide_shift(total, g->L.gcap);
-    const int64_t B = static_cast<int64_t>(((total - 1) >> shift) + 1);
-    *shift_out = shift;
-    (void)slot;
-    // one resident wave (the loop strides over the edges)
-    int occ = 0;
-    PS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_guide_fill, 256, 0));
-    int64_t blocks = (m + 256 * kGuideGroups - 1) / (256 * kGuideGroups);
-    if (blocks > (int64_t)g->sm_count * (occ > 0 ? occ : 1)) blocks = (int64_t)g->sm_count * (occ > 0 ? occ : 1);
-    k_guide_fill<<<(unsigned)blocks, 256, 0, s>>>(m, P, shift, G, B);
+int launch_hub_rows(ps_graph *g, cudaStream_t s) {
+    const int64_t words = g->L.hub_words, rows = std::min(g->L.hub_cap, g->L.n);
+    if (rows <= 0 || words <= 0) return PS_OK;
+    const int64_t blocks = rows * ((words + kHubChunkWords - 1) / kHubChunkWords);
+    k_hub_rows<<<(unsigned)std::min<int64_t>(blocks, (int64_t)g->sm_count * 4), kHubThreads, 0, s>>>(
+        g->L.n, g->L.hub_bit_base, g->off, g->col, g->hub, words, g->status);
     PS_LAUNCH_CHECK();
     return PS_OK;
 }
@@ -171,16 +194,10 @@ int prefix_graph(ps_graph *g, cudaStream_t s) {
     S.d_max = g->d_max;
     if (flags & F_OVERFLOW) return PS_ERR_OVERFLOW;
 
-    // guide tables (with guides off the table has at most 2 buckets)
-    int tshift = 0, lshift = 0;
-    if (S.W > 0) {
-        int rc = build_guide(g, g->ptau, S.W, g->gtau, 4, &tshift, s);
-        if (rc) return rc;
-    }
-    if (S.Lambda > 0) {
-        int rc = build_guide(g, g->plam, S.Lambda, g->glam, 5, &lshift, s);
-        if (rc) return rc;
-    }
+    // the guide tables (with guides off they have at most 2 buckets) and the
+    // hub rows were queued by the load step
+    const int tshift = S.W > 0 ? guide_shift(S.W, g->L.gcap) : 0;
+    const int lshift = S.Lambda > 0 ? guide_shift(S.Lambda, g->L.gcap) : 0;
     S.tau_shift = tshift;
     S.lambda_shift = lshift;
 
@@ -196,18 +213,8 @@ int prefix_graph(ps_graph *g, cudaStream_t s) {
         }
     }
 
-    // hub bitmaps
     const int64_t hubs = static_cast<int64_t>(g->load_totals[4]);
     S.hubs = hubs;
-    if (hubs > 0) {
-        const int64_t words = g->L.hub_words;
-        const int64_t chunks = (words + kHubChunkWords - 1) / kHubChunkWords;
-        const int smem = static_cast<int>((words < kHubChunkWords ? words : kHubChunkWords) * sizeof(uint32_t));
-        PS_CUDA_TRY(cudaFuncSetAttribute(k_hub_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        k_hub_rows<<<(unsigned)(hubs * chunks), kHubThreads, smem, s>>>(n - hubs, g->L.hub_bit_base, g->off, g->col,
-                                                                        g->hub, words, chunks);
-        PS_LAUNCH_CHECK();
-    }
     // The kernels queued after the load's synchronisation cannot fail on
     // valid state; later calls on `stream` are ordered after them.
 

@@ -27,7 +27,7 @@ constexpr int kSortBlock = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortWarps = kSortBlock / 32;
 constexpr int64_t kSortTile = static_cast<int64_t>(kSortBlock) * kSortItems;
-constexpr int64_t kDirectTiles = 32;
+constexpr int64_t kDirectTiles = 64;
 
 int64_t sort_tiles(int64_t count) { return count > 0 ? (count + kSortTile - 1) / kSortTile : 1; }
 
@@ -40,6 +40,13 @@ __device__ __forceinline__ int64_t live_count(int64_t count, const u64 *dcount) 
     return dcount && static_cast<int64_t>(*dcount) < count ? static_cast<int64_t>(*dcount) : count;
 }
 
+// A pass whose digit is zero in every key leaves the order as it is: with the
+// largest key known on the device only, such passes are launched and skipped
+// (the keys then stay where they are; the sort's user looks there).
+__device__ __forceinline__ bool skip_pass(const u64 *max_key, int shift) {
+    return max_key && shift > 0 && (*max_key >> shift) == 0;
+}
+
 // Digit of (key, value): the key's bits from `shift` on and, with CROSS, the
 // value's lowest bits above them (vshift = the key's bits left of shift).
 template <bool CROSS>
@@ -50,8 +57,9 @@ __device__ __forceinline__ uint32_t digit_of(uint32_t k, uint32_t v, int shift, 
 // Digit counts of every tile: counts[digit * tiles + tile].
 template <bool CROSS>
 __global__ void __launch_bounds__(kSortBlock)
-k_sort_hist(int64_t count, const u64 *dcount, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
+k_sort_hist(int64_t count, const u64 *dcount, const u64 *max_key, const uint32_t *__restrict__ key, const uint32_t *__restrict__ val,
             int shift, int vshift, uint32_t mask, uint32_t *counts, int64_t tiles) {
+    if (skip_pass(max_key, shift)) return;
     count = live_count(count, dcount);
     __shared__ uint32_t s_h[kSortWarps][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -112,11 +120,12 @@ enum { kValRead = 0, kValIota = 1, kValCross = 2 };
 
 template <int BITS, bool DIRECT, int VAL>
 __global__ void __launch_bounds__(kSortBlock, 4)
-k_sort_scatter(int64_t count, const u64 *dcount, const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
+k_sort_scatter(int64_t count, const u64 *dcount, const u64 *max_key, const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
                uint32_t *__restrict__ kout, uint32_t *__restrict__ vout, int shift, int vshift,
                const uint32_t *__restrict__ offsets, int64_t tiles) {
     constexpr uint32_t kMask = (1u << BITS) - 1;
     constexpr bool CROSS = VAL == kValCross;
+    if (skip_pass(max_key, shift)) return;
     count = live_count(count, dcount);
     __shared__ uint32_t s_key[kSortTile];
     __shared__ uint32_t s_val[kSortTile];
@@ -212,10 +221,10 @@ template <int BITS, int VAL>
 static void launch_scatter(const SortPass &p, int64_t tiles, cudaStream_t s) {
     const unsigned blocks = static_cast<unsigned>(tiles);
     if (tiles <= kDirectTiles)
-        k_sort_scatter<BITS, true, VAL><<<blocks, kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, p.vin, p.kout, p.vout,
+        k_sort_scatter<BITS, true, VAL><<<blocks, kSortBlock, 0, s>>>(p.count, p.dcount, p.max_key, p.kin, p.vin, p.kout, p.vout,
                                                                       p.shift, p.vshift, p.counts, tiles);
     else
-        k_sort_scatter<BITS, false, VAL><<<blocks, kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, p.vin, p.kout, p.vout,
+        k_sort_scatter<BITS, false, VAL><<<blocks, kSortBlock, 0, s>>>(p.count, p.dcount, p.max_key, p.kin, p.vin, p.kout, p.vout,
                                                                        p.shift, p.vshift, p.counts, tiles);
 }
 
@@ -233,10 +242,10 @@ int sort_pass(const SortPass &p, const ScanState<uint32_t> &scan, cudaStream_t s
     const int bits = (p.bits + 1) & ~1;  // the keys have no bits above the sort's last digit
     const uint32_t mask = (1u << bits) - 1u;
     if (p.vshift)
-        k_sort_hist<true><<<static_cast<unsigned>(tiles), kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, p.vin, p.shift,
+        k_sort_hist<true><<<static_cast<unsigned>(tiles), kSortBlock, 0, s>>>(p.count, p.dcount, p.max_key, p.kin, p.vin, p.shift,
                                                                               p.vshift, mask, p.counts, tiles);
     else
-        k_sort_hist<false><<<static_cast<unsigned>(tiles), kSortBlock, 0, s>>>(p.count, p.dcount, p.kin, nullptr,
+        k_sort_hist<false><<<static_cast<unsigned>(tiles), kSortBlock, 0, s>>>(p.count, p.dcount, p.max_key, p.kin, nullptr,
                                                                                p.shift, 0, mask, p.counts, tiles);
     PS_LAUNCH_CHECK();
     if (tiles > kDirectTiles) {
