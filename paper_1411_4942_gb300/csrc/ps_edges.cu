@@ -39,13 +39,32 @@ namespace ps {
 // row above.  An asymmetric input can have
 // more lower arcs than the buffers hold; those beyond m_cap are dropped (the
 // status check after the load rejects the graph).
+//
+// The listing also sets the bits of every edge that no hub row holds in the
+// edge filter (one atomic without a result per edge): it streams little else,
+// so the filter stays in L2.  (From the edge-table kernel, which streams 60
+// bytes per edge, the same atomics took 0.96 ms on the 3M-vertex graph.)
+struct EdgeFilter {
+    uint32_t *words;  // null: no filter
+    uint32_t count;
+    int32_t hub_bit_base;
+
+    // The edge u < v, hubs from hub_start up.
+    __device__ __forceinline__ void add(int32_t u, int32_t v, int32_t hub_start) const {
+        if (!words || (v >= hub_start && u >= hub_bit_base)) return;
+        const uint64_t h = edge_hash(u, v);
+        atomicOr(words + filter_word(h, count), filter_mask(h));
+    }
+};
+
 constexpr int kListBatch = 4;
 constexpr int64_t kFewRows = int64_t{1} << 18;
 
 __global__ void __launch_bounds__(256)
 k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
              const int64_t *__restrict__ ubase, uint32_t *__restrict__ key, uint32_t *__restrict__ val,
-             int64_t m_cap, const u64 *__restrict__ status) {
+             int64_t m_cap, const u64 *__restrict__ status, EdgeFilter F) {
+    const int32_t hub_start = static_cast<int32_t>(n - static_cast<int64_t>(status[ST_HUBS]));
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
     const int64_t r_long = static_cast<int64_t>(status[ST_LONG]);
@@ -61,7 +80,7 @@ k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restr
         const int64_t lb0 = __shfl_sync(0xffffffffu, lb, 0);
         for (int64_t t0 = lb0; t0 < lb_end; t0 += 32 * kListBatch) {
             int64_t t[kListBatch], i[kListBatch];
-            int32_t c[kListBatch];
+            int32_t c[kListBatch], row[kListBatch];
 #pragma unroll
             for (int u = 0; u < kListBatch; u++) {
                 t[u] = t0 + 32 * u + lane;
@@ -72,6 +91,7 @@ k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restr
                     const int64_t x = __shfl_sync(0xffffffffu, lb, at + step);
                     if (x <= t[u]) at += step;
                 }
+                row[u] = static_cast<int32_t>(w * 32 + at);
                 i[u] = __shfl_sync(0xffffffffu, o, at) + (t[u] - __shfl_sync(0xffffffffu, lb, at));
             }
 #pragma unroll
@@ -81,6 +101,7 @@ k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restr
                 if (t[u] < lb_end && t[u] < m_cap) {
                     key[t[u]] = static_cast<uint32_t>(c[u]);
                     val[t[u]] = static_cast<uint32_t>(i[u]);
+                    F.add(c[u], row[u], hub_start);
                 }
         }
     }
@@ -92,7 +113,8 @@ __global__ void __launch_bounds__(256)
 k_lower_arcs_mid(const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                  const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase,
                  uint32_t *__restrict__ key, uint32_t *__restrict__ val, int64_t m_cap,
-                 const u64 *__restrict__ status, int first_slot) {
+                 const u64 *__restrict__ status, int first_slot, int64_t n, EdgeFilter F) {
+    const int32_t hub_start = static_cast<int32_t>(n - static_cast<int64_t>(status[ST_HUBS]));
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
     const int64_t r_end = static_cast<int64_t>(status[ST_TIER + 3]);
@@ -125,6 +147,7 @@ k_lower_arcs_mid(const int64_t *__restrict__ coff, const int32_t *__restrict__ c
                 if (p < low && lb + p < m_cap) {
                     key[lb + p] = static_cast<uint32_t>(c[u]);
                     val[lb + p] = static_cast<uint32_t>(o + p);
+                    F.add(c[u], static_cast<int32_t>(r), hub_start);
                 }
             }
         }
@@ -136,7 +159,8 @@ __global__ void __launch_bounds__(256)
 k_lower_arcs_long(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                   const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase,
                   uint32_t *__restrict__ key, uint32_t *__restrict__ val, int64_t m_cap,
-                  const u64 *__restrict__ status) {
+                  const u64 *__restrict__ status, EdgeFilter F) {
+    const int32_t hub_start = static_cast<int32_t>(n - static_cast<int64_t>(status[ST_HUBS]));
     const int64_t r0 = static_cast<int64_t>(status[ST_TIER + 3]);
     for (int64_t r = r0 + blockIdx.x; r < n; r += gridDim.x) {
         const int64_t o = ldg_i64(coff + r), low = ldg_i32(lowcnt + r);
@@ -154,6 +178,7 @@ k_lower_arcs_long(int64_t n, const int64_t *__restrict__ coff, const int32_t *__
                 if (p < low && lb + p < m_cap) {
                     key[lb + p] = static_cast<uint32_t>(c[u]);
                     val[lb + p] = static_cast<uint32_t>(o + p);
+                    F.add(c[u], static_cast<int32_t>(r), hub_start);
                 }
             }
         }
@@ -168,22 +193,13 @@ k_lower_arcs_long(int64_t n, const int64_t *__restrict__ coff, const int32_t *__
 // thread builds Q edges at j0, j0 + step, ..., their loads issued together
 // stage by stage (the chain sorted entry -> row of u -> v -> row of v is
 // otherwise a string of dependent round trips per edge), and returns their
-// weights (zero past m or for a bad edge).  With an edge filter, every edge
-// that no hub row holds also sets its bits there (one atomic without a
-// result per edge).
-struct EdgeFilter {
-    uint32_t *words;  // null: no filter
-    uint32_t count;
-    int32_t hub_bit_base;
-};
-
+// weights (zero past m or for a bad edge).
 template <int Q>
 __device__ __forceinline__ void edge_group(int64_t j0, int step, int64_t m, int64_t n,
                                            const uint32_t *__restrict__ skey, const uint32_t *__restrict__ sval,
                                            const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                                            const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase,
-                                           EdgeRec *rec, const EdgeFilter &F, int32_t hub_start, U64x2 (&w)[Q],
-                                           bool &asym) {
+                                           EdgeRec *rec, U64x2 (&w)[Q], bool &asym) {
     // every offset, label and degree is below 2^31 (nnz < 2^31), so the
     // stages work in 32 bits
     int32_t u[Q], i[Q], ou[Q], du[Q], iu[Q], v[Q], ov[Q], dv[Q];
@@ -228,10 +244,6 @@ __device__ __forceinline__ void edge_group(int64_t j0, int step, int64_t m, int6
         e[0] = make_int4(u[q], v[q], du[q], dv[q]);
         e[1] = make_int4(iu[q], jv, ou[q], ov[q]);
         w[q] = edge_weights(du[q], dv[q], iu[q], jv);
-        if (F.words && !(v[q] >= hub_start && u[q] >= F.hub_bit_base)) {
-            const uint64_t h = edge_hash(u[q], v[q]);
-            atomicOr(F.words + filter_word(h, F.count), filter_mask(h));
-        }
     }
 }
 
@@ -253,16 +265,15 @@ __global__ void __launch_bounds__(kScanBlock, 4)
 k_edge_records_scan(int64_t m, int64_t n, const uint32_t *__restrict__ skey, const uint32_t *__restrict__ sval,
                     const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                     const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase, EdgeRec *rec,
-                    u64 *status, EdgeFilter F, ScanState<U64x2> st, uint64_t *ptau, uint64_t *plam) {
+                    u64 *status, ScanState<U64x2> st, uint64_t *ptau, uint64_t *plam) {
     __shared__ U64x2 s_w[kRecScanItems * kScanBlock];
     const int64_t tile = scan_ticket(st);
     const int64_t wbase = scan_wbase<kScanBlock, kRecScanItems>(tile);
     bool asym = false;
-    const int32_t hub_start = static_cast<int32_t>(n - static_cast<int64_t>(status[ST_HUBS]));
 #pragma unroll
     for (int g0 = 0; g0 < kRecScanItems; g0 += kRecItems) {
         U64x2 w[kRecItems];
-        edge_group<kRecItems>(wbase + 32 * g0, 32, m, n, skey, sval, coff, ccol, lowcnt, ubase, rec, F, hub_start, w, asym);
+        edge_group<kRecItems>(wbase + 32 * g0, 32, m, n, skey, sval, coff, ccol, lowcnt, ubase, rec, w, asym);
 #pragma unroll
         for (int q = 0; q < kRecItems; q++) s_w[(g0 + q) * kScanBlock + threadIdx.x] = w[q];
     }
@@ -291,6 +302,7 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
     int bits = 0;
     while (bits < 31 && (static_cast<uint64_t>(n > 0 ? n - 1 : 0) >> bits) != 0) bits++;
     const int passes = bits > 0 ? (bits + 7) / 8 : 1;
+    const EdgeFilter F{g->filt, static_cast<uint32_t>(L.filt_words), static_cast<int32_t>(L.hub_bit_base)};
     if (n > 0) {
         // few rows: a warp each for the short ones too (5,000 rows: 16 -> 4 us;
         // 32 short rows are up to 32 steps for one warp)
@@ -298,17 +310,17 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
         if (!few) {
             int64_t blocks = (n + 255) / 256;  // a warp per 32 rows
             if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-            k_lower_arcs<<<(unsigned)blocks, 256, 0, s>>>(n, g->off, g->col, g->ubase, ka, va, m, g->status);
+            k_lower_arcs<<<(unsigned)blocks, 256, 0, s>>>(n, g->off, g->col, g->ubase, ka, va, m, g->status, F);
             PS_LAUNCH_CHECK();
         }
         if (few || g->d_max > kLongRow) {
             k_lower_arcs_mid<<<(unsigned)(sms * (few ? 8 : 6)), 256, 0, s>>>(g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
-                                                                             g->status, few ? ST_TIER : ST_LONG);
+                                                                             g->status, few ? ST_TIER : ST_LONG, n, F);
             PS_LAUNCH_CHECK();
         }
         if (g->d_max > kTierC) {
             k_lower_arcs_long<<<(unsigned)(sms * 4), 256, 0, s>>>(n, g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
-                                                                   g->status);
+                                                                   g->status, F);
             PS_LAUNCH_CHECK();
         }
     }
@@ -328,13 +340,12 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
         va = vo;
     }
     // ka/va: the sorted list, in the G_tau region
-    const EdgeFilter F{g->filt, static_cast<uint32_t>(L.filt_words), static_cast<int32_t>(L.hub_bit_base)};
     const int64_t stiles = (m + kScanBlock * kRecScanItems - 1) / (kScanBlock * kRecScanItems);
     ScanState<U64x2> scan;
     const int rc = take_scan(g, stiles, &scan);
     if (rc) return rc;
     k_edge_records_scan<<<(unsigned)stiles, kScanBlock, 0, s>>>(
-        m, n, ka, va, g->off, g->col, g->lowcnt, g->ubase, g->rec, g->status, F,
+        m, n, ka, va, g->off, g->col, g->lowcnt, g->ubase, g->rec, g->status,
         scan, g->ptau, g->plam);
     PS_LAUNCH_CHECK();
     return PS_OK;

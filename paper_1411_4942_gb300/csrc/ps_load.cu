@@ -61,8 +61,8 @@ __global__ void __launch_bounds__(256) k_check_columns(int64_t n, int64_t nnz, c
 __global__ void __launch_bounds__(256)
 k_rank(int64_t n, int bits, const uint32_t *__restrict__ k0, const uint32_t *__restrict__ v0,
        const uint32_t *__restrict__ k1, const uint32_t *__restrict__ v1, int32_t *rank, uint32_t *inv, int32_t *dnew,
-       int32_t *lowcnt, int64_t hub_cap, int64_t hub_min, u64 *status) {
-    const uint32_t lim[5] = {0, kTierA, kTierB, kTierC, kLongRow};
+       int32_t *lowcnt, uint32_t tier_b_end, int64_t hub_cap, int64_t hub_min, u64 *status) {
+    const uint32_t lim[5] = {0, kTierA, tier_b_end, kTierC, kLongRow};
     const int slot[5] = {ST_TIER, ST_TIER + 1, ST_TIER + 2, ST_TIER + 3, ST_LONG};
     bool second = true;  // the first pass moves the pairs to the second buffers, and so on
     for (int shift = 8; shift < bits && (status[ST_DMAX] >> shift) != 0; shift += 8) second = !second;
@@ -257,7 +257,7 @@ __device__ __forceinline__ void sort_row_warp(const RowIn &R, int64_t r, uint32_
     if (lane == 0) R.lowcnt[r] = low;
 }
 
-// Tier B: rows of 33..1024 entries, one warp, bitonic network in registers,
+// Tier B: rows of 33..1024 (or 512, tier_b) entries, one warp, bitonic network in registers,
 // in two kernels: rows up to kLongRow entries (two or four keys per lane)
 // at 32 registers and full occupancy, the longer ones capped at 64
 // registers (four blocks per SM beat the spill-free 105-register build; the
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(256, 4) k_sort_tier_b2(RowIn R) {
     report(R, bad, nsimple);
 }
 
-// Tier C: rows of 1025..4096 entries, one block of 512, bitonic network in
+// Tier C: rows from there to 4096 entries, one block of 512, bitonic network in
 // registers with the cross-warp stages in shared memory (16 KB, several
 // blocks per SM).
 template <int E>
@@ -786,7 +786,8 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     }
     uint32_t *inv = reinterpret_cast<uint32_t *>(ws + L.inv);
     if (n > 0) {
-        k_rank<<<sms * 8, 256, 0, s>>>(n, bits, k0, v0, k1, v1, g->rank, inv, g->dnew, g->lowcnt, L.hub_cap,
+        k_rank<<<sms * 8, 256, 0, s>>>(n, bits, k0, v0, k1, v1, g->rank, inv, g->dnew, g->lowcnt,
+                                       static_cast<uint32_t>(tier_b(nnz)), L.hub_cap,
                                        g->tune.hub_min_degree, g->status);
         PS_LAUNCH_CHECK();
     } else {
@@ -821,7 +822,7 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     RowIn R{d_off, d_col, inv, g->rank, g->off, g->col, g->lowcnt, n, g->status};
     if (n > 0) {
         SideFork fork(g, s);
-        if (g->d_max > kTierB) {
+        if (g->d_max > tier_b(nnz)) {
             rc = fork.fork(2);
             if (rc) return rc;
         }
@@ -841,7 +842,7 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
             k_sort_tier_d<<<sms * 2, 1024, 0, fork.side(1)>>>(R, reinterpret_cast<int32_t *>(g->rec), vb);
             PS_LAUNCH_CHECK();
         }
-        if (g->d_max > kTierB) {
+        if (g->d_max > tier_b(nnz)) {
             k_sort_tier_c<<<sms * 3, 512, 0, fork.side(0)>>>(R);
             PS_LAUNCH_CHECK();
         }
