@@ -19,7 +19,7 @@
 // and puts the ids into up to kOrderBuckets buckets of a fixed capacity (8
 // standard deviations above the mean), reserving room tile by tile, with no
 // counting pass before it.  The second sorts every bucket by the next
-// 11 or 12 bits in one block's shared memory and writes the ids out densely.
+// kLocalBits bits in one block's shared memory and writes the ids out densely.
 // Should a bucket ever run over, the sampling kernel takes the ids in their
 // own order instead.
 //
@@ -35,18 +35,20 @@
 namespace ps {
 
 constexpr int kOrderBuckets = 4096;              // of the first kernel, at most
-// Buckets of the second kernel: a block of 1024 with 34 ids per thread for
-// means of 2^14 to 2^15 ids, or, for chunks that would leave SMs without a
-// bucket, a block of 512 with 18 per thread for means of 2^12 to 2^13.
-constexpr int kLargeThreads = 1024, kLargeItems = 34, kLargeMeanBits = 15;
-constexpr int kSmallThreads = 512, kSmallItems = 18, kSmallMeanBits = 13;
-constexpr uint64_t kLargeFrom = 1u << 22;        // ids per chunk
-constexpr uint64_t kOrderMaxSorted = static_cast<uint64_t>(kOrderBuckets) << kLargeMeanBits;  // ids sorted at once
+// A bucket is one block of the second kernel: 1024 threads with up to 34 ids
+// each.  (Smaller buckets for short chunks, a block of 512 with 18 each, left
+// fewer SMs idle but cost the first kernel more: 3M ids 179 / 169 against 172 /
+// 162 us on a 10M-edge graph.)
+constexpr int kLocalThreads = 1024;
+constexpr int kLocalItems = 34;
+constexpr int kLocalBits = 12;                   // four counters per thread
+constexpr int kMeanBits = 15;                    // ids per bucket: 2^14 to 2^15 on average
+constexpr uint64_t kOrderMaxSorted = static_cast<uint64_t>(kOrderBuckets) << kMeanBits;  // ids sorted at once
 constexpr int kOrderItems = 16;                  // ids per thread and tile of the first kernel
 constexpr int kCursorStride = 8;                 // cursors in sectors of their own
 // Scratch: the cursors and the overflow flag in a header, then per sample of a
 // chunk its id (uint32) in the final order, and per place of the buckets an id
-// (uint32) and its key's next bits (uint16): at most 10.9 bytes per sample.
+// (uint32) and its key's next bits (uint16): at most 10.4 bytes per sample.
 constexpr size_t kOrderHeader = (1u << 20) + 1024;
 constexpr size_t kOrderPerSample = 11;
 static_assert((kOrderBuckets * kCursorStride + 1) * sizeof(uint32_t) <= kOrderHeader, "cursors and flag");
@@ -56,7 +58,7 @@ static_assert((kOrderBuckets * kCursorStride + 1) * sizeof(uint32_t) <= kOrderHe
 // against plain, 3-path / centred (Chung-Lu; R-MAT crosses a little earlier):
 //   2.5M edges: 2^23 ids 285 / 272 against 287 / 266 us;
 //   5M edges: 2^21 ids 121 / 115 against 113 / 107, 2^22 184 / 174 against 204 / 192;
-//   10M edges: 2^20 ids 92 / 93 against 80 / 79, 2^21 138 / 138 against 143 / 137;
+//   10M edges: 2^20 ids 101 / 102 against 83 / 82, 2^21 138 / 137 against 150 / 153;
 //   40M edges: 2^20 ids 120 / 117 against 116 / 113, 2^24 971 / 777 against 1493 / 1506.
 constexpr int64_t kOrderMinEdges = 1ll << 22;
 static uint64_t order_min_chunk(int64_t m) { return m >= (1ll << 23) ? 1ull << 21 : 1ull << 22; }
@@ -66,12 +68,10 @@ static uint64_t order_min_chunk(int64_t m) { return m >= (1ll << 23) ? 1ull << 2
 struct OrderPlan {
     int bits;          // log2 of the buckets
     uint32_t room;     // ids per bucket
-    bool large;        // which second kernel
 };
 static OrderPlan order_plan(uint64_t kk) {
-    OrderPlan p{0, static_cast<uint32_t>(kk), kk >= kLargeFrom};
-    const int mean_bits = p.large ? kLargeMeanBits : kSmallMeanBits;
-    while (((kk - 1) >> mean_bits) >> p.bits) p.bits++;
+    OrderPlan p{0, static_cast<uint32_t>(kk)};
+    while (((kk - 1) >> kMeanBits) >> p.bits) p.bits++;
     if (p.bits) {
         const uint32_t mean = static_cast<uint32_t>((kk >> p.bits) + 1);
         uint32_t root = 1;
@@ -188,44 +188,40 @@ k_order_partition(uint64_t kk, uint64_t seed, uint64_t first_id, int bits, uint3
     }
 }
 
-// The second kernel, a block per bucket: its ids by the next bits (11 or 12,
-// four counters per thread), behind the ids of the buckets before it.
-template <int THREADS, int ITEMS>
+// The second kernel, a block per bucket: its ids by the next kLocalBits bits,
+// behind the ids of the buckets before it.
 struct LocalSmem {
-    uint32_t id[THREADS * ITEMS];
-    uint32_t cnt[4 * THREADS];
+    uint32_t id[kLocalThreads * kLocalItems];
+    uint32_t cnt[1 << kLocalBits];
     uint32_t warp[32];
 };
+static_assert((1 << kLocalBits) == 4 * kLocalThreads, "four counters per thread");
 
-template <int THREADS, int ITEMS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+__global__ void __launch_bounds__(kLocalThreads, 1)
 k_order_local(uint32_t room, const uint32_t *__restrict__ cursor, const uint32_t *__restrict__ spilled,
               const uint32_t *__restrict__ ids, const uint16_t *__restrict__ keys, uint32_t *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    using Smem = LocalSmem<THREADS, ITEMS>;
-    Smem &S = *reinterpret_cast<Smem *>(s_raw);
-    constexpr int kDown = THREADS == 1024 ? 4 : 5;  // of the 16 key bits, those not sorted by
-    static_assert((1 << (16 - kDown)) == 4 * THREADS, "four counters per thread");
+    LocalSmem &S = *reinterpret_cast<LocalSmem *>(s_raw);
     if (*spilled) return;
     const int t = threadIdx.x;
     const uint32_t n = __ldg(cursor + blockIdx.x * kCursorStride);  // at most room
     ids += static_cast<size_t>(blockIdx.x) * room;
     keys += static_cast<size_t>(blockIdx.x) * room;
 #pragma unroll
-    for (int q = 0; q < 4; q++) S.cnt[q * THREADS + t] = 0;
+    for (int q = 0; q < 4; q++) S.cnt[q * kLocalThreads + t] = 0;
     // ids in the buckets before this one
     uint32_t before = 0;
-    for (uint32_t b = t; b < blockIdx.x; b += THREADS) before += __ldg(cursor + b * kCursorStride);
+    for (uint32_t b = t; b < blockIdx.x; b += kLocalThreads) before += __ldg(cursor + b * kCursorStride);
     __syncthreads();
-    uint32_t place[ITEMS];  // key << 16 | rank among the bucket's ids of that key
+    uint32_t place[kLocalItems];  // key << 16 | rank among the bucket's ids of that key
 #pragma unroll
-    for (int i = 0; i < ITEMS; i++) {
-        const uint32_t q = i * THREADS + t;
-        place[i] = q < n ? static_cast<uint32_t>(__ldg(keys + q)) >> kDown : 0u;
+    for (int i = 0; i < kLocalItems; i++) {
+        const uint32_t q = i * kLocalThreads + t;
+        place[i] = q < n ? static_cast<uint32_t>(__ldg(keys + q)) >> (16 - kLocalBits) : 0u;
     }
 #pragma unroll
-    for (int i = 0; i < ITEMS; i++)
-        if (i * THREADS + t < n) place[i] = place[i] << 16 | atomicAdd(&S.cnt[place[i]], 1u);
+    for (int i = 0; i < kLocalItems; i++)
+        if (i * kLocalThreads + t < n) place[i] = place[i] << 16 | atomicAdd(&S.cnt[place[i]], 1u);
     before = __reduce_add_sync(0xffffffffu, before);
     __syncthreads();
     uint32_t c[4], sum = 0;
@@ -234,7 +230,7 @@ k_order_local(uint32_t room, const uint32_t *__restrict__ cursor, const uint32_t
         c[q] = S.cnt[4 * t + q];
         sum += c[q];
     }
-    uint32_t run = block_excl_sum<THREADS>(sum, S.warp);
+    uint32_t run = block_excl_sum<kLocalThreads>(sum, S.warp);
 #pragma unroll
     for (int q = 0; q < 4; q++) {
         S.cnt[4 * t + q] = run;
@@ -243,13 +239,13 @@ k_order_local(uint32_t room, const uint32_t *__restrict__ cursor, const uint32_t
     __syncthreads();
     if ((t & 31) == 0) S.warp[t >> 5] = before;
 #pragma unroll
-    for (int i = 0; i < ITEMS; i++) {
-        const uint32_t q = i * THREADS + t;
+    for (int i = 0; i < kLocalItems; i++) {
+        const uint32_t q = i * kLocalThreads + t;
         if (q < n) S.id[S.cnt[place[i] >> 16] + (place[i] & 0xffffu)] = __ldg(ids + q);
     }
     __syncthreads();
-    out += __reduce_add_sync(0xffffffffu, (t & 31) < THREADS / 32 ? S.warp[t & 31] : 0u);
-    for (uint32_t p = t; p < n; p += THREADS) out[p] = S.id[p];
+    out += __reduce_add_sync(0xffffffffu, S.warp[t & 31]);
+    for (uint32_t p = t; p < n; p += kLocalThreads) out[p] = S.id[p];
 }
 
 template <int SAMPLER, int BLOCK, int ADJ>
@@ -280,16 +276,6 @@ static int launch_partition(const ps_graph *g, uint64_t kk, uint64_t seed, uint6
     return PS_OK;
 }
 
-template <int THREADS, int ITEMS>
-static int launch_local(const OrderPlan &plan, const uint32_t *cursor, const uint32_t *spilled, const uint32_t *ids,
-                        const uint16_t *keys, uint32_t *sorted, cudaStream_t s) {
-    const int smem = static_cast<int>(sizeof(LocalSmem<THREADS, ITEMS>));
-    PS_CUDA_TRY(cudaFuncSetAttribute(k_order_local<THREADS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_order_local<THREADS, ITEMS><<<1u << plan.bits, THREADS, smem, s>>>(plan.room, cursor, spilled, ids, keys, sorted);
-    PS_LAUNCH_CHECK();
-    return PS_OK;
-}
-
 template <int SAMPLER, int BLOCK, int ADJ>
 static int ordered_t(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t first_id, uint64_t *hist,
                      char *scratch, uint64_t chunk, cudaStream_t s) {
@@ -316,18 +302,15 @@ static int ordered_t(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t firs
             uint16_t *keys = reinterpret_cast<uint16_t *>(ids + places);
             PS_CUDA_TRY(cudaMemsetAsync(cursor, 0, (kOrderBuckets * kCursorStride + 1) * sizeof(uint32_t), s));
             int rc;
-            // smaller blocks with smaller tiles overlap their phases and fill
-            // the SMs on short chunks; with many buckets, longer tiles keep a
-            // bucket's runs from getting too short
-            if (!plan.large) {
-                rc = launch_partition<SAMPLER, 256>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
-                if (!rc) rc = launch_local<kSmallThreads, kSmallItems>(plan, cursor, spilled, ids, keys, sorted, s);
-            } else {
-                if (plan.bits <= 11) rc = launch_partition<SAMPLER, 512>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
-                else rc = launch_partition<SAMPLER, 1024>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
-                if (!rc) rc = launch_local<kLargeThreads, kLargeItems>(plan, cursor, spilled, ids, keys, sorted, s);
-            }
+            // up to 2048 buckets two smaller blocks per SM overlap their phases;
+            // above, longer tiles keep the runs of a bucket from getting too short
+            if (plan.bits <= 11) rc = launch_partition<SAMPLER, 512>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
+            else rc = launch_partition<SAMPLER, 1024>(g, kk, seed, first_id, plan, cursor, spilled, ids, keys, s);
             if (rc) return rc;
+            const int smem = static_cast<int>(sizeof(LocalSmem));
+            PS_CUDA_TRY(cudaFuncSetAttribute(k_order_local, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            k_order_local<<<1u << plan.bits, kLocalThreads, smem, s>>>(plan.room, cursor, spilled, ids, keys, sorted);
+            PS_LAUNCH_CHECK();
             uint64_t blocks = (kk + BLOCK - 1) / BLOCK;
             if (blocks > full) blocks = full;
             k_sample_ordered<SAMPLER, BLOCK, ADJ><<<(unsigned)blocks, BLOCK, 0, s>>>(g->dev, kk, seed, first_id, sorted,

@@ -1,5 +1,5 @@
 """The draw order at the sizes where its plan changes: one bucket and two, a
-bucket just full and one id more, both bucket sizes, more ids than are sorted
+bucket just full and one id more, both tile lengths, more ids than are sorted
 at once; with a scratch of exactly the documented size, whose surroundings must
 stay untouched."""
 import pytest
@@ -21,8 +21,10 @@ def graph():
 
 
 @pytest.mark.parametrize("k, chunk", [(1, 1), (31, 31), (8191, 8191), (8192, 8192), (8193, 8193), (16385, 16385),
+                                      (32768, 32768), (32769, 32769), (65537, 65537),
                                       (100_003, 100_003), ((1 << 22) - 1, (1 << 22) - 1), (1 << 22, 1 << 22),
                                       ((1 << 22) + 1, (1 << 22) + 1), (10_000_019, 10_000_019), (50_000, 8193),
+                                      (100_000, 32769),
                                       ((1 << 26) + 77, (1 << 26) + 77), ((1 << 27) + 5, (1 << 27) + 5)])
 def test_plan_edges(graph, k, chunk):
     nbytes = ps.ps_ordered_scratch_bytes(chunk)
