@@ -14,7 +14,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_NAME = "libpathsample.so"
 LIB_PATH = os.path.join(PKG, LIB_NAME)
-SOURCES = ["ps_load.cu", "ps_sort.cu", "ps_prefix.cu", "ps_sample.cu", "ps_batch.cu", "ps_api.cu", "ps_static.cu", "ps_exact.cu", "ps_ingest.cu", "ps_order.cu", "ps_edges.cu", "ps_probe.cu"]
+SOURCES = ["ps_load.cu", "ps_sort.cu", "ps_prefix.cu", "ps_sample.cu", "ps_batch.cu", "ps_api.cu", "ps_static.cu", "ps_exact.cu", "ps_ingest.cu", "ps_order.cu", "ps_edges.cu", "ps_probe.cu", "ps_readback.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host FP64 (the estimates and bars) without fused multiply-adds: on Arm the
 # compiler would pick them by inlining, and the last bit of a bar with them

@@ -521,14 +521,17 @@ int ps_count_adaptive(const ps_graph *g, uint64_t seed, double target, double de
     const double delta_look = delta / static_cast<double>(adaptive_looks(k0, k_max));
     uint64_t done = 0, k = k0;
     int rc = PS_OK;
+    Readback back;
     while (true) {
         const uint64_t add = k - done;
         if (g->stats.W > 0) rc = launch_sampler(g, 0, add, seed, done, d_hist6, s);
         if (rc == PS_OK && g->stats.Lambda > 0) rc = launch_sampler(g, 1, add, seed, done, d_hist4, s);
         if (rc != PS_OK) return rc;
-        PS_CUDA_TRY(cudaMemcpyAsync(hist6, d_hist6, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-        PS_CUDA_TRY(cudaMemcpyAsync(hist4, d_hist4, 4 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+        rc = back.queue(d_hist6, 6, d_hist4, 4, s);
+        if (rc != PS_OK) return rc;
         PS_CUDA_TRY(cudaStreamSynchronize(s));
+        std::memcpy(hist6, back.words, 6 * sizeof(uint64_t));
+        std::memcpy(hist4, back.words + 6, 4 * sizeof(uint64_t));
         done = k;
         rc = ps_estimate_ex(&g->stats, hist6, k, hist4, k, delta_look, flags, est, lo, hi);
         if (rc != PS_OK && rc != PS_NO_PATHS) return rc;
@@ -648,11 +651,13 @@ int ps_count_motifs_host(int64_t n, int64_t nnz, const int64_t *h_off, const int
         ps_graph_free(g);
         return rc;
     }
-    uint64_t h[16];
-    const cudaError_t e1 = cudaMemcpyAsync(h, d_hist, sizeof(h), cudaMemcpyDeviceToHost, s);
-    const cudaError_t e2 = cudaStreamSynchronize(s);
+    Readback back;
+    rc = back.queue(d_hist, 16, nullptr, 0, s);
+    const cudaError_t e = cudaStreamSynchronize(s);
     ps_graph_free(g);
-    if (e1 != cudaSuccess || e2 != cudaSuccess) return PS_ERR_CUDA;
+    if (rc != PS_OK) return rc;
+    if (e != cudaSuccess) return PS_ERR_CUDA;
+    const uint64_t *h = back.words;
     if (hist6) std::memcpy(hist6, h, 6 * sizeof(uint64_t));
     if (hist4) std::memcpy(hist4, h + 8, 4 * sizeof(uint64_t));
     if (stats) *stats = st;

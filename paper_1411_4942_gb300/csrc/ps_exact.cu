@@ -643,9 +643,12 @@ extern "C" int ps_count_exact(const ps_graph *g, void *d_scratch, size_t scratch
             PS_LAUNCH_CHECK();
         }
     }
-    uint64_t h[XA_WORDS];
-    PS_CUDA_TRY(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
+    static_assert(XA_WORDS <= Readback::kWords, "the words fit a read-back");
+    Readback r;
+    const int rc = r.queue(acc, XA_WORDS, nullptr, 0, s);
+    if (rc) return rc;
     PS_CUDA_TRY(cudaStreamSynchronize(s));
+    const uint64_t *h = r.words;
     auto pair = [&](int w) { return (static_cast<u128>(h[w + 1]) << 64) | h[w]; };
     const ps_stats &S = g->stats;
     const u128 T3 = pair(XA_T3);

@@ -262,9 +262,12 @@ extern "C" int ps_csr_from_edges(int64_t n, int64_t n_edges, const int32_t *d_sr
     } else {
         PS_CUDA_TRY(cudaMemsetAsync(d_off, 0, static_cast<size_t>(n + 1) * sizeof(int64_t), s));
     }
-    uint64_t st[IS_WORDS];
-    PS_CUDA_TRY(cudaMemcpyAsync(st, status, sizeof(st), cudaMemcpyDeviceToHost, s));
+    static_assert(IS_WORDS <= Readback::kWords, "the words fit a read-back");
+    Readback r;
+    const int rc = r.queue(status, IS_WORDS, nullptr, 0, s);
+    if (rc) return rc;
     PS_CUDA_TRY(cudaStreamSynchronize(s));
+    const uint64_t *st = r.words;
     const int status_code = flags_to_status(st[IS_FLAGS]);
     if (status_code != PS_OK) return status_code;
     *nnz = 2 * static_cast<int64_t>(st[IS_PAIRS]);

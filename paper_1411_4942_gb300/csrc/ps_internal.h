@@ -113,6 +113,31 @@ int flags_to_status(uint64_t flags);
 // their own events, so concurrent calls stay ordered correctly).
 int get_side_streams(int device, cudaStream_t out[2]);
 
+// Id of the context current on this thread; 0 when there is none or the
+// driver cannot say.  (Unlike context handles, ids are never reused.)
+unsigned long long current_context_id();
+
+// Device words brought to the host (ps_readback.cu): `words` holds them once
+// the stream they were queued on has been synchronised, which the caller does
+// before this object ends.
+class Readback {
+  public:
+    static constexpr int kWords = 64;
+    Readback();
+    ~Readback();
+    Readback(const Readback &) = delete;
+    Readback &operator=(const Readback &) = delete;
+    // words[0, na) = a[0, na), words[na, na + nb) = b[0, nb) (device, 8-byte words)
+    int queue(const void *a, int na, const void *b, int nb, cudaStream_t s);
+
+  private:
+    uint64_t own_[kWords];
+    int dev_ = -1, slot_ = -1, generation_ = 0;
+
+  public:
+    uint64_t *words = own_;
+};
+
 // Every kernel launch is followed by this: counts the launch (reported by
 // ps_kernel_launches) and checks the launch error.
 void count_launch();

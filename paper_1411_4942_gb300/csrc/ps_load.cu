@@ -799,9 +799,12 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
 
     // the offsets' verdict and the largest degree, read on the side while the
     // sort runs
-    uint64_t st[ST_WORDS];
-    PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, read.side(0)));
+    static_assert(ST_WORDS <= Readback::kWords, "the words fit a read-back");
+    Readback back;
+    rc = back.queue(g->status, ST_WORDS, nullptr, 0, read.side(0));
+    if (rc) return rc;
     PS_CUDA_TRY(cudaStreamSynchronize(read.side(0)));
+    const uint64_t *st = back.words;
     rc = read.join();
     if (rc) return rc;
     g->d_max = static_cast<int64_t>(st[ST_DMAX]);
@@ -812,7 +815,8 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
             k_check_columns<<<sms * 8, 256, 0, s>>>(n, nnz, d_col, g->status);
             PS_LAUNCH_CHECK();
         }
-        PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));
+        rc = back.queue(g->status, ST_WORDS, nullptr, 0, s);
+        if (rc) return rc;
         PS_CUDA_TRY(cudaStreamSynchronize(s));
         return flags_to_status(st[ST_FLAGS] | F_NOT_SIMPLE);
     }
@@ -878,7 +882,8 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     rc = hubs.join();
     if (rc) return rc;
 
-    PS_CUDA_TRY(cudaMemcpyAsync(st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s));
+    rc = back.queue(g->status, ST_WORDS, nullptr, 0, s);
+    if (rc) return rc;
     PS_CUDA_TRY(cudaStreamSynchronize(s));
     g->load_totals[0] = st[ST_W_LO];
     g->load_totals[1] = st[ST_L_LO];

@@ -3,8 +3,6 @@
 // prefixes) for callers that cannot allocate device memory.  Its scratch --
 // the scan's tile slots and tile counter -- lives in one
 // fixed-size array in this file instead of a caller's workspace.
-#include <cuda.h>
-
 #include <mutex>
 
 #include "ps_internal.h"
@@ -34,33 +32,6 @@ struct ScratchAddr {
     void *ptr;
 };
 ScratchAddr g_scratch_addr[kMaxDevices] = {};
-
-typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long *);
-
-// Id of the context current on this thread; 0 when there is none or the
-// driver cannot say (the address is then looked up again).
-unsigned long long current_context_id() {
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess && q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<CtxGetCurrentFn>(f);
-        f = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<CtxGetIdFn>(f);
-    });
-    CUcontext ctx = nullptr;
-    unsigned long long id = 0;
-    if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx) return 0;
-    if (get_id(ctx, &id) != CUDA_SUCCESS) return 0;
-    return id;
-}
 
 // Device address of the array on the current device (the host-side name is
 // only a stand-in for it).
