@@ -324,25 +324,25 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
             PS_LAUNCH_CHECK();
         }
     }
+    SortPass sort[kMaxPasses];
     for (int pass = 0; pass < passes; pass++) {
         const int shift = 8 * pass;
         const bool last = pass == passes - 1;
         uint32_t *ko = last ? kg : kb, *vo = last ? vg : vb;
-        ScanState<uint32_t> scan{};
-        int rc = sort_scan_tiles(m) ? take_scan(g, sort_scan_tiles(m), &scan) : PS_OK;
-        if (rc) return rc;
-        rc = sort_pass({m, nullptr, ka, va, ko, vo, shift, std::max(1, std::min(8, bits - shift)), 0,
-                        reinterpret_cast<uint32_t *>(ws + L.counts)}, scan, s);
-        if (rc) return rc;
+        sort[pass] = {m, nullptr, ka, va, ko, vo, shift, std::max(1, std::min(8, bits - shift)), 0,
+                      reinterpret_cast<uint32_t *>(ws + L.counts)};
         kb = ka;
         vb = va;
         ka = ko;
         va = vo;
     }
+    auto take = [g](int64_t tiles, ScanState<uint32_t> *scan) { return take_scan(g, tiles, scan); };
+    int rc = sort_passes(sort, passes, take, s);
+    if (rc) return rc;
     // ka/va: the sorted list, in the G_tau region
     const int64_t stiles = (m + kScanBlock * kRecScanItems - 1) / (kScanBlock * kRecScanItems);
     ScanState<U64x2> scan;
-    const int rc = take_scan(g, stiles, &scan);
+    rc = take_scan(g, stiles, &scan);
     if (rc) return rc;
     k_edge_records_scan<<<(unsigned)stiles, kScanBlock, 0, s>>>(
         m, n, ka, va, g->off, g->col, g->lowcnt, g->ubase, g->rec, g->status,

@@ -215,24 +215,22 @@ extern "C" int ps_csr_from_edges(int64_t n, int64_t n_edges, const int32_t *d_sr
         k_ingest_pairs<<<blocks(n_edges), 256, 0, s>>>(n, n_edges, d_src, d_dst, k[0], v[0], status);
         PS_LAUNCH_CHECK();
         const int bits = id_bits(n);
-        auto pass = [&](const u64 *dcount, const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
-                        int shift, int nbits, int vshift) {
-            const int64_t tiles = sort_scan_tiles(n_edges);
-            ScanState<uint32_t> scan{};
-            if (tiles) scan = ingest_scan_state<uint32_t>(ws, L, tiles, &used);
-            return sort_pass({n_edges, dcount, kin, vin, kout, vout, shift, nbits, vshift, counts}, scan, s);
+        auto take = [&](int64_t tiles, ScanState<uint32_t> *scan) {
+            *scan = ingest_scan_state<uint32_t>(ws, L, tiles, &used);
+            return PS_OK;
         };
         // (hi, lo) pairs by lo * 2^bits + hi, 8 bits at a time
-        int a = 0, b = 1;
+        SortPass sort[kMaxPasses];
+        int passes = 0, a = 0, b = 1, rc;
         for (int shift = 0; shift < 2 * bits; shift += 8) {
             const int nbits = std::min(8, 2 * bits - shift);
-            int rc;
-            if (shift + nbits <= bits) rc = pass(nullptr, k[a], v[a], k[b], v[b], shift, nbits, 0);
-            else if (shift >= bits) rc = pass(nullptr, v[a], k[a], v[b], k[b], shift - bits, nbits, 0);
-            else rc = pass(nullptr, k[a], v[a], k[b], v[b], shift, nbits, bits - shift);
-            if (rc) return rc;
+            SortPass &p = sort[passes++];
+            if (shift >= bits) p = {n_edges, nullptr, v[a], k[a], v[b], k[b], shift - bits, nbits, 0, counts};
+            else p = {n_edges, nullptr, k[a], v[a], k[b], v[b], shift, nbits, shift + nbits <= bits ? 0 : bits - shift, counts};
             std::swap(a, b);
         }
+        rc = sort_passes(sort, passes, take, s);
+        if (rc) return rc;
         // the kept pairs into list b
         const int64_t tiles = (n_edges + kScanTile - 1) / kScanTile;
         k_scan<uint32_t, kScanBlock, kScanItems><<<(unsigned)tiles, kScanBlock, 0, s>>>(
@@ -242,12 +240,14 @@ extern "C" int ps_csr_from_edges(int64_t n, int64_t n_edges, const int32_t *d_sr
         // the same pairs sorted by hi: from list b between the other two
         const u64 *kept = status + IS_PAIRS;
         int from = b, to = a, spare = kPairLists - 1;
+        passes = 0;
         for (int shift = 0; shift < bits; shift += 8) {
-            const int rc = pass(kept, k[from], v[from], k[to], v[to], shift, std::min(8, bits - shift), 0);
-            if (rc) return rc;
+            sort[passes++] = {n_edges, kept, k[from], v[from], k[to], v[to], shift, std::min(8, bits - shift), 0, counts};
             from = to;
             std::swap(to, spare);
         }
+        rc = sort_passes(sort, passes, take, s);
+        if (rc) return rc;
         k_ingest_spans<<<blocks(n_edges), 256, 0, s>>>(kept, k[from], below);
         PS_LAUNCH_CHECK();
         if (n > 0) {

@@ -774,16 +774,17 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     // passes above its bits do nothing.
     int bits = 1;
     while (bits < 31 && (static_cast<uint64_t>(n > 0 ? n - 1 : 0) >> bits) != 0) bits++;
+    SortPass order[kMaxPasses];
+    int passes = 0;
     for (int shift = 0; shift < bits && n > 0; shift += 8) {
         const bool even = shift % 16 == 0;
-        ScanState<uint32_t> scan{};
-        if (sort_scan_tiles(n)) rc = take_scan(g, sort_scan_tiles(n), &scan);
-        if (rc) return rc;
-        rc = sort_pass({n, nullptr, even ? k0 : k1, shift ? (even ? v0 : v1) : nullptr, even ? k1 : k0, even ? v1 : v0,
-                        shift, std::min(8, bits - shift), 0, reinterpret_cast<uint32_t *>(ws + L.counts),
-                        g->status + ST_DMAX}, scan, s);
-        if (rc) return rc;
+        order[passes++] = {n, nullptr, even ? k0 : k1, shift ? (even ? v0 : v1) : nullptr, even ? k1 : k0,
+                           even ? v1 : v0, shift, std::min(8, bits - shift), 0,
+                           reinterpret_cast<uint32_t *>(ws + L.counts), g->status + ST_DMAX};
     }
+    auto take = [g](int64_t tiles, ScanState<uint32_t> *scan) { return take_scan(g, tiles, scan); };
+    rc = sort_passes(order, passes, take, s);
+    if (rc) return rc;
     uint32_t *inv = reinterpret_cast<uint32_t *>(ws + L.inv);
     if (n > 0) {
         k_rank<<<sms * 8, 256, 0, s>>>(n, bits, k0, v0, k1, v1, g->rank, inv, g->dnew, g->lowcnt,

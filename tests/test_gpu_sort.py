@@ -37,6 +37,27 @@ def test_structure_at_tile_edges(n):
     _check_structure(gg.chung_lu(n, 3.0, 2.5, 60.0, 9, exact_pairs=False))
 
 
+@pytest.mark.parametrize("n", [3, 200, 256, 5000, 1 << 20])
+@pytest.mark.parametrize("e", [31, 1023, 1024, 1025, 2049, 4097, 8192, 8193, 16_385, 40_000, 65_536, 131_071,
+                               131_072, 131_073])
+def test_one_cluster(n, e):
+    """The sort of short lists in one launch: one block and the first of two,
+    four, eight and sixteen, rows just full and one item more, the largest list and the
+    first that is sorted pass by pass; with repeats, so the second sort is
+    shorter than its launch."""
+    rs = np.random.Generator(np.random.PCG64(n + e))
+    src, dst = rs.integers(0, n, e).astype(np.int32), rs.integers(0, n, e).astype(np.int32)
+    off, col = O.csr_from_edges(n, src, dst)
+    g_off, g_col = ps.csr_from_edges(n, src, dst)
+    assert np.array_equal(g_off.cpu().numpy(), off) and np.array_equal(g_col.cpu().numpy(), col)
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 8193, 16_385, 65_536, 100_003, 131_072, 131_073])
+def test_one_cluster_structure(n):
+    """Degree order and edge table from lists sorted in one launch."""
+    _check_structure(gg.chung_lu(n, 2.0, 2.5, 40.0, 9, exact_pairs=False))
+
+
 def test_equal_degrees():
     """All degrees equal: the order is by id alone; and all zero."""
     _check_structure(gg.cycle(5000))
