@@ -25,7 +25,7 @@
 namespace ps {
 
 constexpr int kSortBlock = 256;
-constexpr int kSortItems = 16;
+constexpr int kSortItems = 14;
 constexpr int kSortWarps = kSortBlock / 32;
 constexpr int64_t kSortTile = static_cast<int64_t>(kSortBlock) * kSortItems;
 constexpr int64_t kDirectTiles = 64;
@@ -113,7 +113,13 @@ __device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t *s_wsum) {
 // Stable scatter of one tile.  Item order within a tile: warp w owns the w-th
 // slice of 32 * kSortItems items and walks it in rows of 32 lanes, so (warp,
 // row, lane) is index order.  Only the keys and their ranks stay in registers
-// (values are read when placed), which keeps four blocks resident per SM.
+// (values are read when placed), which keeps four blocks resident per SM: what
+// bounds the kernel is the latency of the ranking, with ballots and shared
+// memory each busy about half the time.  Ingest of 15.7M pairs, whole: three
+// blocks of the same tile 1.81 ms, four 1.38, five with spills 1.58; tiles of
+// 12, 14, 16 and 18 rows per warp 1.47, 1.36, 1.40 and 1.41 (shorter tiles write
+// shorter runs).  Warp bases that include the digit's start and items moved
+// as 8 bytes take two shared-memory accesses per item fewer: 1.45 -> 1.39 ms.
 // DIRECT: `offsets` holds the raw counts; otherwise offsets[digit * tiles +
 // tile] is where the tile's run of that digit starts.  VAL: values read from
 // vin, or the items' indices, or read and part of the digit.
@@ -128,10 +134,8 @@ k_sort_scatter(int64_t count, const u64 *dcount, const u64 *max_key, const uint3
     constexpr bool CROSS = VAL == kValCross;
     if (skip_pass(max_key, shift)) return;
     count = live_count(count, dcount);
-    __shared__ uint32_t s_key[kSortTile];
-    __shared__ uint32_t s_val[kSortTile];
+    __shared__ uint2 s_item[kSortTile];          // (key, value) in the tile's order
     __shared__ uint32_t s_cnt[kSortWarps][256];  // per-warp counts, then per-warp bases
-    __shared__ uint32_t s_start[256];            // first tile-local slot of each digit
     __shared__ uint32_t s_glob[256];             // global start of the tile's run of each digit
     __shared__ uint32_t s_wsum[2 * kSortWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -163,39 +167,55 @@ k_sort_scatter(int64_t count, const u64 *dcount, const u64 *max_key, const uint3
     // (below 32 * kSortItems, two to a register)
     static_assert(32 * kSortItems <= 65536 && kSortItems % 2 == 0, "ranks packed in 16 bits");
     uint32_t rank2[kSortItems / 2];
+    // (a crossing digit reads the value here and again when placing it)
+    auto digit_at = [&](int q) {
+        const bool read = CROSS && base + 32 * q < n_tile;
+        return digit_of<CROSS>(k[q], read ? __ldg(vin + base + 32 * q) : 0u, shift, vshift, kMask);
+    };
 #pragma unroll
-    for (int q = 0; q < kSortItems; q++) {
-        const bool ok = base + 32 * q < n_tile;
-        // (a crossing digit reads the value here and again when placing it)
-        const uint32_t d = digit_of<CROSS>(k[q], CROSS && ok ? __ldg(vin + base + 32 * q) : 0u, shift, vshift, kMask);
-        uint32_t peers = __ballot_sync(0xffffffffu, ok);
+    for (int q0 = 0; q0 < kSortItems; q0 += 2) {  // two rows' ballots in flight
+        uint32_t peers[2];
 #pragma unroll
-        for (int b = 0; b < BITS; b++) {
-            const bool bit = (d >> b) & 1u;
-            const uint32_t v = __ballot_sync(0xffffffffu, bit);
-            peers &= bit ? v : ~v;
+        for (int h = 0; h < 2; h++) {
+            const uint32_t d = digit_at(q0 + h);
+            peers[h] = __ballot_sync(0xffffffffu, base + 32 * (q0 + h) < n_tile);
+#pragma unroll
+            for (int b = 0; b < BITS; b++) {
+                const bool bit = (d >> b) & 1u;
+                const uint32_t v = __ballot_sync(0xffffffffu, bit);
+                peers[h] &= bit ? v : ~v;
+            }
         }
-        const uint32_t before = s_cnt[warp][d];
-        const uint32_t r = before + __popc(peers & lanemask_lt());
-        if (q & 1) rank2[q / 2] |= r << 16;
-        else rank2[q / 2] = r;
-        __syncwarp();
-        if (ok && lane == __ffs(peers) - 1) s_cnt[warp][d] = before + __popc(peers);
-        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const uint32_t d = digit_at(q0 + h), before = s_cnt[warp][d];
+            const uint32_t r = before + __popc(peers[h] & lanemask_lt());
+            if (h) rank2[q0 / 2] |= r << 16;
+            else rank2[q0 / 2] = r;
+            __syncwarp();
+            if (base + 32 * (q0 + h) < n_tile && lane == __ffs(peers[h]) - 1) s_cnt[warp][d] = before + __popc(peers[h]);
+            __syncwarp();
+        }
     }
     __syncthreads();
-    // thread t = digit t: per-warp bases within the digit, then the digits'
-    // tile-local starts (a block scan of the digit totals)
+    // thread t = digit t: the digits' tile-local starts (a block scan of the
+    // digit totals), from there the warps' bases, and how far the tile's run of
+    // the digit lies from its place in the tile
     {
         const int d = threadIdx.x;
-        uint32_t run = 0;
+        uint32_t c[kSortWarps], run = 0;
 #pragma unroll
         for (int w = 0; w < kSortWarps; w++) {
-            const uint32_t c = s_cnt[w][d];
-            s_cnt[w][d] = run;
-            run += c;
+            c[w] = s_cnt[w][d];
+            run += c[w];
         }
-        s_start[d] = block_excl(run, s_wsum);
+        run = block_excl(run, s_wsum);
+        s_glob[d] -= run;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; w++) {
+            s_cnt[w][d] = run;
+            run += c[w];
+        }
     }
     __syncthreads();
 #pragma unroll
@@ -203,18 +223,15 @@ k_sort_scatter(int64_t count, const u64 *dcount, const u64 *max_key, const uint3
         if (base + 32 * q < n_tile) {
             const uint32_t v = VAL == kValIota ? static_cast<uint32_t>(tile0) + base + 32 * q : __ldg(vin + base + 32 * q);
             const uint32_t d = digit_of<CROSS>(k[q], v, shift, vshift, kMask);
-            const uint32_t p = s_start[d] + s_cnt[warp][d] + ((rank2[q / 2] >> (16 * (q & 1))) & 0xFFFFu);
-            s_key[p] = k[q];
-            s_val[p] = v;
+            s_item[s_cnt[warp][d] + ((rank2[q / 2] >> (16 * (q & 1))) & 0xFFFFu)] = make_uint2(k[q], v);
         }
     }
     __syncthreads();
     for (int p = threadIdx.x; p < n_tile; p += kSortBlock) {
-        const uint32_t kk = s_key[p], vv = s_val[p];
-        const uint32_t d = digit_of<CROSS>(kk, vv, shift, vshift, kMask);
-        const uint32_t g = s_glob[d] + (p - s_start[d]);
-        kout[g] = kk;
-        vout[g] = vv;
+        const uint2 x = s_item[p];
+        const uint32_t g = s_glob[digit_of<CROSS>(x.x, x.y, shift, vshift, kMask)] + p;
+        kout[g] = x.x;
+        vout[g] = x.y;
     }
 }
 

@@ -16,6 +16,7 @@ from paper_1411_4942_gb300 import pathsample as ps  # noqa: E402
 
 
 @pytest.mark.parametrize("n, e", [(1, 1), (1, 3), (2, 1), (2, 9), (3, 7), (5, 40), (9, 4095), (300, 4096), (257, 4097),
+                                  (300, 3583), (300, 3584), (300, 3585), (4097, 64 * 3584), (4097, 64 * 3584 + 1),
                                   (4097, 64 * 4096 - 1), (70_000, 64 * 4096), (1 << 17, 64 * 4096 + 1),
                                   ((1 << 18) + 1, 300_001)])
 def test_ingest_sizes(n, e):
@@ -30,7 +31,8 @@ def test_ingest_sizes(n, e):
     assert np.array_equal(g_off.cpu().numpy(), off) and np.array_equal(g_col.cpu().numpy(), col)
 
 
-@pytest.mark.parametrize("n", [255, 257, 4095, 4097, 65_535, 65_537, 64 * 4096, 64 * 4096 + 1])
+@pytest.mark.parametrize("n", [255, 257, 4095, 4097, 65_535, 65_537, 64 * 3584, 64 * 3584 + 1, 64 * 4096,
+                               64 * 4096 + 1])
 def test_structure_at_tile_edges(n):
     """Every load array against the oracle with n vertices and about n (one
     sort tile per sort tile of vertices) to 2 n edges."""
