@@ -524,8 +524,7 @@ int ps_count_adaptive(const ps_graph *g, uint64_t seed, double target, double de
     Readback back;
     while (true) {
         const uint64_t add = k - done;
-        if (g->stats.W > 0) rc = launch_sampler(g, 0, add, seed, done, d_hist6, s);
-        if (rc == PS_OK && g->stats.Lambda > 0) rc = launch_sampler(g, 1, add, seed, done, d_hist4, s);
+        rc = launch_samplers(g, add, d_hist6, add, d_hist4, seed, done, s);
         if (rc != PS_OK) return rc;
         rc = back.queue(d_hist6, 6, d_hist4, 4, s);
         if (rc != PS_OK) return rc;
@@ -641,12 +640,13 @@ int ps_count_motifs_host(int64_t n, int64_t nnz, const int64_t *h_off, const int
     void *oscr = static_cast<char *>(d_workspace) + used;
     const size_t obytes = ws_bytes - used;
     const bool ordered = obytes >= ordered_scratch_bytes(1);
-    if (st.W > 0)
-        rc = ordered ? ps_sample_3paths_ordered(g, k3, seed, 0, d_hist, oscr, obytes, stream)
-                     : ps_sample_3paths(g, k3, seed, 0, d_hist, stream);
-    if (rc >= 0 && st.Lambda > 0)
-        rc = ordered ? ps_sample_centered_ordered(g, kc, seed, 0, d_hist + 8, oscr, obytes, stream)
-                     : ps_sample_centered(g, kc, seed, 0, d_hist + 8, stream);
+    if (!ordered || order_never(g)) {
+        rc = launch_samplers(g, k3, d_hist, kc, d_hist + 8, seed, 0, s);
+    } else {
+        if (st.W > 0) rc = ps_sample_3paths_ordered(g, k3, seed, 0, d_hist, oscr, obytes, stream);
+        if (rc >= 0 && st.Lambda > 0)
+            rc = ps_sample_centered_ordered(g, kc, seed, 0, d_hist + 8, oscr, obytes, stream);
+    }
     if (rc < 0) {
         ps_graph_free(g);
         return rc;

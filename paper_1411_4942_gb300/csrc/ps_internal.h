@@ -244,10 +244,14 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
 int prefix_graph(ps_graph *g, cudaStream_t s);
 int launch_sampler(const ps_graph *g, int sampler, uint64_t k, uint64_t seed, uint64_t first_id,
                    uint64_t *d_hist, cudaStream_t s);
+// Both samplers over ids first_id ..; one without anything to draw is left out.
+int launch_samplers(const ps_graph *g, uint64_t k3, uint64_t *d_hist6, uint64_t kc, uint64_t *d_hist4, uint64_t seed,
+                    uint64_t first_id, cudaStream_t s);
 // Samples in the order of their edge draws (ps_order.cu); ids of a chunk are
 // 32-bit offsets, so a chunk holds at most kOrderMaxChunk samples.
 constexpr uint64_t kOrderMaxChunk = 1ull << 31;
 size_t ordered_scratch_bytes(uint64_t k_chunk);
+bool order_never(const ps_graph *g);  // every number of samples of this graph is drawn plainly
 int launch_ordered(const ps_graph *g, int sampler, uint64_t k, uint64_t seed, uint64_t first_id, uint64_t *d_hist,
                    void *d_scratch, size_t scratch_bytes, cudaStream_t s);
 int launch_batch(const void *d_table, int32_t n_graphs, const ps_work *d_items, int64_t n_items,

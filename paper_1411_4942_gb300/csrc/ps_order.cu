@@ -350,13 +350,16 @@ size_t ordered_scratch_bytes(uint64_t k_chunk) {
     return kOrderHeader + static_cast<size_t>(k_chunk) * kOrderPerSample;
 }
 
+bool order_never(const ps_graph *g) {
+    return g->tune.draw_order < 0 || (g->tune.draw_order == 0 && g->m < kOrderMinEdges);
+}
+
 int launch_ordered(const ps_graph *g, int sampler, uint64_t k, uint64_t seed, uint64_t first_id, uint64_t *d_hist,
                    void *d_scratch, size_t scratch_bytes, cudaStream_t s) {
     if (scratch_bytes < ordered_scratch_bytes(1)) return PS_ERR_WORKSPACE;
     uint64_t chunk = (scratch_bytes - kOrderHeader) / kOrderPerSample;
     if (chunk > kOrderMaxSorted) chunk = kOrderMaxSorted;
-    if (g->tune.draw_order < 0 || (g->tune.draw_order == 0 && g->m < kOrderMinEdges))
-        return launch_sampler(g, sampler, k, seed, first_id, d_hist, s);
+    if (order_never(g)) return launch_sampler(g, sampler, k, seed, first_id, d_hist, s);
     char *scratch = static_cast<char *>(d_scratch);
     return sampler == 0 ? ordered_s<0>(g, k, seed, first_id, d_hist, scratch, chunk, s)
                         : ordered_s<1>(g, k, seed, first_id, d_hist, scratch, chunk, s);
