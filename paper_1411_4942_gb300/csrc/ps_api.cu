@@ -188,6 +188,8 @@ bool make_layout(int64_t n, int64_t nnz, const Tuning &t, Layout *L) {
     l.lowcnt = take(n1 * sizeof(int32_t));
     l.ubase = take((n1 + 1) * sizeof(int64_t));
     l.dnew = take(n1 * sizeof(int32_t));
+    l.row_span = take(n1 * sizeof(int2));
+    l.row_upper = take(n1 * sizeof(int2));
     l.rec = take(static_cast<size_t>(l.m_cap) * sizeof(EdgeRec));
     l.ptau = take(static_cast<size_t>(l.m_cap) * sizeof(uint64_t));
     l.plam = take(static_cast<size_t>(l.m_cap) * sizeof(uint64_t));
@@ -348,6 +350,8 @@ int ps_load_csr(int64_t n, int64_t nnz, const int64_t *d_off, const int32_t *d_c
     g->rank = reinterpret_cast<int32_t *>(ws + L.rank);
     g->lowcnt = reinterpret_cast<int32_t *>(ws + L.lowcnt);
     g->ubase = reinterpret_cast<int64_t *>(ws + L.ubase);
+    g->row_span = reinterpret_cast<int2 *>(ws + L.row_span);
+    g->row_upper = reinterpret_cast<int2 *>(ws + L.row_upper);
     g->dnew = reinterpret_cast<int32_t *>(ws + L.dnew);
     g->rec = reinterpret_cast<EdgeRec *>(ws + L.rec);
     g->ptau = reinterpret_cast<uint64_t *>(ws + L.ptau);

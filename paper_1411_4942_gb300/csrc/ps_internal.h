@@ -53,7 +53,7 @@ struct Layout {
     int64_t scan_words;    // 64-bit words of one load's scans (tile counters and slots)
     int64_t filt_words;    // 32-bit words of the edge filter; 0 without it
     int64_t vtab_slots;    // 0 without the per-vertex tables
-    size_t status, off, col, rank, lowcnt, ubase, dnew, rec, ptau, plam, gtau, glam, hub, filt, vtab;
+    size_t status, off, col, rank, lowcnt, ubase, dnew, row_span, row_upper, rec, ptau, plam, gtau, glam, hub, filt, vtab;
     size_t keys0, keys1, vals0, vals1, inv, counts, scan;
     size_t total;
 };
@@ -76,6 +76,7 @@ struct ps_graph {
     int32_t *rank;
     int32_t *lowcnt;
     int64_t *ubase;
+    int2 *row_span, *row_upper;  // of each row: (offset, degree) and (lower arcs, first edge)
     int32_t *dnew;
     ps::EdgeRec *rec;
     uint64_t *ptau, *plam;

@@ -694,10 +694,15 @@ struct LoadUp {
 };
 struct StoreUbase {
     int64_t *ubase;
+    const int64_t *off;
+    const int32_t *dnew, *low;
+    int2 *row_span, *row_upper;  // below 2^31 all (nnz < 2^31)
     int64_t n;
     u64 *status;
     __device__ void operator()(int64_t i, int64_t exc, int64_t inc) const {
         ubase[i] = exc;
+        row_span[i] = make_int2(static_cast<int32_t>(off[i]), dnew[i]);
+        row_upper[i] = make_int2(low[i], static_cast<int32_t>(exc));
         if (i == n - 1) {
             ubase[n] = inc;
             status[ST_M_UPPER] = static_cast<u64>(inc);
@@ -865,7 +870,7 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
 
     // (4) the edge numbering: ubase[r] = the edges (upper arcs) of the rows before r
     rc = run_scan<int64_t>(g, n, (int64_t)0, OpSum(), LoadUp{g->dnew, g->lowcnt},
-                           StoreUbase{g->ubase, n, g->status}, s);
+                           StoreUbase{g->ubase, g->off, g->dnew, g->lowcnt, g->row_span, g->row_upper, n, g->status}, s);
     if (rc) return rc;
 
     // (5) on a side stream the hub rows, which need only the sorted rows; here
