@@ -107,18 +107,50 @@ k_lower_arcs(int64_t n, const int64_t *__restrict__ coff, const int32_t *__restr
     }
 }
 
-// Rows of kLongRow + 1 .. kTierC entries (from status[first_slot] on): a warp
-// per row, the next row's offsets fetched while the current one is copied.
+// Rows of kLongRow + 1 .. kTierC entries: a warp per row, the next row's
+// offsets fetched while the current one is copied.  With SHORT, before them
+// the shorter rows, 8 lanes each (150k rows of about 20 entries 32 -> 20 us),
+// or a warp each where there are no more rows than warps.
+constexpr int kShortLanes = 8;
+template <bool SHORT>
 __global__ void __launch_bounds__(256)
 k_lower_arcs_mid(const int64_t *__restrict__ coff, const int32_t *__restrict__ ccol,
                  const int32_t *__restrict__ lowcnt, const int64_t *__restrict__ ubase,
                  uint32_t *__restrict__ key, uint32_t *__restrict__ val, int64_t m_cap,
-                 const u64 *__restrict__ status, int first_slot, int64_t n, EdgeFilter F) {
+                 const u64 *__restrict__ status, int64_t n, EdgeFilter F) {
     const int32_t hub_start = static_cast<int32_t>(n - static_cast<int64_t>(status[ST_HUBS]));
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * blockDim.x / 32;
+    const bool share = SHORT && n > nw;
+    if (share) {
+        const int at = lane % kShortLanes;
+        const int64_t s_end = static_cast<int64_t>(status[ST_LONG]);
+        for (int64_t q = static_cast<int64_t>(status[ST_TIER]) + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kShortLanes;
+             q < s_end; q += nw * (32 / kShortLanes)) {
+            const int64_t o = ldg_i64(coff + q), lb = o - ldg_i64(ubase + q);
+            const int32_t low = ldg_i32(lowcnt + q);
+            for (int32_t p0 = 0; p0 < low; p0 += kShortLanes * kListBatch) {
+                int32_t c[kListBatch];
+#pragma unroll
+                for (int u = 0; u < kListBatch; u++) {
+                    const int32_t p = p0 + kShortLanes * u + at;
+                    c[u] = (p < low && lb + p < m_cap) ? ldg_i32(ccol + o + p) : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < kListBatch; u++) {
+                    const int32_t p = p0 + kShortLanes * u + at;
+                    if (p < low && lb + p < m_cap) {
+                        key[lb + p] = static_cast<uint32_t>(c[u]);
+                        val[lb + p] = static_cast<uint32_t>(o + p);
+                        F.add(c[u], static_cast<int32_t>(q), hub_start);
+                    }
+                }
+            }
+        }
+    }
     const int64_t r_end = static_cast<int64_t>(status[ST_TIER + 3]);
-    int64_t r = static_cast<int64_t>(status[first_slot]) + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    int64_t r = static_cast<int64_t>(status[SHORT && !share ? ST_TIER : ST_LONG]) +
+                ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     int64_t o_ = 0, ub_ = 0;
     int32_t low_ = 0;
     if (r < r_end) {
@@ -317,9 +349,13 @@ int build_edge_table(ps_graph *g, cudaStream_t s) {
             k_lower_arcs<<<(unsigned)blocks, 256, 0, s>>>(n, g->off, g->col, g->ubase, ka, va, m, g->status, F);
             PS_LAUNCH_CHECK();
         }
-        if (few || g->d_max > kLongRow) {
-            k_lower_arcs_mid<<<(unsigned)(sms * (few ? 8 : 6)), 256, 0, s>>>(g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
-                                                                             g->status, few ? ST_TIER : ST_LONG, n, F);
+        if (few) {
+            k_lower_arcs_mid<true><<<(unsigned)(sms * 8), 256, 0, s>>>(g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
+                                                                       g->status, n, F);
+            PS_LAUNCH_CHECK();
+        } else if (g->d_max > kLongRow) {
+            k_lower_arcs_mid<false><<<(unsigned)(sms * 6), 256, 0, s>>>(g->off, g->col, g->lowcnt, g->ubase, ka, va, m,
+                                                                        g->status, n, F);
             PS_LAUNCH_CHECK();
         }
         if (g->d_max > kTierC) {
