@@ -48,7 +48,7 @@ SECTOR = 32
 # one 32-byte sector per random access): 3-path = edge draw, edge record,
 # both endpoint offsets, the two neighbour reads and three adjacency lookups
 BYTES_3PATH = 9 * SECTOR
-# largest chunk of the draw-ordered samplers (their scratch is 5 B per sample
+# largest chunk of the draw-ordered samplers (their scratch is 11 B per sample
 # of a chunk); by default one chunk holds all of a call's samples up to this
 MAX_ORDER_CHUNK = 1 << 27
 # the load step's streaming bytes per edge in the O(m) preprocessing model:
