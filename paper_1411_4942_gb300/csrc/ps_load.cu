@@ -199,12 +199,6 @@ __global__ void __launch_bounds__(256, 6) k_sort_tier_a(RowIn R) {
     report(R, bad, nsimple);
 }
 
-__device__ __forceinline__ int next_pow2(int d) {
-    int p = 1;
-    while (p < d) p <<= 1;
-    return p;
-}
-
 // Bitonic sort, ascending, of N = E * THREADS keys held E per thread in
 // blocked order (thread t holds keys t*E .. t*E + E - 1).  A compare-exchange
 // stage whose partner key sits in the same thread works on registers, one
