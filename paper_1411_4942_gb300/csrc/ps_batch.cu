@@ -108,7 +108,7 @@ k_batch(const GraphDev *__restrict__ table, int32_t n_graphs, const ps_work *__r
         if (it < n_items) s_w[0] = items[it];
     }
     __syncthreads();
-    uint32_t graph = kNone;  // of s_g
+    uint32_t graph = kNone;  // of s_g; n_graphs: the empty one
     for (int at = 0; s_item[at] < n_items; at ^= 1) {
         if (threadIdx.x == 0) {
             s_item[at ^ 1] = claim;
@@ -122,9 +122,11 @@ k_batch(const GraphDev *__restrict__ table, int32_t n_graphs, const ps_work *__r
             }
         }
         const ps_work w = s_w[at];
-        if (w.graph != graph) {
-            // (an item that names no graph leaves an empty one: nothing to sample)
-            graph = w.graph;
+        // an item that names no graph, whatever number stands there (kNone too),
+        // takes the empty one: nothing to sample
+        const uint32_t named = min(w.graph, static_cast<uint32_t>(n_graphs));
+        if (named != graph) {
+            graph = named;
             if (graph < static_cast<uint32_t>(n_graphs)) {
                 for (int i = threadIdx.x; i < static_cast<int>(sizeof(GraphDev) / 4); i += BLOCK)
                     reinterpret_cast<uint32_t *>(&s_g)[i] = __ldg(reinterpret_cast<const uint32_t *>(table + graph) + i);

@@ -75,3 +75,28 @@ def test_items_that_do_not_run(graphs, n):
     assert skipped == 0 and not hist[2].any()
     for s, G in enumerate((graphs[0], other)):
         assert hist[s].tolist() == _plain(G, 0, 11 * int((i % 3 == s).sum()))
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("name", [99, 0xFFFFFFFE, 0xFFFFFFFF])
+@pytest.mark.parametrize("n", [1, 3000])
+def test_blocks_that_start_on_an_item_without_a_graph(graphs, n, name, mixed):
+    """The queue opens with items that name no graph, so that every block's
+    first one is such an item: nothing sampled, none counted as skipped, and
+    the items behind them run."""
+    second = graphs[1]
+    if mixed:
+        g = gg.complete(12)
+        second = ps.Graph(g.off, g.col, tuning=ps.make_tuning(adjacency=ps.ADJ_SEARCH))
+    gset = psb.GraphSet([graphs[0], second])
+    items = np.zeros(n + 6, dtype=ps.WORK_DTYPE)
+    items["graph"][:n], items["slot"][:n] = name, 2
+    i = np.arange(6)
+    items["graph"][n:] = items["slot"][n:] = i % 2
+    items["first_id"][n:] = 11 * (i // 2)
+    items["sampler"][:n] = np.arange(n) % 2
+    items["count"], items["seed"] = 11, SEED
+    hist, skipped = _launch(gset, items, 3)
+    assert skipped == 0 and not hist[2].any()
+    for s, G in enumerate((graphs[0], second)):
+        assert hist[s].tolist() == _plain(G, 0, 33)
