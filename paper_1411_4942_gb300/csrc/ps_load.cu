@@ -708,6 +708,9 @@ __global__ void __launch_bounds__(kBitmapThreads, 1) k_sort_bitmap(RowIn R, int3
             written += total;
             __syncthreads();  // s_warp / s_low reused by the next chunk
         }
+        // repeated entries leave the row short: later kernels of the load take
+        // every column for a label
+        for (int i = written + tid; i < d; i += kBitmapThreads) dst[i] = static_cast<int32_t>(r);
 #pragma unroll
         for (int q = 16; q > 0; q >>= 1) low += __shfl_xor_sync(0xffffffffu, low, q);
         if (lane == 0) s_low[warp] = low;
