@@ -22,3 +22,22 @@ def test_bars_equal_plain_bisection(k, delta):
         rc, est, lo, hi = ps.ps_estimate(st, h6, k, h4, k, delta)
         _, oest, olo, ohi = O.estimate(int(st.W), int(st.Lambda), st.N1, h6, k, h4, k, delta)
         assert est.tolist() == list(oest) and lo.tolist() == list(olo) and hi.tolist() == list(ohi)
+
+
+@pytest.mark.parametrize("k, c, delta", [
+    (20601542668580, 20601542668542, 6.501372376723512e-92),
+    (105277841728479, 105277841728475, 0.004123769651538563),
+    (6968, 6942, 1e-305), (89765, 89760, 2.3e-50), (154357, 154326, 1e-317), (121166605, 121166564, 1e-308),
+    (1498341142809319936, 1466, 3e-308), (1568932294595252992, 1452, 1e-308),
+] + [(k, k - r, 10.0 ** -e) for k in (1000, 24001, 10 ** 6 + 3, (1 << 30) + 1, 1 << 45)
+     for r in (1, 4, 15, 40) for e in (2, 30, 90, 150, 200, 250, 300)])
+def test_bars_next_to_the_ends(k, c, delta):
+    """Roots within a few ulp of 1 or of alpha, where D is steep or flat and
+    Newton's last step says little about how far the root is."""
+    st = ps.PsStats()
+    st.W, st.Lambda, st.N1_lo, st.n, st.m = 1 << 40, 1 << 38, 10 ** 7, 10, 9
+    h6 = np.array([0, c, k - c, c, c, k - c], dtype=np.uint64)
+    h4 = np.array([0, c, k - c, c], dtype=np.uint64)
+    rc, est, lo, hi = ps.ps_estimate(st, h6, k, h4, k, delta)
+    _, oest, olo, ohi = O.estimate(int(st.W), int(st.Lambda), st.N1, h6, k, h4, k, delta)
+    assert est.tolist() == list(oest) and lo.tolist() == list(olo) and hi.tolist() == list(ohi)
