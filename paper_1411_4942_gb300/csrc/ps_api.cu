@@ -48,20 +48,60 @@ int sm_count_of_current_device() {
     return sms > 0 ? sms : 1;
 }
 
-int get_side_streams(int device, cudaStream_t out[2]) {
-    constexpr int kMaxDevices = 64;
-    static std::mutex mu;
-    static cudaStream_t streams[kMaxDevices][2] = {};
-    if (device < 0 || device >= kMaxDevices) return PS_ERR_ARG;
-    std::lock_guard<std::mutex> lock(mu);
-    for (int i = 0; i < 2; ++i)
-        if (!streams[device][i] && cudaStreamCreateWithFlags(&streams[device][i], cudaStreamNonBlocking) != cudaSuccess) {
-            streams[device][i] = nullptr;
-            return PS_ERR_CUDA;
+namespace {
+
+// Pairs of side streams per device, made when a call finds none free; they
+// belong to a context, and a device reset brings a new one.  A call past
+// kSidePairs at a time, or on a device past its kSideContexts contexts, runs
+// on its own stream alone.
+constexpr int kSidePairs = 16;
+constexpr int kSideContexts = 16;
+constexpr int kSideDevices = 64;
+struct SidePool {
+    unsigned long long ctx_id = 0;
+    int generation = 0;
+    uint32_t taken = 0;
+    cudaStream_t pair[kSidePairs][2] = {};
+};
+std::mutex g_side_mutex;
+SidePool g_side[kSideDevices];
+
+}  // namespace
+
+SideStreams::SideStreams(int device) : dev_(device) {
+    if (device < 0 || device >= kSideDevices) return;
+    std::lock_guard<std::mutex> lock(g_side_mutex);
+    const unsigned long long id = current_context_id();
+    if (id == 0) return;
+    SidePool &p = g_side[device];
+    if (p.ctx_id != id) {
+        if (p.generation >= kSideContexts) return;
+        const int generation = p.generation + 1;
+        p = SidePool{};
+        p.ctx_id = id;
+        p.generation = generation;
+    }
+    int i = 0;
+    while (i < kSidePairs && (p.taken >> i & 1u)) i++;
+    if (i == kSidePairs) return;
+    for (cudaStream_t &s : p.pair[i])
+        if (!s && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            s = nullptr;
+            return;
         }
-    out[0] = streams[device][0];
-    out[1] = streams[device][1];
-    return PS_OK;
+    p.taken |= 1u << i;
+    pair_ = i;
+    generation_ = p.generation;
+    stream[0] = p.pair[i][0];
+    stream[1] = p.pair[i][1];
+}
+
+SideStreams::~SideStreams() {
+    if (pair_ < 0) return;
+    std::lock_guard<std::mutex> lock(g_side_mutex);
+    SidePool &p = g_side[dev_];
+    if (p.generation == generation_) p.taken &= ~(1u << pair_);
 }
 
 // A scan whose bounded wait expired put identity in place of a predecessor's

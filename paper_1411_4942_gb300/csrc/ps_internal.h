@@ -110,9 +110,22 @@ namespace ps {
 int sm_count_of_current_device();
 int flags_to_status(uint64_t flags);
 // Two non-blocking streams of `device` for independent kernels within one
-// call (created on first use, kept for the process; calls join them with
-// their own events, so concurrent calls stay ordered correctly).
-int get_side_streams(int device, cudaStream_t out[2]);
+// call, which has them to itself while this object lives: with streams shared
+// by the calls of a device, a call that joins them, or reads from them, stands
+// behind everything that another call's stream still has before its own.
+// The caller joins them to its stream and synchronises that before the end.
+// stream[0] null: none free.
+class SideStreams {
+  public:
+    explicit SideStreams(int device);
+    ~SideStreams();
+    SideStreams(const SideStreams &) = delete;
+    SideStreams &operator=(const SideStreams &) = delete;
+    cudaStream_t stream[2] = {nullptr, nullptr};
+
+  private:
+    int dev_, pair_ = -1, generation_ = 0;
+};
 
 // Id of the context current on this thread; 0 when there is none or the
 // driver cannot say.  (Unlike context handles, ids are never reused.)

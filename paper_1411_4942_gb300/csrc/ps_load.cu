@@ -753,25 +753,24 @@ struct StoreUbase {
 
 // ------------------------------------------------------------------- driver
 
-// Runs independent kernels of one call on the device's side streams: fork()
+// Runs independent kernels of one call on its side streams: fork()
 // makes them wait for the caller's stream, join() makes the caller's stream
 // wait for them.  The destructor joins on every return path, so no side work
 // outlives a call that failed halfway.  Without side streams every kernel
 // runs on the caller's stream.
 class SideFork {
   public:
-    SideFork(ps_graph *g, cudaStream_t s) : g_(g), s_(s) { side_[0] = side_[1] = s; }
+    SideFork(ps_graph *g, const SideStreams &streams, cudaStream_t s) : g_(g), streams_(streams), s_(s) { side_[0] = side_[1] = s; }
     ~SideFork() { join(); }
     SideFork(const SideFork &) = delete;
     SideFork &operator=(const SideFork &) = delete;
 
     int fork(int count) {
-        cudaStream_t side[2];
-        if (get_side_streams(g_->device, side) != PS_OK) return PS_OK;
+        if (!streams_.stream[0]) return PS_OK;
         PS_CUDA_TRY(cudaEventRecord(g_->ev[0], s_));
         for (int i = 0; i < count; i++) {
-            PS_CUDA_TRY(cudaStreamWaitEvent(side[i], g_->ev[0], 0));
-            side_[i] = side[i];
+            PS_CUDA_TRY(cudaStreamWaitEvent(streams_.stream[i], g_->ev[0], 0));
+            side_[i] = streams_.stream[i];
             used_ = i + 1;
         }
         return PS_OK;
@@ -789,6 +788,7 @@ class SideFork {
 
   private:
     ps_graph *g_;
+    const SideStreams &streams_;
     cudaStream_t s_;
     cudaStream_t side_[2];
     int used_ = 0;
@@ -811,7 +811,8 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     // (1) degrees and offset validation; nothing else may index with bad offsets
     k_degrees<<<sms * 8, 256, 0, s>>>(n, nnz, d_off, k0, g->status);
     PS_LAUNCH_CHECK();
-    SideFork read(g, s);
+    SideStreams streams(g->device);
+    SideFork read(g, streams, s);
     int rc = read.fork(1);
     if (rc) return rc;
 
@@ -872,7 +873,7 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
     // the long-row tiers run on side streams next to the short-row ones
     RowIn R{d_off, d_col, inv, g->rank, g->off, g->col, g->lowcnt, n, g->status};
     if (n > 0) {
-        SideFork fork(g, s);
+        SideFork fork(g, streams, s);
         if (g->d_max > tier_b(nnz)) {
             rc = fork.fork(2);
             if (rc) return rc;
@@ -916,7 +917,7 @@ int load_graph(ps_graph *g, const int64_t *d_off, const int32_t *d_col, cudaStre
 
     // (5) on a side stream the hub rows, which need only the sorted rows; here
     // the edge table, the prefixes and the edge filter, then the guide tables
-    SideFork hubs(g, s);
+    SideFork hubs(g, streams, s);
     rc = hubs.fork(1);
     if (rc) return rc;
     rc = launch_hub_rows(g, hubs.side(0));
