@@ -48,8 +48,9 @@ __device__ __forceinline__ void batch_sample2_hash(const GraphDev &g, int sample
         path3_draw(g, seed, id0, e0, a0, b0);
         path3_draw(g, seed, id1, e1, a1, b1);
         const int32_t x[6] = {a0, e0.u, a0, a1, e1.u, a1}, y[6] = {e0.v, b0, b0, e1.v, b1, b1};
+        const PairRow none[6] = {{0, -1}, {0, -1}, {0, -1}, {0, -1}, {0, -1}, {0, -1}};
         bool r[6];
-        pair_tests<6>(g, x, y, r);
+        pair_tests<6>(g, x, y, none, r);
         c0 = a0 == b0 ? 0 : class3(r[0], r[1], r[2]);
         c1 = a1 == b1 ? 0 : class3(r[3], r[4], r[5]);
     } else {
@@ -57,18 +58,21 @@ __device__ __forceinline__ void batch_sample2_hash(const GraphDev &g, int sample
         centred_draw(g, seed, id1, e1, a1, b1);
         // the chords only for centred paths (u' == v' is not one)
         const int32_t x[2] = {a0, a1}, y[2] = {b0, b1};
+        const PairRow none[2] = {{0, -1}, {0, -1}};
         bool k[2];
-        pair_tests<2>(g, x, y, k);
+        pair_tests<2>(g, x, y, none, k);
         c0 = c1 = 0;
         bool r[2];
         if (k[0] && a0 != b0) {
             const int32_t p[2] = {a0, e0.u}, q[2] = {e0.v, b0};
-            pair_tests<2>(g, p, q, r);
+            const PairRow row[2] = {{e0.ov, e0.dv}, {e0.ou, e0.du}};
+            pair_tests<2>(g, p, q, row, r);
             c0 = 1 + (int)r[0] + (int)r[1];
         }
         if (k[1] && a1 != b1) {
             const int32_t p[2] = {a1, e1.u}, q[2] = {e1.v, b1};
-            pair_tests<2>(g, p, q, r);
+            const PairRow row[2] = {{e1.ov, e1.dv}, {e1.ou, e1.du}};
+            pair_tests<2>(g, p, q, row, r);
             c1 = 1 + (int)r[0] + (int)r[1];
         }
     }

@@ -58,8 +58,9 @@ __device__ __forceinline__ int sample_3path(const GraphDev &g, uint64_t seed, ui
     bool e1, e2, e3;
     if (ADJ == kAdjHash) {
         const int32_t x[3] = {up, e.u, up}, y[3] = {e.v, vp, vp};
+        const PairRow row[3] = {{e.ov, up > e.v ? e.dv : -1}, {e.ou, vp > e.u ? e.du : -1}, {0, -1}};
         bool r[3];
-        pair_tests<3>(g, x, y, r);
+        pair_tests<3>(g, x, y, row, r);
         e1 = r[0];
         e2 = r[1];
         e3 = r[2];
@@ -132,10 +133,12 @@ __device__ __forceinline__ int sample_centred(const GraphDev &g, uint64_t seed, 
     }
     if (ADJ == kAdjHash) {
         // the closing edge first; the two chords only for centred paths
+        // (u' > v and v' > u in label order: the smaller one's row is in the record)
         if (!pair_test(g, up, vp)) return 0;  // also u' == v'
         const int32_t x[2] = {up, e.u}, y[2] = {e.v, vp};
+        const PairRow row[2] = {{e.ov, e.dv}, {e.ou, e.du}};
         bool c[2];
-        pair_tests<2>(g, x, y, c);
+        pair_tests<2>(g, x, y, row, c);
         return 1 + (int)c[0] + (int)c[1];
     }
     if (!adjacent(g, up, vp)) return 0;  // also covers u' == v'
