@@ -85,9 +85,11 @@ constexpr int kAheadItems = 4;
 // graph does not use the variant this kernel was compiled for.  Registers
 // are capped for 1024 resident threads per SM with one sample per thread in
 // flight (SPT = 1), 512 with two (SPT = 2, graphs with an edge filter; other variants
-// take their two samples one after the other).
+// take their two samples one after the other), 640 in blocks of 128: capped for
+// 512 those took up to 108 registers, so that a fifth block did not fit (36
+// R-MAT graphs, all by filter 886 -> 752 us, of mixed variants 2038 -> 1866).
 template <int BLOCK, int ADJ, int SPT>
-__global__ void __launch_bounds__(BLOCK, (SPT == 1 ? 1024 : 512) / BLOCK)
+__global__ void __launch_bounds__(BLOCK, (SPT == 1 ? 1024 : 640) / BLOCK)
 k_batch(const GraphDev *__restrict__ table, int32_t n_graphs, const ps_work *__restrict__ items,
         int64_t n_items, uint64_t *hist, uint32_t *counter) {
     // The next item is copied, and the one after it claimed, while this one
