@@ -52,7 +52,8 @@ typedef struct CUstream_st *ps_stream_t; /* same type as cudaStream_t */
  * Pass NULL for the defaults; a zero field also means "default". */
 typedef struct {
     int32_t block_size;         /* sampling threads per block: 128, 256 (default), 512, 1024 */
-    int32_t blocks_per_sm;      /* resident sampling blocks per SM (default: occupancy)      */
+    int32_t blocks_per_sm;      /* resident sampling blocks per SM (default: occupancy, or
+                                   768 threads for plain samples of large graphs)          */
     int32_t guide_log2_ratio;   /* guide buckets ~ m * 2^ratio, 1..4 (default 1, or m / 4
                                    buckets on graphs of 2^25 edges and more); -1 = none     */
     int32_t hub_count;          /* top-degree vertices (degree >= hub_min_degree) given an

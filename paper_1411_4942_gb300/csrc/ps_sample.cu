@@ -38,6 +38,31 @@ k_sample_both(GraphDev g, uint64_t k3, uint64_t kc, uint64_t seed, uint64_t firs
     flush_counts<BLOCK>(cnt, 4, hist4);
 }
 
+// From these many edges the plain samplers run 768 threads per SM instead of
+// 1024 (in blocks that divide it): where the records, rows and tables no longer
+// stay in L2, a quarter more threads evict more of each other's lines than the
+// latency they hide is worth.  Ids drawn in order (ps_order.cu) share their
+// lines and keep 1024.  2^23 samples, 1024 / 768 threads, 3-path and centred:
+//   filter   7.7M edges 541 / 522 and 380 / 416 us, 10M 677 / 628 and 579 / 543,
+//            R-MAT 20 (15.7M) 812 / 786 and 608 / 566, 117M 1261 / 1176 and 1009 / 974;
+//   tables   15.7M 953 / 992 and 1002 / 957, 10M centred 856 / 823, 7.7M centred
+//            692 / 734; 2^22 3-path, unskewed graphs of 20M: 719 / 660, 700 / 660;
+//   search   47M 2093 / 2107 and 1217 / 1342, 64M 2957 / 2897 and 2009 / 1985.
+// On clustered graphs of that size the filter's centred samples wait for their
+// confirmed hits and would rather keep 1024 (2^22 on random cliques over
+// Chung-Lu graphs of 21M and 102M edges 364 / 383 and 399 / 405 us).
+template <int ADJ>
+static int64_t few_threads_from(int sampler) {
+    if (ADJ == kAdjSearch) return int64_t{3} << 24;
+    return ADJ == kAdjVtab && sampler == 0 ? int64_t{1} << 24 : int64_t{1} << 23;
+}
+
+template <int BLOCK, int ADJ>
+static int resident_blocks(const ps_graph *g, int sampler, int occupancy) {
+    if (768 % BLOCK == 0 && occupancy > 768 / BLOCK && g->m >= few_threads_from<ADJ>(sampler)) return 768 / BLOCK;
+    return occupancy > 0 ? occupancy : 1;
+}
+
 template <int SAMPLER, int BLOCK, int ADJ>
 static int launch_t(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t first_id, uint64_t *hist,
                     cudaStream_t s) {
@@ -45,7 +70,7 @@ static int launch_t(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t first
     if (per_sm <= 0) {
         int occ = 0;
         PS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sample<SAMPLER, BLOCK, ADJ>, BLOCK, 0));
-        per_sm = occ > 0 ? occ : 1;
+        per_sm = resident_blocks<BLOCK, ADJ>(g, SAMPLER, occ);
     }
     const uint64_t full = (uint64_t)g->sm_count * per_sm;
     // per-thread counters are 32-bit: keep every thread under 2^30 samples per launch
@@ -82,7 +107,7 @@ static int launch_both_t(const ps_graph *g, uint64_t k3, uint64_t kc, uint64_t s
     if (per_sm <= 0) {
         int occ = 0;
         PS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sample_both<BLOCK, ADJ>, BLOCK, 0));
-        per_sm = occ > 0 ? occ : 1;
+        per_sm = resident_blocks<BLOCK, ADJ>(g, 1, occ);
     }
     const uint64_t full = (uint64_t)g->sm_count * per_sm;
     uint64_t blocks = (k3 + kc + BLOCK - 1) / BLOCK;

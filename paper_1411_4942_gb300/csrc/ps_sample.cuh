@@ -153,7 +153,8 @@ __device__ __forceinline__ int sample_centred(const GraphDev &g, uint64_t seed, 
 // more than registers.  With the hash set's 32-byte buckets the tests needed
 // 80 registers (768 threads); against that, 1024 threads took the adaptive
 // run on a 1M-edge graph from 1.57 to 1.46 ms and 3M + 3M samples on a
-// 10M-edge graph from 394 to 367 us.
+// 10M-edge graph from 394 to 367 us (in order of their draws; plain samples of
+// such graphs run fewer threads, ps_sample.cu).
 template <int BLOCK>
 constexpr int sample_min_blocks() { return BLOCK <= 256 ? 1024 / BLOCK : 1; }
 
