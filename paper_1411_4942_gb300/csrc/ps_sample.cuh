@@ -13,10 +13,11 @@ namespace ps {
 
 // From this many edges the draw of v' from N(v) takes no line of L1: the rows
 // of the heavy endpoints no longer stay near, and their lines push out the
-// records and rows of the samples beside this one (3-path sampling kernel on
-// the 3M-vertex graph, 115M edges: 10.97 -> 10.44 ms; on R-MAT 20, 15.7M
-// edges, the same load made it slower, 725 -> 762 us).
-constexpr int64_t kFarRowsEdges = int64_t{1} << 25;
+// records and rows of the samples beside this one.  2^24 3-path samples in
+// order of their draws, L1 / no L1: 15.7M edges 709 / 756 us, 32M 907 / 957,
+// 47M 1067 / 1094, 64M 1280 / 1276, 78M 1299 / 1294, 117M 1427 / 1396 (2^27
+// there 10.97 / 10.44 ms); plain samples lose less below and are even above.
+constexpr int64_t kFarRowsEdges = int64_t{1} << 26;
 
 // Alg. 1 up to the induced subgraph: the edge e drawn with probability
 // tau_e / W and the two neighbours u' (of u, not v) and v' (of v, not u).
