@@ -165,8 +165,9 @@ int ps_sample_centered(const ps_graph *g, uint64_t k, uint64_t seed, uint64_t fi
  *
  * d_scratch: caller-owned device memory, 16-byte aligned, of
  * ps_ordered_scratch_bytes(k_chunk) bytes (about 1 MB + 11 B per sample)
- * for chunks of k_chunk samples
- * (1 <= k_chunk <= 2^31; larger k runs in several chunks).  It is the
+ * for chunks of k_chunk samples (1 <= k_chunk <= 2^31, 0 is returned for
+ * others).  Larger k runs in several chunks, of at most 2^27 samples each: a
+ * call never uses more than ps_ordered_scratch_bytes(2^27), 1.5 GB.  It is the
  * call's own working memory until the work queued on `stream` has run, so
  * concurrent calls need separate scratch.  Asynchronous.  Returns
  * PS_ERR_WORKSPACE when the scratch is missing, misaligned or smaller than
@@ -326,7 +327,8 @@ int ps_batch_sample_prepared(const void *d_table, int32_t n_graphs, const ps_wor
  * ascending -- d_off (device int64 [n + 1]) and d_col (device int32, room
  * for 2 n_edges entries; the first *nnz are written) -- ready for
  * ps_load_csr.  d_workspace: device, 256-byte aligned, at least
- * ps_ingest_workspace_bytes(n, n_edges) bytes (about 20 bytes per edge).
+ * ps_ingest_workspace_bytes(n, n_edges) bytes (about 25 bytes per edge and 16
+ * per vertex).
  * *nnz (host) receives the number of arcs.  Synchronises `stream`.  Returns
  * PS_ERR_ARG for an id outside [0, n) (or n, n_edges out of range: n < 2^31 - 1,
  * 2 n_edges < 2^31 - 1), PS_ERR_WORKSPACE for a missing, misaligned or small

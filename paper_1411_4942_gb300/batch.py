@@ -34,8 +34,10 @@ class Request:
     slot: int = -1      # histogram slot (6 uint64); assigned by plan_items when -1
 
 
-# graphs with at least this many edges can have their large requests taken
-# in draw order (their records and rows no longer stay in L2)
+# graphs with at least this many edges can have their large requests run
+# through the draw-ordered samplers, beside the queue.  Those order the samples
+# themselves only where it pays (2^22 edges and samples and more); below they
+# are plain launches, which the autotuner times as any other choice.
 ORDERED_MIN_EDGES = 1 << 20
 NEVER = 1 << 62
 

@@ -162,7 +162,7 @@ Tuning resolve_tuning(const ps_tuning *t, int64_t n, int64_t nnz) {
         else if (t->hub_count > 0) r.hub_count = t->hub_count;
         if (t->samples_per_thread > 0) r.samples_per_thread = t->samples_per_thread >= 2 ? 2 : 1;
         if (t->hub_min_degree > 0) r.hub_min_degree = t->hub_min_degree;
-        r.draw_order = t->draw_order >= 2 ? 2 : (t->draw_order > 0 ? 1 : (t->draw_order < 0 ? -1 : 0));
+        r.draw_order = t->draw_order > 0 ? 1 : (t->draw_order < 0 ? -1 : 0);
     }
     if (r.hub_count > n) r.hub_count = static_cast<int>(n);
     return r;

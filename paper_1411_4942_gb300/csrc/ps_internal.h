@@ -261,8 +261,9 @@ int launch_sampler(const ps_graph *g, int sampler, uint64_t k, uint64_t seed, ui
 // Both samplers over ids first_id ..; one without anything to draw is left out.
 int launch_samplers(const ps_graph *g, uint64_t k3, uint64_t *d_hist6, uint64_t kc, uint64_t *d_hist4, uint64_t seed,
                     uint64_t first_id, cudaStream_t s);
-// Samples in the order of their edge draws (ps_order.cu); ids of a chunk are
-// 32-bit offsets, so a chunk holds at most kOrderMaxChunk samples.
+// Samples in the order of their edge draws (ps_order.cu), in chunks of what the
+// scratch holds and at most 2^27; the largest k_chunk that a scratch can be
+// asked for is kOrderMaxChunk.
 constexpr uint64_t kOrderMaxChunk = 1ull << 31;
 size_t ordered_scratch_bytes(uint64_t k_chunk);
 bool order_never(const ps_graph *g);  // every number of samples of this graph is drawn plainly

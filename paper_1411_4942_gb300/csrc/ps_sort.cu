@@ -120,6 +120,8 @@ __device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t *s_wsum) {
 // 12, 14, 16 and 18 rows per warp 1.47, 1.36, 1.40 and 1.41 (shorter tiles write
 // shorter runs).  Warp bases that include the digit's start and items moved
 // as 8 bytes take two shared-memory accesses per item fewer: 1.45 -> 1.39 ms.
+// (At 64 registers the crossing digits spill nothing, read values 24 bytes a
+// thread above kDirectTiles tiles, indices up to 56.)
 // DIRECT: `offsets` holds the raw counts; otherwise offsets[digit * tiles +
 // tile] is where the tile's run of that digit starts.  VAL: values read from
 // vin, or the items' indices, or read and part of the digit.
