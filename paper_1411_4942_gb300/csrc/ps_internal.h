@@ -16,8 +16,10 @@ namespace ps {
 constexpr int kTierA = 32;      // one warp, one key per lane
 constexpr int kTierB = 1024;    // one warp, up to 32 keys per lane in registers
 // (512 on graphs below kSmallArcs arcs: there one warp's 1024-entry row is the
-// step's tail.  1.5M-edge cold request 626 -> 599 us; the 3M-vertex graph
-// 22.6 -> 22.8 ms.)
+// load's tail.  Loads with rows of up to 512 / 1024 entries here: 1.8M arcs
+// 260 / 269 us, 4M 382 / 386, 15.5M 856 / 865 and 930 / 944 (but R-MAT 18, 7.6M
+// arcs, 593 / 572), 31M 1511 / 1501 and 1570 / 1580, 54M 2345 / 2309, 64M
+// 3003 / 2867, 128M 5489 / 5358, 233M 9174 / 9025.)
 constexpr int kTierBSmall = 512;
 constexpr int64_t kSmallArcs = int64_t{1} << 24;
 inline int tier_b(int64_t nnz) { return nnz < kSmallArcs ? kTierBSmall : kTierB; }
