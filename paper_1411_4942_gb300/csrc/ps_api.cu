@@ -265,13 +265,13 @@ static double kl_div(double a, double b) {
 // target is that of p's side; false when no such distance is certain.
 //
 // D falls towards alpha and grows away from it, and the computed value is off
-// by less than 5 u (1 + D), u = 2^-53: two quotients and two logarithms of
-// which each factor is at most 1 / e beside D itself.  So where D, computed
-// at root - margin and root + margin, clears the target by twice that (16 u
-// with room), every point further out is on the side it lies on.  Newton's
-// last step alone does not show it: next to p = 1, where 1 - p has few bits
-// and D bends within one step, it once settled 2.6e-15 from the root with a
-// margin of 1.8e-15.
+// by less than 5 u (1 + D), u = 2^-53: it is the sum of two terms, neither
+// larger than D + 1 / e, each off by 3 u of itself and u or 2 u besides (its
+// quotient within the logarithm).  So where D, computed at root - margin and
+// root + margin, clears the target by twice that (16 u (1 + target), with
+// room), every point further out is on the side it lies on.  Newton's last
+// step alone does not show it: next to p = 1, where D bends within one step,
+// it settled 2.6e-15 from a root with a margin of 1.8e-15.
 static bool kl_newton(double alpha, double target, double far, double *root, double *margin) {
     double near_ = alpha, out = far;  // D < target on alpha's side, > target on the other
     const double away = far > alpha ? 1.0 : -1.0;
